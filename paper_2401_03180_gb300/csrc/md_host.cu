@@ -51,6 +51,10 @@ struct md_handle {
     double* d_scratch = nullptr;         // [3N] doubles for state exchange
     double* d_ekin = nullptr;
     long long* d_epot = nullptr;
+    int energy_parts = 0;                // blocks of the energy sums, replica r's from d_part_off[r]
+    int* d_part_off = nullptr;
+    double* d_ekin_part = nullptr;
+    long long* d_epot_part = nullptr;
     std::vector<long long> n_of_species;   // [R][NS] atoms per replica and species
 };
 
@@ -973,6 +977,16 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     }
     P.cond = 0;
     DALLOC(h->d_ekin, R); DALLOC(h->d_epot, R);
+    {
+        std::vector<int> off(R + 1, 0);
+        for (int r = 0; r < R; ++r)
+            off[r + 1] = off[r] + (h->rep_off[r + 1] - h->rep_off[r] + kEnergyAtoms - 1) / kEnergyAtoms;
+        h->energy_parts = off[R];
+        DALLOC(h->d_part_off, R + 1);
+        DALLOC(h->d_ekin_part, h->energy_parts);
+        DALLOC(h->d_epot_part, h->energy_parts);
+        CU(cudaMemcpy(h->d_part_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
+    }
 
     // ---- uploads (synchronous, init only) ----
     {
@@ -1636,7 +1650,7 @@ static md_status md_rdf_body(md_handle* h, double r_max, int n_bins, int64_t* co
     // positions, and the packed records hold the current positions
     CU(cudaMemsetAsync(d_hist, 0, nh * sizeof(unsigned long long), h->stream));
     CU(cudaMemsetAsync(h->P.counters + 2, 0, sizeof(int), h->stream));
-    launch_rdf(h->P, h->stream, h->n_sm * 4, n_bins, r_max, d_hist);
+    launch_rdf(h->P, h->stream, h->n_sm, n_bins, r_max, d_hist);
     CU(cudaMemsetAsync(h->P.counters + 2, 0, sizeof(int), h->stream));
     CU(cudaGetLastError());
     std::vector<unsigned long long> tmp(nh);
@@ -1697,7 +1711,7 @@ static md_status md_fragments_body(md_handle* h, double r_frag, int mass_max, in
         e = cudaMemsetAsync(h->P.counters + 2, 0, sizeof(int), s);
     }
     if (e == cudaSuccess) {
-        launch_frag_link(h->P, s, h->n_sm * 4, r_frag, d_parent);
+        launch_frag_link(h->P, s, h->n_sm, r_frag, d_parent);
         e = cudaMemsetAsync(h->P.counters + 2, 0, sizeof(int), s);
     }
     if (e == cudaSuccess) {
@@ -1837,7 +1851,7 @@ static md_status md_get_energies_body(md_handle* h, double* e_kin, double* e_pot
     launch_refresh(h->P, h->stream);
     set_build_step(h, h->stream, false);
     launch_pair_forces(h->P, h->stream, true, h->pair_blocks, h->pair_warps);
-    launch_energy(h->P, h->d_ekin, h->d_epot, h->stream);
+    launch_energy(h->P, h->energy_parts, h->d_part_off, h->d_ekin_part, h->d_epot_part, h->d_ekin, h->d_epot, h->stream);
     CU(cudaGetLastError());
     std::vector<double> ek(R);
     std::vector<long long> ep(R);

@@ -30,6 +30,7 @@ constexpr double kLn2 = 0.69314718055994530942;   // ln 2 (scales the LJ table's
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kChargeTable = 1;                  // MD_CHARGE_TABLE
 constexpr float kBBoxMargin = 1e-4f;               // nm, slack of the cluster prefilter
+constexpr int kEnergyAtoms = 1024;                 // atoms per block of the energy sums
 constexpr int kScanCtasMax = 1024;                 // CTAs of the multi-CTA scans (cells, super-clusters)
 
 // device error bits (mirrored to md_status by the host)
@@ -330,14 +331,16 @@ int launch_cells(const Params& p, cudaStream_t s, int grid_atoms, int grid_cells
 int launch_pair_list(const Params& p, cudaStream_t s, int blocks);
 void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks, int warps);
 void launch_velocity_out(const Params& p, double* d_v_out, cudaStream_t s);
-void launch_energy(const Params& p, double* d_ekin, long long* d_epot, cudaStream_t s);
+// energies: n_parts blocks of kEnergyAtoms atoms, replica r's from part_off[r]
+void launch_energy(const Params& p, int n_parts, const int* part_off, double* ekin_part, long long* epot_part, double* d_ekin,
+                   long long* d_epot, cudaStream_t s);
 void launch_philox(unsigned long long seed, const uint32_t* ctr, long long n, uint32_t* out,
                    cudaStream_t s);
 void launch_force_out(const Params& p, double* d_f_out, cudaStream_t s);
 void launch_refresh(const Params& p, cudaStream_t s);
-void launch_rdf(const Params& p, cudaStream_t s, int blocks, int n_bins, double r_max, unsigned long long* hist);
+void launch_rdf(const Params& p, cudaStream_t s, int n_sm, int n_bins, double r_max, unsigned long long* hist);
 void launch_probe(const Params& p, cudaStream_t s, bool rewrite);
-void launch_frag_link(const Params& p, cudaStream_t s, int blocks, double r_frag, int* parent);
+void launch_frag_link(const Params& p, cudaStream_t s, int n_sm, double r_frag, int* parent);
 void launch_frag_init(const Params& p, cudaStream_t s, int* parent, int* mass, int* charge);
 void launch_frag_count(const Params& p, cudaStream_t s, const int* parent, int* label, int* mass, int* charge,
                        const int* mass_number, int mass_max, int charge_max, unsigned long long* counts);
