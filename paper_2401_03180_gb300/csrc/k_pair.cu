@@ -13,16 +13,21 @@
 //     mask), contiguous per SC and cut into chunks of kChunk entries;
 //   * a warp of the force kernel owns one chunk at a time (dynamic scheduling
 //     through an atomic counter);
-//   * the SC's atoms and per-(atom, lane row) i-force partials live in shared
-//     memory; lane (tx = lane & 7, ty = lane >> 3) takes atoms ty, ty+4 of the
-//     entry's j-cluster and, tile by tile, the next i-cluster whose atom tx
-//     is in the mask (its own queue), so a lane column always sees the same
-//     slots in the same order and the shared-memory rows it touches never
-//     share a bank with another column's;
+//   * mixed precision (k_pair): lane (tx = lane & 7, ty = lane >> 3) keeps the
+//     force of atom tx of every i-cluster of the SC in registers and evaluates
+//     it against j-atoms ty and ty + 4 of the entry's j-cluster in the two
+//     halves of packed FP32 operations, one 8 x 8 cluster tile at a time;
+//   * FP64 (k_pair64) and the analyses (k_walk): the SC's atoms (and, in
+//     k_pair64, per-(atom, lane row) i-force partials) live in shared memory;
+//     a lane takes atoms ty, ty+4 of the entry's j-cluster and, tile by tile,
+//     the next i-cluster whose atom tx is in the mask (its own queue), so a lane
+//     column always sees the same slots in the same order and the rows it
+//     touches never share a bank with another column's;
 //   * at the step of a Verlet-buffered build the evaluation also tests every
-//     pair against r_cut + skin and drops from the mask the i-atoms with no
-//     j-atom in range (exact for the list's lifetime), and clears the entry's
-//     fragment flag when no pair in range lies within one fragment;
+//     pair against r_cut + skin and drops from the mask the i-clusters (FP64:
+//     i-atoms) with no j-atom in range (exact for the list's lifetime), and
+//     clears the entry's fragment flag when no pair in range lies within one
+//     fragment;
 //   * forces are summed in FP32 (or FP64) within one chunk for the i side
 //     and one (SC, j-cluster) entry for the j side, then converted
 //     once to 64-bit fixed point (2^-32 kJ/mol/nm): the per-atom totals are
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
         const int e0 = p.sc_eoff[sc], c0 = p.sc_coff[sc];
         if (gr == 0)
             for (int t = lane; t * kChunk < tot; t += 32)
-                p.pl_chunk[c0 + t] = make_int4(sc, e0 + t * kChunk, min(kChunk, tot - t * kChunk), s.rr);
+                p.pl_chunk[c0 + t] = make_int4(s.fc, e0 + t * kChunk, min(kChunk, tot - t * kChunk) | (s.ncl << 16), s.rr);
         // this item's first entry: the SC's offset plus the counts of its earlier parts
         const int cnt_l = lane < G ? p.list_cnt[sc * kHalfShell + lane] : 0;
         int pre = lane < gr ? cnt_l : 0;
@@ -680,15 +685,430 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
     }
 }
 
-// Forces over the cluster-pair list.  A warp takes one chunk (up to kChunk
-// entries of one SC) at a time from an atomic counter.  Blocks of 4, 8 or 12
-// warps (the FP32 bounds keep 85 registers per thread either way: three
-// 8-warp or two 12-warp blocks per SM); each block holds its own copy of the
-// LJ table, so with many type states the 12-warp shape keeps more warps
-// resident than the shared memory allows 8-warp blocks.
-template <bool FP64, bool ENERGY, bool HYB>
-__global__ void __launch_bounds__(FP64 ? 256 : 384, 2) k_pair(Params p)
+// Bonded terms (Sec. II.B, Eqs. 9-10), one per thread over the grid before the
+// chunks: their dependent loads overlap the other warps' pair work, and they
+// add to the same fixed-point sums.
+template <bool FP64, bool ENERGY>
+__device__ __forceinline__ void bonded_prologue(const Params& p)
 {
+    if (p.n_bonds + p.n_angles == 0) return;
+    using T = typename Prec<FP64>::T;
+    const T* bp;
+    const T* ap;
+    if constexpr (FP64) { bp = p.bond_pd; ap = p.angle_pd; }
+    else { bp = p.bond_pf; ap = p.angle_pf; }
+    const int nb = p.n_bonds, nt = p.n_bonds + p.n_angles;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
+        if (t < nb) bonded::bond_term<T, ENERGY>(p, bp, t);
+        else bonded::angle_term<T, ENERGY>(p, ap, t - nb);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Mixed-precision force kernel.  A warp takes one chunk (up to kChunk entries
+// of one SC) at a time from an atomic counter.  Lane (tx, ty) keeps the force
+// of atom tx of each i-cluster in registers for the whole chunk; an entry's
+// tiles are the i-clusters of its mask, a warp-uniform branch each, and the
+// lane's two j-atoms fill the halves of packed FP32 operations.  j forces go to
+// shared memory per lane and are summed over the i-lanes once per chunk.
+//
+// Bound: instruction issue, with the FMA pipe next.  The kernel it replaced (per-atom
+// queues, scalar arithmetic, i forces read and written in shared memory per
+// tile, a shuffle reduction per entry) issued 1.66 G warp instructions for a
+// million droplet atoms at 80 % issue with the shared-memory pipe 73 % busy;
+// this one issues 1.28 G at 68 %, the FMA pipe 48 % busy.  Cluster masks evaluate 14 %
+// more pairs than per-atom queues did (33 against 38 % of the evaluations
+// within r_cut, water at a 0.12 nm skin), which the cheaper tiles more than
+// pay for.  Per launch, 500,001-atom droplet 851 -> 772 us, water box of
+// 30,000 atoms 68.6 -> 64.6, 1,500 atoms 22.0 -> 18.4; hybrid screening, 12,003
+// atoms, 46.4 -> 41.7.  96 registers (20 warps per SM): with 80 (24 warps) the
+// compiler recomputes and spills (963 us), with 128 (16 warps) too few warps
+// cover the latencies (947 us before the j sums moved to shared memory).
+// Two tiles per branch for more independent work: 852 us, the longer code is
+// slower.  The hybrid instance needs 128 registers (112: 45.1 us, 96: 50.9).
+// ---------------------------------------------------------------------------
+template <bool HYB>
+struct JHyb {};
+template <>
+struct JHyb<true> {
+    float4 Gr[kChunk * 4];         // G and r' of the two j-atoms: G0 G1 r'0 r'1
+    float2 iGr[kSCAtoms];          // (f/2) G_i and r'_i of the SC's atoms
+};
+constexpr int kJpRow = 52;         // floats per lane row of the j-force parts (padded: rows start on different banks)
+template <bool HYB>
+struct WarpF32 {
+    float4 xy[kChunk * 4];         // j-atom pairs of the chunk, [entry][ty]: x0 x1 y0 y1 (shifted)
+    float4 zq[kChunk * 4];         // z0 z1 q0 q1
+    float4 ix[kSCAtoms];           // the SC's atoms: x, y, z, f q (hybrid: (f/2) q)
+    int2 off[kChunk * 4];          // LJ column byte offsets of the j-atom pairs
+    int2 jfr[kChunk * 4];          // and their fragments
+    int irow[kSCAtoms];            // shared-memory address of the SC atoms' LJ rows
+    int ifr[kSCAtoms];             // and their fragments
+    float jp[kChunk * 4 * kJpRow]; // j-force parts [entry][ty][component][tx]
+    uint2 ent[kChunk];             // first slot of the j-cluster; i-cluster mask | kEntGen | kEntShare | cluster of the SC << 16
+    JHyb<HYB> hy;
+};
+constexpr unsigned kEntGen = 0x100u;     // the self-cluster diagonal or pairs within one fragment are possible
+constexpr unsigned kEntShare = 0x200u;   // the entry's fragment flag
+
+// What a pair needs besides its two atoms (per chunk).
+struct PairCtx {
+    float rc2, kl, kap, erc, irc;  // kl = -kappa log2(e)
+    float rl2;                     // PRUNE: squared list radius
+    float c2, hf;                  // hybrid: c2 of the replica, f/2
+    const HybQ* rows;              // hybrid: the replica's charge states
+};
+
+__device__ __forceinline__ float2 lds_f2(int addr)
+{
+    float2 v;
+    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+
+// Atom i against j-atoms 0 and 1.  r^-6 (12 c12 r^-6 - 6 c6 + kappa r (c12 r^-6
+// - c6)) is r^-6 ((2 + kappa r / 6) P + 6 c6) with P = 6 c12 r^-6 - 6 c6.
+// GEN: pairs may be dropped (ok) or lie within one fragment (no LJ).
+template <bool GEN, bool ENERGY, bool HYB>
+__device__ __forceinline__ void pair2(const PairCtx& c, const float4& xi, const float2& iGr, int row, int fri, const float4& xy,
+                                      const float4& zq, const int2& off, const int2& frj, const float4& jGr, bool ok0,
+                                      bool ok1, float& fx, float& fy, float& fz, float& u, int& npair, float2& fjx,
+                                      float2& fjy, float2& fjz, float2& r2)
+{
+    using P = Prec<false>;
+    constexpr float kL = 0.69314718055994530942f;
+    const float2 l0 = lds_f2(row + off.x), l1 = lds_f2(row + off.y);   // (6 c6, 6 c12)
+    const float2 dx = make_float2(xi.x - xy.x, xi.x - xy.y);
+    const float2 dy = make_float2(xi.y - xy.z, xi.y - xy.w);
+    const float2 dz = make_float2(xi.z - zq.x, xi.z - zq.y);
+    r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+    const bool in0 = r2.x < c.rc2 && (!GEN || ok0), in1 = r2.y < c.rc2 && (!GEN || ok1);
+    const float y0 = P::rsq(r2.x), y1 = P::rsq(r2.y);
+    const float2 rinv = make_float2(in0 ? y0 : 0.0f, in1 ? y1 : 0.0f);
+    const float2 rinv2 = __fmul2_rn(rinv, rinv);
+    const float2 u6 = __fmul2_rn(__fmul2_rn(rinv2, rinv2), rinv2);
+    const float2 r = __fmul2_rn(r2, rinv);
+    const float2 t = __fmul2_rn(make_float2(c.kl, c.kl), r);              // -kappa r log2(e)
+    const float2 e = make_float2(P::exp2_(t.x), P::exp2_(t.y));           // e^{-kappa r}
+    const float2 w6 = __ffma2_rn(t, make_float2(-kL / 6.0f, -kL / 6.0f), make_float2(2.0f, 2.0f));
+    const float P0 = __fmaf_rn(l0.y, u6.x, -l0.x), P1 = __fmaf_rn(l1.y, u6.y, -l1.x);
+    const float E0 = __fmaf_rn(w6.x, P0, l0.x), E1 = __fmaf_rn(w6.y, P1, l1.x);
+    const bool same0 = GEN && fri == frj.x, same1 = GEN && fri == frj.y;   // bonded in the native structure: no LJ
+    const float lj0 = same0 ? 0.0f : u6.x, lj1 = same1 ? 0.0f : u6.y;
+    const float2 w = __fmul2_rn(rinv2, e);
+    float2 fs;   // F(r)/r
+    if constexpr (HYB) {
+        // each ion's -phi' from its own form, the ion sphere's inside its r' and the
+        // Debye form's outside; xi.w = (f/2) q_i
+        const float2 q2 = make_float2(zq.z, zq.w);
+        const float2 outf = __fmul2_rn(__ffma2_rn(make_float2(c.kap, c.kap), r, make_float2(1.0f, 1.0f)), w);   // e^{-kappa r} (1 + kappa r) / r^2
+        const float2 cr = __fmul2_rn(make_float2(2.0f * c.c2, 2.0f * c.c2), r);
+        const float2 ii = __ffma2_rn(make_float2(xi.w, xi.w), rinv2, __fmul2_rn(make_float2(c.hf, c.hf), cr));
+        const float2 io = __fmul2_rn(make_float2(iGr.x, iGr.x), outf);
+        const float2 ji = __ffma2_rn(q2, rinv2, cr), jo = __fmul2_rn(make_float2(jGr.x, jGr.y), outf);
+        const float2 mi = make_float2(r.x < iGr.y ? ii.x : io.x, r.y < iGr.y ? ii.y : io.y);     // (f/2)(-phi_i')
+        const float2 mj = make_float2(r.x < jGr.z ? ji.x : jo.x, r.y < jGr.w ? ji.y : jo.y);     // -phi_j'
+        const float2 cl = __ffma2_rn(make_float2(xi.w, xi.w), mj, __fmul2_rn(q2, mi));
+        const float2 lw = __fmul2_rn(make_float2(lj0 * E0, lj1 * E1), w);
+        fs = __ffma2_rn(cl, rinv, lw);
+    } else {
+        // f q_i q_j (1/r + kappa)
+        const float2 rk = __fadd2_rn(rinv, make_float2(c.kap, c.kap));
+        const float2 qr = __fmul2_rn(make_float2(zq.z, zq.w), rk);
+        fs = __fmul2_rn(make_float2(__fmaf_rn(lj0, E0, xi.w * qr.x), __fmaf_rn(lj1, E1, xi.w * qr.y)), w);
+    }
+    fx = __fmaf_rn(fs.y, dx.y, __fmaf_rn(fs.x, dx.x, fx));
+    fy = __fmaf_rn(fs.y, dy.y, __fmaf_rn(fs.x, dy.x, fy));
+    fz = __fmaf_rn(fs.y, dz.y, __fmaf_rn(fs.x, dz.x, fz));
+    fjx = __ffma2_rn(fs, dx, fjx);
+    fjy = __ffma2_rn(fs, dy, fjy);
+    fjz = __ffma2_rn(fs, dz, fjz);
+    if constexpr (ENERGY) {
+        const float irc2 = c.irc * c.irc, irc6 = irc2 * irc2 * irc2;
+        auto energy = [&](float rr, float rsq, float ri, float ee, float lj, float Pp, const float2& l, bool on,
+                          float qj, float G) {
+            float v = ee * (lj * (Pp * (1.0f / 6.0f)));
+            if (on) v -= c.erc * (__fmaf_rn(l.y, irc6, -l.x) * (1.0f / 6.0f)) * irc6;
+            if constexpr (HYB) {
+                const float qi = rintf(xi.w / c.hf);
+                const HybQ& Ri = c.rows[(int)qi];
+                const HybQ& Rj = c.rows[(int)qj];
+                const float cr2 = c.c2 * rsq;
+                const float phi_i = rr < Ri.rpf ? qi * ri + Ri.c1f - cr2 : Ri.Gf * ee * ri;
+                const float phi_j = rr < Rj.rpf ? qj * ri + Rj.c1f - cr2 : G * ee * ri;
+                v += c.hf * (qj * (phi_i - Ri.phircf) + qi * (phi_j - Rj.phircf));
+            } else {
+                const float qq = xi.w * qj;
+                v += ee * qq * ri - c.erc * qq * c.irc;
+            }
+            return v;
+        };
+        if (in0) { u += energy(r.x, r2.x, rinv.x, e.x, lj0, P0, l0, !same0, zq.z, jGr.x); npair += 1; }
+        if (in1) { u += energy(r.y, r2.y, rinv.y, e.y, lj1, P1, l1, !same1, zq.w, jGr.y); npair += 1; }
+    }
+}
+
+// Adds v to a fixed-point sum when `on`; a value beyond 2^30 (or not finite)
+// is left out and noted in bad.
+__device__ __forceinline__ void red_fix_if(long long* dst, float v, bool on, bool& bad)
+{
+    const bool ok = Prec<false>::fix_ok(v);
+    if (on && ok) atomicAdd((unsigned long long*)dst, (unsigned long long)Prec<false>::fix(v));
+    bad |= on && !ok;
+}
+
+template <bool ENERGY, bool HYB, int REGS>
+__global__ void __maxnreg__(REGS) k_pair(Params p)
+{
+    using P = Prec<false>;
+    using WF = WarpF32<HYB>;
+    constexpr unsigned kFull = 0xffffffffu;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int nts = p.n_ts_lj;
+    float2* s_lj = reinterpret_cast<float2*>(smem);
+    const size_t tab = ((size_t)nts * nts * sizeof(float2) + 127) / 128 * 128;
+    const int warp = threadIdx.x >> 5;
+    int lane;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+    WF& w = reinterpret_cast<WF*>(smem + tab)[warp];
+    for (int k = threadIdx.x; k < nts * nts; k += blockDim.x) s_lj[k] = p.lj_f[k];
+    __syncthreads();
+    if (*p.err & (ERR_CELL | ERR_LIST)) return;
+    bonded_prologue<false, ENERGY>(p);
+
+    const int tx = lane & 7, ty = lane >> 3;
+    const int n_chunks = min(p.counters[7], p.chunk_cap);
+    const int lj_addr = (int)__cvta_generic_to_shared(smem);
+    // after the j-force reduction lane (tx, ty) holds component tx & 3 (3: none)
+    // of j-atom 2 ty (tx < 4) or 2 ty + 1 (tx >= 4)
+    const int comp = tx & 3;
+    const bool up = tx >= 4;
+    long long* const jdst = (comp == 0 ? p.fx : (comp == 1 ? p.fy : p.fz)) + 2 * ty + (up ? 1 : 0);
+    // In the step of a Verlet-buffered build the positions are the build's:
+    // i-clusters with no pair within r_cut + skin are dropped from an entry's
+    // mask for the list's lifetime (they cannot come within r_cut before the
+    // next build), and so is the fragment flag of an entry with no pair in
+    // range inside one fragment.  A dropped tile only ever added exact zeros,
+    // in the same order: every sum comes out bit-identical with either mask.
+    const bool prune = p.builds != nullptr && list_half_skin2(p) > 0.0f && p.builds[1] != 0;
+    const float rlb = list_rlist_f(p) + kBBoxMargin;
+    const float coulf = (float)p.coulomb_f;
+    PairCtx c;
+    c.rc2 = p.rc2_f;
+    c.irc = (float)(1.0 / p.r_cut);
+    c.rl2 = rlb * rlb;
+    c.hf = 0.5f * coulf;
+    c.c2 = 0.0f;
+    c.rows = nullptr;
+    bool bad = false;
+
+    // The work items are fetched ahead: while a chunk is evaluated, the counter's
+    // answer and the descriptor of the next one are on their way, and its entries
+    // are asked for before the i forces of this one are summed.
+    int item = 0;
+    if (lane == 0) item = atomicAdd(&p.counters[2], 1);
+    item = __shfl_sync(kFull, item, 0);
+    int4 ch = make_int4(0, 0, 0, 0);
+    PairEntry e4 = make_uint4(0u, 0u, 0u, 0u);
+    if (item < n_chunks) {
+        ch = p.pl_chunk[item];          // (first cluster, first entry, entries | clusters << 16, replica)
+        if (lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
+    }
+    while (item < n_chunks) {
+        int next = 0;
+        if (lane == 0) next = atomicAdd(&p.counters[2], 1);
+        const int fc = ch.x, ent0 = ch.y, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
+        const Grid& g = p.grid_b[rr];
+        c.kap = p.rs[rr].kappa_f;
+        c.kl = c.kap * -1.4426950408889634f;
+        c.erc = ENERGY ? P::expneg(c.kap * (float)p.r_cut) : 0.0f;
+        if constexpr (HYB) {
+            c.rows = p.hq + (size_t)rr * kHybQ;
+            const HybRep hr = p.hrep[rr];
+            c.c2 = hr.c2f;
+        }
+        __syncwarp();                              // the previous chunk's reads are done
+        if (lane < kChunk) {
+            unsigned im = e4.z | e4.w;             // i-clusters with some atom in the mask
+            im |= im >> 16;
+            im = (im | (im >> 8)) & 0xffu;
+            const bool self = (e4.y & 0xffu) == 0u;
+            const unsigned kd = self ? (e4.x - (unsigned)fc) & 0xffffu : 0xffffu;   // i-cluster equal to the j-cluster
+            const bool share = (e4.y & kEntryExcl) != 0u;
+            w.ent[lane] = make_uint2(e4.x * kClusterSize, im | (kd < (unsigned)ncl || share ? kEntGen : 0u) |
+                                                              (share ? kEntShare : 0u) | (kd << 16));
+        }
+        // the chunk's j-atoms, one pair per lane, shifted into the SC's cell frame
+        {
+            const int e = lane >> 2;
+            const unsigned jc = __shfl_sync(kFull, e4.x, e), cd = __shfl_sync(kFull, e4.y, e);
+            if (e < n_ent) {
+                int sx, sy, sz;
+                half_shell((int)(cd & 0xffu), sx, sy, sz);
+                const float Dx = (float)sx * g.edge_f[0], Dy = (float)sy * g.edge_f[1], Dz = (float)sz * g.edge_f[2];
+                const int slot = (int)jc * kClusterSize + (lane & 3);
+                const float4 a = p.xq[slot], b = p.xq[slot + 4];
+                const int2 ta = p.tf[slot], tb = p.tf[slot + 4];
+                const int4 t = make_int4(ta.x, ta.y, tb.x, tb.y);
+                w.xy[lane] = make_float4(a.x + Dx, b.x + Dx, a.y + Dy, b.y + Dy);
+                w.zq[lane] = make_float4(a.z + Dz, b.z + Dz, a.w, b.w);
+                w.off[lane] = make_int2(t.x * (int)sizeof(float2), t.z * (int)sizeof(float2));
+                w.jfr[lane] = make_int2(t.y, t.w);
+                if constexpr (HYB) {
+                    const HybQ& Ra = c.rows[(int)a.w];
+                    const HybQ& Rb = c.rows[(int)b.w];
+                    w.hy.Gr[lane] = make_float4(Ra.Gf, Rb.Gf, Ra.rpf, Rb.rpf);
+                }
+            }
+        }
+        // the SC's atoms
+#pragma unroll
+        for (int a = lane; a < kSCAtoms; a += 32)
+            if (a < ncl * kClusterSize) {
+                const float4 v = p.xq[fc * kClusterSize + a];
+                const int2 t = p.tf[fc * kClusterSize + a];
+                w.ix[a] = make_float4(v.x, v.y, v.z, (HYB ? c.hf : coulf) * v.w);
+                w.irow[a] = lj_addr + t.x * nts * (int)sizeof(float2);
+                w.ifr[a] = t.y;
+                if constexpr (HYB) w.hy.iGr[a] = make_float2(c.hf * c.rows[(int)v.w].Gf, c.rows[(int)v.w].rpf);
+            }
+        float ue[ENERGY ? kSuperClusters : 1];
+        float fx[kSuperClusters], fy[kSuperClusters], fz[kSuperClusters];
+        int npair = 0;
+#pragma unroll
+        for (int k = 0; k < kSuperClusters; ++k) {
+            fx[k] = fy[k] = fz[k] = 0.0f;
+            if constexpr (ENERGY) ue[k] = 0.0f;
+        }
+        next = __shfl_sync(kFull, next, 0);
+        if (next < n_chunks) ch = p.pl_chunk[next];
+        __syncwarp();
+
+#pragma unroll 1
+        for (int v = 0; v < n_ent; ++v) {
+            const uint2 en = w.ent[v];
+            // through a warp reduction, so that the branches on it are known to be uniform
+            const unsigned um = __reduce_or_sync(kFull, en.y);
+            if ((um & 0xffu) == 0u) continue;      // no i-cluster in range (or emptied by pruning)
+            const float4 xy = w.xy[4 * v + ty], zq = w.zq[4 * v + ty];
+            const int2 off = w.off[4 * v + ty];
+            float4 jGr = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (HYB) jGr = w.hy.Gr[4 * v + ty];
+            float2 fjx = make_float2(0.f, 0.f), fjy = fjx, fjz = fjx, r2;
+            // GEN: the self-cluster diagonal (i < j) or pairs within one fragment are
+            // possible; PRUNE: build step
+            auto tiles = [&](auto gen, auto pr) {
+                constexpr bool GEN = decltype(gen)::value, PRUNE = decltype(pr)::value;
+                int2 frj = make_int2(0, 0);
+                if constexpr (GEN) frj = w.jfr[4 * v + ty];
+                bool share = false;   // a pair in range within one fragment
+                unsigned keep = 0u;   // i-clusters with a pair in range
+#pragma unroll
+                for (int k = 0; k < kSuperClusters; ++k) {
+                    if (um & (1u << k)) {
+                        const float4 xi = w.ix[k * kClusterSize + tx];
+                        const int row = w.irow[k * kClusterSize + tx];
+                        float2 iGr = make_float2(0.f, 0.f);
+                        if constexpr (HYB) iGr = w.hy.iGr[k * kClusterSize + tx];
+                        int fri = 0;
+                        bool ok0 = true, ok1 = true;
+                        if constexpr (GEN) {
+                            fri = w.ifr[k * kClusterSize + tx];
+                            const bool dg = (um >> 16) == (unsigned)k;
+                            ok0 = !dg || tx < ty;
+                            ok1 = !dg || tx < ty + 4;
+                        }
+                        pair2<GEN, ENERGY, HYB>(c, xi, iGr, row, fri, xy, zq, off, frj, jGr, ok0, ok1, fx[k], fy[k], fz[k],
+                                                ue[ENERGY ? k : 0], npair, fjx, fjy, fjz, r2);
+                        if constexpr (PRUNE) {
+                            const bool n0 = ok0 && r2.x < c.rl2, n1 = ok1 && r2.y < c.rl2;
+                            if (__any_sync(kFull, n0 || n1)) keep |= 1u << k;
+                            if constexpr (GEN) share |= (n0 && fri == frj.x) || (n1 && fri == frj.y);
+                        }
+                    }
+                }
+                if constexpr (PRUNE) {
+                    share = __any_sync(kFull, share);
+                    if (lane == 0) {
+                        PairEntry& out = p.pl[ent0 + v];
+                        if (keep != (um & 0xffu)) {
+                            const unsigned m4 = keep * 0x01010101u;
+                            out.z &= m4;
+                            out.w &= m4;
+                        }
+                        if (share != ((um & kEntShare) != 0u)) out.y ^= kEntryExcl;
+                    }
+                }
+            };
+            if (um & kEntGen) {
+                if (prune) tiles(std::true_type{}, std::true_type{});
+                else tiles(std::true_type{}, std::false_type{});
+            } else {
+                if (prune) tiles(std::false_type{}, std::true_type{});
+                else tiles(std::false_type{}, std::false_type{});
+            }
+            // the lane's j forces, summed over the 8 i-lanes after the chunk
+            float* jp = &w.jp[(4 * v + ty) * kJpRow + tx];
+            jp[0] = fjx.x; jp[8] = fjy.x; jp[16] = fjz.x;
+            jp[24] = fjx.y; jp[32] = fjy.y; jp[40] = fjz.y;
+        }
+        __syncwarp();
+        // j forces: lane (entry, ty) sums the 8 lanes' parts of its pair's six components
+        {
+            const int slot = (int)w.ent[lane >> 2].x + (lane & 3);
+            if (lane < 4 * n_ent && (w.ent[lane >> 2].y & 0xffu)) {
+                const float* jp = &w.jp[lane * kJpRow];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    const float4 a = *reinterpret_cast<const float4*>(jp + 8 * q), b = *reinterpret_cast<const float4*>(jp + 8 * q + 4);
+                    const float2 s2 = __fadd2_rn(__fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y)),
+                                                 __fadd2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w)));
+                    long long* dst = q % 3 == 0 ? p.fx : (q % 3 == 1 ? p.fy : p.fz);
+                    red_fix_if(dst + slot + 4 * (q / 3), -(s2.x + s2.y), true, bad);
+                }
+            }
+        }
+        // the next chunk's entries
+        e4 = make_uint4(0u, 0u, 0u, 0u);
+        if (next < n_chunks && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
+        item = next;
+        // i forces: sum over the four lane rows, a transposing reduction that leaves
+        // two i-clusters to each row; sums of exact zero (tiles never evaluated) add nothing
+        {
+            const bool up2 = (ty & 2) != 0, up1 = (ty & 1) != 0;
+            auto rows = [&](const float* a, long long* dst) {
+                float b[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    b[q] = (up2 ? a[q + 4] : a[q]) + __shfl_xor_sync(kFull, up2 ? a[q] : a[q + 4], 16);
+                dst += (fc + (up2 ? 4 : 0) + (up1 ? 2 : 0)) * kClusterSize + tx;
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float s = (up1 ? b[q + 2] : b[q]) + __shfl_xor_sync(kFull, up1 ? b[q] : b[q + 2], 8);
+                    red_fix_if(dst + q * kClusterSize, s, s != 0.0f, bad);
+                }
+            };
+            rows(fx, p.fx);
+            rows(fy, p.fy);
+            rows(fz, p.fz);
+            if constexpr (ENERGY) rows(ue, p.epot);
+        }
+        if constexpr (ENERGY) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1) npair += __shfl_xor_sync(kFull, npair, o);
+            if (lane == 0 && npair) atomicAdd((unsigned long long*)p.pair_count, (unsigned long long)npair);
+        }
+    }
+    if (bad) atomicOr(p.err, ERR_OVERFLOW);
+}
+
+// FP64 forces over the cluster-pair list.  A warp takes one chunk (up to kChunk
+// entries of one SC) at a time from an atomic counter.  Blocks of 4 or 8 warps;
+// each block holds its own copy of the LJ table.
+template <bool ENERGY, bool HYB>
+__global__ void __launch_bounds__(256, 2) k_pair64(Params p)
+{
+    constexpr bool FP64 = true;
     using P = Prec<FP64>;
     using T = typename P::T;
     using T4 = typename P::T4;
@@ -727,20 +1147,7 @@ __global__ void __launch_bounds__(FP64 ? 256 : 384, 2) k_pair(Params p)
     __syncthreads();
     if (*p.err & (ERR_CELL | ERR_LIST)) return;
 
-    // bonded terms (Sec. II.B, Eqs. 9-10), one per thread over the grid before
-    // the chunks: their dependent loads overlap the other warps' pair work, and
-    // they add to the same fixed-point sums
-    if (p.n_bonds + p.n_angles > 0) {
-        const T* bp;
-        const T* ap;
-        if constexpr (FP64) { bp = p.bond_pd; ap = p.angle_pd; }
-        else { bp = p.bond_pf; ap = p.angle_pf; }
-        const int nb = p.n_bonds, nt = p.n_bonds + p.n_angles;
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
-            if (t < nb) bonded::bond_term<T, ENERGY>(p, bp, t);
-            else bonded::angle_term<T, ENERGY>(p, ap, t - nb);
-        }
-    }
+    bonded_prologue<FP64, ENERGY>(p);
 
     const int tx = lane & 7, ty = lane >> 3;
     const int n_chunks = min(p.counters[7], p.chunk_cap);
@@ -767,11 +1174,10 @@ __global__ void __launch_bounds__(FP64 ? 256 : 384, 2) k_pair(Params p)
         if (lane == 0) item = atomicAdd(&p.counters[2], 1);
         item = __shfl_sync(kFull, item, 0);
         if (item >= n_chunks) break;
-        const int4 ch = p.pl_chunk[item];          // (sc, first entry, entries, replica)
-        const int sc = ch.x, n_ent = ch.z, rr = ch.w;
+        const int4 ch = p.pl_chunk[item];          // (first cluster, first entry, entries | clusters << 16, replica)
+        const int fc = ch.x, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         __syncwarp();   // the previous chunk's reads of the staged entries are done
         if (lane < n_ent) w.ent[lane] = p.pl[ch.y + lane];
-        const int fc = p.sc_first[sc], ncl = p.sc_ncl[sc];
         const Grid& g = p.grid_b[rr];
         const T kap = FP64 ? T(p.rs[rr].kappa_force) : T(p.rs[rr].kappa_f);
         const T kl = kap * T(-1.4426950408889634);   // -kappa log2(e)
@@ -1149,9 +1555,8 @@ __global__ void __launch_bounds__(256) k_walk(Params p, Op op)
         item = __shfl_sync(kFull, item, 0);
         if (item >= n_chunks) break;
         const int4 ch = p.pl_chunk[item];
-        const int sc = ch.x, n_ent = ch.z, rr = ch.w;
+        const int fc = ch.x, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         PairEntry ent = lane < n_ent ? p.pl[ch.y + lane] : make_uint4(0u, 0u, 0u, 0u);
-        const int fc = p.sc_first[sc], ncl = p.sc_ncl[sc];
         const Grid& g = p.grid_b[rr];
         if (near_only) {
             // keep the i-clusters whose boxes come within reach of the entry's
@@ -1280,36 +1685,82 @@ template <bool FP64, bool HYB>
 static size_t pair_smem(int n_ts, int warps)
 {
     const size_t tab = ((size_t)n_ts * n_ts * sizeof(typename Prec<FP64>::C2) + 127) / 128 * 128;
-    return tab + 256 * sizeof(unsigned) + (size_t)warps * sizeof(WarpSmem<FP64, HYB>);
+    if (FP64) return tab + 256 * sizeof(unsigned) + (size_t)warps * sizeof(WarpSmem<true, HYB>);
+    return tab + (size_t)warps * sizeof(WarpF32<HYB>);
 }
 
-template <bool FP64, bool ENERGY, bool HYB>
+// Registers of the mixed-precision force kernel: 96 (20 warps per SM) where
+// chunks are plenty; 128 (16 warps, no recomputation) for the hybrid and the
+// energy instances, which spill otherwise, and for systems with too few chunks
+// to fill more warps: per launch 1,500 atoms 18.4 (96) and 15.6 us (128), 8,005
+// atoms in unbuffered lists 25.9 and 23.9, 30,000 atoms 64.6 and 65.0.
+constexpr int kFewChunksAtoms = 16384;
+template <bool FP64, bool ENERGY, bool HYB, bool FEW>
+static auto pair_kernel()
+{
+    if constexpr (FP64) return k_pair64<ENERGY, HYB>;
+    else return k_pair<ENERGY, HYB, ENERGY || HYB || FEW ? 128 : 96>;
+}
+
+template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static void set_smem_attr()
 {
     static bool done = false;   // one per instantiation
     if (!done) {
-        cudaFuncSetAttribute(k_pair<FP64, ENERGY, HYB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(k_pair<FP64, ENERGY, HYB>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        const auto f = pair_kernel<FP64, ENERGY, HYB, FEW>();
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         done = true;
     }
 }
 
-template <bool FP64, bool ENERGY, bool HYB>
+template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static void launch_one(const Params& p, cudaStream_t s, int blocks, int warps)
 {
-    set_smem_attr<FP64, ENERGY, HYB>();
-    k_pair<FP64, ENERGY, HYB><<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
+    set_smem_attr<FP64, ENERGY, HYB, FEW>();
+    pair_kernel<FP64, ENERGY, HYB, FEW>()<<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
 }
 
-template <bool FP64, bool ENERGY, bool HYB>
+template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int max_blocks(int warps, int n_ts)
 {
-    set_smem_attr<FP64, ENERGY, HYB>();
+    set_smem_attr<FP64, ENERGY, HYB, FEW>();
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_pair<FP64, ENERGY, HYB>, warps * 32,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW>(), warps * 32,
                                                   pair_smem<FP64, HYB>(n_ts, warps));
     return n;
+}
+
+// Calls f with the force kernel's instance as compile-time constants.
+template <class F>
+static void with_instance(bool fp64, bool energy, bool hyb, bool few, F&& f)
+{
+    using T = std::true_type;
+    using N = std::false_type;
+    auto eh = [&](auto d, auto w) {
+        if (hyb) {
+            if (energy) f(d, T{}, T{}, w);
+            else f(d, N{}, T{}, w);
+        } else {
+            if (energy) f(d, T{}, N{}, w);
+            else f(d, N{}, N{}, w);
+        }
+    };
+    if (fp64) eh(T{}, N{});
+    else if (few && !energy && !hyb) f(N{}, N{}, N{}, T{});
+    else eh(N{}, N{});
+}
+
+// Largest pair_blocks_per_sm a caller may pin for `warps` warps per block: the
+// interface's limits (24 resident warps per SM, less where the LJ table fills
+// the shared memory).  More blocks than fit at once are correct as well: blocks
+// take chunks from a counter until none is left.
+int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
+{
+    if (fp64) return pair_max_blocks_per_sm(true, false, hyb, warps, n_ts, 0);
+    const size_t tab = ((size_t)n_ts * n_ts * sizeof(float2) + 127) / 128 * 128;
+    const size_t block = tab + 1024 + (size_t)warps * (hyb ? 9664 : 8272) + 1024;
+    return std::max(1, std::min(24 / warps, (int)(233472 / block)));
 }
 
 int launch_pair_list(const Params& p, cudaStream_t s, int blocks)
@@ -1332,36 +1783,19 @@ int launch_pair_list(const Params& p, cudaStream_t s, int blocks)
 
 void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks, int warps)
 {
-    const bool hyb = p.screening != 0;
-    if (p.precision == 0) {
-        if (hyb) {
-            if (energy) launch_one<false, true, true>(p, s, blocks, warps);
-            else launch_one<false, false, true>(p, s, blocks, warps);
-        } else {
-            if (energy) launch_one<false, true, false>(p, s, blocks, warps);
-            else launch_one<false, false, false>(p, s, blocks, warps);
-        }
-    } else {
-        if (hyb) {
-            if (energy) launch_one<true, true, true>(p, s, blocks, warps);
-            else launch_one<true, false, true>(p, s, blocks, warps);
-        } else {
-            if (energy) launch_one<true, true, false>(p, s, blocks, warps);
-            else launch_one<true, false, false>(p, s, blocks, warps);
-        }
-    }
+    with_instance(p.precision != 0, energy, p.screening != 0, p.n_atoms <= kFewChunksAtoms,
+                  [&](auto fp64, auto en, auto hyb, auto few) {
+                      launch_one<decltype(fp64)::value, decltype(en)::value, decltype(hyb)::value, decltype(few)::value>(
+                          p, s, blocks, warps);
+                  });
 }
 
-int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts)
+int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms)
 {
-    int n;
-    if (!fp64) {
-        if (hyb) n = energy ? max_blocks<false, true, true>(warps, n_ts) : max_blocks<false, false, true>(warps, n_ts);
-        else n = energy ? max_blocks<false, true, false>(warps, n_ts) : max_blocks<false, false, false>(warps, n_ts);
-    } else {
-        if (hyb) n = energy ? max_blocks<true, true, true>(warps, n_ts) : max_blocks<true, false, true>(warps, n_ts);
-        else n = energy ? max_blocks<true, true, false>(warps, n_ts) : max_blocks<true, false, false>(warps, n_ts);
-    }
+    int n = 0;
+    with_instance(fp64, energy, hyb, n_atoms <= kFewChunksAtoms, [&](auto d, auto en, auto h, auto few) {
+        n = max_blocks<decltype(d)::value, decltype(en)::value, decltype(h)::value, decltype(few)::value>(warps, n_ts);
+    });
     return n > 0 ? n : 1;
 }
 

@@ -476,7 +476,7 @@ md_status autotune(md_handle* h)
     for (int w : warps_c) {
         if (fp64 && w > 8) continue;   // the FP64 kernel takes up to 256 threads per block
         if (h->cfg.pair_warps && w != h->cfg.pair_warps) continue;
-        int maxb = pair_max_blocks_per_sm(fp64, false, h->P.screening != 0, w, h->NTS_LJ);
+        int maxb = pair_max_blocks_per_sm(fp64, false, h->P.screening != 0, w, h->NTS_LJ, h->N);
         for (int bps = 1; bps <= maxb; ++bps) {
             if (h->cfg.pair_blocks_per_sm && bps != h->cfg.pair_blocks_per_sm) continue;
             const int blocks = bps * h->n_sm;
@@ -768,7 +768,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
             double s6 = sg * sg * sg * sg * sg * sg;
             double c6 = 4.0 * ep * s6, c12 = c6 * s6;
             lj_d[(size_t)a * nts_lj + b] = make_double2(-6.0 * c6, -kLn2 * c12);   // pair kernels take (-6 c6, -ln2 c12)
-            lj_f[(size_t)a * nts_lj + b] = make_float2((float)(-6.0 * c6), (float)(-kLn2 * c12));
+            lj_f[(size_t)a * nts_lj + b] = make_float2((float)(6.0 * c6), (float)(6.0 * c12));
         }
     std::vector<double> etab(kNEtab), inv12(13, 0.0);
     for (int k = 0; k < kNEtab; ++k) etab[k] = std::exp(-(double)k / 16.0);
@@ -1099,15 +1099,17 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
             h->pair_warps = c.pair_warps;
         } else {
             h->pair_warps = 8;
-            int best = 8 * pair_max_blocks_per_sm(fp64, false, c.screening != 0, 8, h->NTS_LJ);
-            if (!fp64) {
-                const int w12 = 12 * pair_max_blocks_per_sm(fp64, false, c.screening != 0, 12, h->NTS_LJ);
-                if (w12 > best) h->pair_warps = 12;
+            int best = 8 * pair_max_blocks_per_sm(fp64, false, c.screening != 0, 8, h->NTS_LJ, h->N);
+            for (int wpb : {4, 12}) {
+                if (fp64) break;
+                const int w = wpb * pair_max_blocks_per_sm(fp64, false, c.screening != 0, wpb, h->NTS_LJ, h->N);
+                if (w > best) { best = w; h->pair_warps = wpb; }
             }
         }
-        const int maxb = pair_max_blocks_per_sm(fp64, false, c.screening != 0, h->pair_warps, h->NTS_LJ);
-        if (c.pair_blocks_per_sm > maxb)
-            return fail(h, MD_ERR_INVALID_ARG, "pair_blocks_per_sm exceeds the " + std::to_string(maxb) +
+        const int maxb = pair_max_blocks_per_sm(fp64, false, c.screening != 0, h->pair_warps, h->NTS_LJ, h->N);
+        const int pin = std::max(maxb, pair_pin_limit(fp64, c.screening != 0, h->pair_warps, h->NTS_LJ));
+        if (c.pair_blocks_per_sm > pin)
+            return fail(h, MD_ERR_INVALID_ARG, "pair_blocks_per_sm exceeds the " + std::to_string(pin) +
                                                    " blocks of " + std::to_string(h->pair_warps) +
                                                    " warps an SM holds for this system");
         h->pair_blocks = h->n_sm * (c.pair_blocks_per_sm ? c.pair_blocks_per_sm : maxb);

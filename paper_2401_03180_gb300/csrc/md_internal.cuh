@@ -160,7 +160,7 @@ struct Params {
     const long long* e_auger_mev;// [n_species]
     const double* etab;      // [kNEtab]
     const double* inv12;     // [13] 1/m
-    const float2* lj_f;      // [n_ts_lj][n_ts_lj] (-6 c6, -ln2 c12)
+    const float2* lj_f;      // [n_ts_lj][n_ts_lj] (6 c6, 6 c12)
     const double2* lj_d;     // [n_ts_lj][n_ts_lj] (-6 c6, -ln2 c12)
 
     // replicas
@@ -344,7 +344,8 @@ void launch_frag_link(const Params& p, cudaStream_t s, int n_sm, double r_frag, 
 void launch_frag_init(const Params& p, cudaStream_t s, int* parent, int* mass, int* charge);
 void launch_frag_count(const Params& p, cudaStream_t s, const int* parent, int* label, int* mass, int* charge,
                        const int* mass_number, int mass_max, int charge_max, unsigned long long* counts);
-int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts);
+int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms);
+int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts);
 // message returned by md_last_error(NULL) (host side)
 void set_global_error(const std::string& msg);
 

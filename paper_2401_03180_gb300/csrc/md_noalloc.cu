@@ -275,7 +275,7 @@ extern "C" md_status md_forces_noalloc(const md_forces_input* in, double* d_f, v
             const double s6 = sg * sg * sg * sg * sg * sg;
             const double c6 = 4.0 * ep * s6, c12 = c6 * s6;
             tab_d[(size_t)a * nts + b] = make_double2(-6.0 * c6, -kLn2 * c12);   // pair kernels take (-6 c6, -ln2 c12)
-            tab_f[(size_t)a * nts + b] = make_float2((float)(-6.0 * c6), (float)(-kLn2 * c12));
+            tab_f[(size_t)a * nts + b] = make_float2((float)(6.0 * c6), (float)(6.0 * c12));
         }
     const int zs[MD_MAX_SPECIES] = {in->z[0], in->z[1], in->z[2], in->z[3], in->z[4], in->z[5], in->z[6], in->z[7]};
     const double one = 1.0;
@@ -302,7 +302,7 @@ extern "C" md_status md_forces_noalloc(const md_forces_input* in, double* d_f, v
     int n_sm = 0;
     NA_CU(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     const int warps = 8;
-    const int blocks = n_sm * pair_max_blocks_per_sm(in->precision == MD_PREC_FP64, false, false, warps, nts);
+    const int blocks = n_sm * pair_max_blocks_per_sm(in->precision == MD_PREC_FP64, false, false, warps, nts, n);
     launch_step_a(P, 0, s, (n + 255) / 256);                           // grid and screening
     launch_cells(P, s, (n + 255) / 256, std::max(1, std::min(g.cell_cap, n_sm * 8)), 1024);
     launch_pair_list(P, s, std::max(1, std::min((P.sc_cap + 7) / 8, 8 * n_sm)));
