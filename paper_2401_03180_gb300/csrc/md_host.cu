@@ -49,6 +49,7 @@ struct md_handle {
     double pair_ms = 0.0;
     long long pair_launches = 0, steps = 0, last_pairs = 0;
     double* d_scratch = nullptr;         // [3N] doubles for state exchange
+    unsigned* d_bad = nullptr;           // md_set_state's failed checks
     double* d_ekin = nullptr;
     long long* d_epot = nullptr;
     int energy_parts = 0;                // blocks of the energy sums, replica r's from d_part_off[r]
@@ -278,7 +279,7 @@ md_status rebuild_checked(md_handle* h, bool* grown, bool from_ref = false)
         unsigned e = 0;
         md_status st = read_flags(h, &e);
         if (st != MD_OK) return st;
-        if (e != ERR_LIST) return check_device_flags(h);
+        if (e != ERR_LIST) return flags_status(h, e);
         int need[2] = {0, 0};
         CU(cudaMemcpy(need, h->P.counters + 6, sizeof(need), cudaMemcpyDeviceToHost));
         st = size_list(h, std::max<long long>(2LL * need[0], 2LL * h->P.pl_cap));
@@ -963,6 +964,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     DALLOC(P.pair_count, 1);
     DALLOC(P.err, 1); DALLOC(P.step, 1); DALLOC(P.kick_full, 1);
     DALLOC(h->d_scratch, 3 * (size_t)N);
+    DALLOC(h->d_bad, 1);
     DALLOC(P.cl_cen, P.cluster_cap);
     DALLOC(P.maxd2, 1);
     DALLOC(P.builds, 2);
@@ -1416,21 +1418,34 @@ md_status md_step(md_handle* h, int n_steps)
     return guarded(h, [&]() { return md_step_body(h, n_steps); });
 }
 
-// The copies of md_get_state that need no host-side reordering (velocities,
-// forces, charges, K holes, the replicas' plasma state into pinned memory),
-// enqueued on the handle's stream.
+// The copies of md_get_state (the replicas' plasma state goes into pinned
+// memory), enqueued on the handle's stream.
 static md_status get_state_async(md_handle* h, md_state* out, unsigned fields)
 {
     const int N = h->N, R = h->R;
+    const size_t nv = 3 * (size_t)N * sizeof(double);
+    if (fields & MD_FIELD_X) {
+        if (!out->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
+        const double* src[3] = {h->P.x, h->P.y, h->P.z};
+        launch_join_vectors(src, N, h->d_scratch, h->stream);
+        CU(cudaMemcpyAsync(out->x, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
+    }
+    if (fields & MD_FIELD_XLIST) {
+        if (!out->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
+        const bool buffered = h->P.xr != nullptr;
+        const double* src[3] = {buffered ? h->P.xr : h->P.x, buffered ? h->P.yr : h->P.y, buffered ? h->P.zr : h->P.z};
+        launch_join_vectors(src, N, h->d_scratch, h->stream);
+        CU(cudaMemcpyAsync(out->x_list, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
+    }
     if (fields & MD_FIELD_V) {
         if (!out->v) return fail(h, MD_ERR_INVALID_ARG, "v buffer missing");
         launch_velocity_out(h->P, h->d_scratch, h->stream);
-        CU(cudaMemcpyAsync(out->v, h->d_scratch, 3 * (size_t)N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CU(cudaMemcpyAsync(out->v, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_F) {
         if (!out->f) return fail(h, MD_ERR_INVALID_ARG, "f buffer missing");
         launch_force_out(h->P, h->d_scratch, h->stream);
-        CU(cudaMemcpyAsync(out->f, h->d_scratch, 3 * (size_t)N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CU(cudaMemcpyAsync(out->f, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_Q) {
         if (!out->q) return fail(h, MD_ERR_INVALID_ARG, "q buffer missing");
@@ -1467,11 +1482,10 @@ static md_status md_get_state_body(md_handle* h, md_state* out, unsigned fields)
 {
     if (!h) return fail(nullptr, MD_ERR_INVALID_ARG, "null handle");
     if (!out) return fail(h, MD_ERR_INVALID_ARG, "null state");
-    // Fields copied without host-side reordering, after steps still in flight:
-    // the copies and the error flags are read in one round trip.  Any flag
-    // set (a list overflow, an error) falls back to md_sync and copies again.
-    const unsigned host_side = MD_FIELD_X | MD_FIELD_XLIST;
-    if (h->pending && !h->poisoned && !(fields & host_side)) {
+    // After steps still in flight the copies and the error flags are read in one
+    // round trip.  Any flag set (a list overflow, an error) falls back to md_sync
+    // and copies again.
+    if (h->pending && !h->poisoned) {
         md_status st = get_state_async(h, out, fields);
         if (st != MD_OK) return st;
         CU(cudaMemcpyAsync(h->h_err, h->P.err, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
@@ -1490,36 +1504,11 @@ static md_status md_get_state_body(md_handle* h, md_state* out, unsigned fields)
         md_status st_ = md_sync(h);
         if (st_ != MD_OK) return st_;
     }
-    const int N = h->N;
+    md_status st = get_state_async(h, out, fields);
+    if (st != MD_OK) return st;
     CU(cudaStreamSynchronize(h->stream));
-    std::vector<double> tmp;
-    if (fields & MD_FIELD_X) {
-        if (!out->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
-        tmp.resize(N);
-        double* src[3] = {h->P.x, h->P.y, h->P.z};
-        for (int d = 0; d < 3; ++d) {
-            CU(cudaMemcpy(tmp.data(), src[d], N * sizeof(double), cudaMemcpyDeviceToHost));
-            for (int i = 0; i < N; ++i) out->x[3 * i + d] = tmp[i];
-        }
-    }
-    {
-        md_status st = get_state_async(h, out, fields);
-        if (st != MD_OK) return st;
-        CU(cudaStreamSynchronize(h->stream));
-        unpack_rep_state(h, out, fields);
-    }
+    unpack_rep_state(h, out, fields);
     if (fields & MD_FIELD_STEP) out->step = h->host_step;
-    if (fields & MD_FIELD_XLIST) {
-        if (!out->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
-        tmp.resize(N);
-        const bool buffered = h->P.xr != nullptr;
-        double* src[3] = {buffered ? h->P.xr : h->P.x, buffered ? h->P.yr : h->P.y, buffered ? h->P.zr : h->P.z};
-        for (int d = 0; d < 3; ++d) {
-            CU(cudaMemcpy(tmp.data(), src[d], N * sizeof(double), cudaMemcpyDeviceToHost));
-            for (int i = 0; i < N; ++i) out->x_list[3 * i + d] = tmp[i];
-        }
-    }
-    CU(cudaStreamSynchronize(h->stream));
     return MD_OK;
 }
 
@@ -1537,53 +1526,49 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
         if (st_ != MD_OK) return st_;
     }
     const int N = h->N, R = h->R;
-    CU(cudaStreamSynchronize(h->stream));
-    // bring velocities to the integer step with the current forces first
-    launch_velocity_out(h->P, h->d_scratch, h->stream);
-    {
-        std::vector<double> v(3 * (size_t)N), tmp(N);
-        CU(cudaMemcpyAsync(v.data(), h->d_scratch, v.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-        CU(cudaStreamSynchronize(h->stream));
-        const double* vs = (fields & MD_FIELD_V) ? in->v : v.data();
-        if ((fields & MD_FIELD_V) && !in->v) return fail(h, MD_ERR_INVALID_ARG, "v buffer missing");
-        double* dst[3] = {h->P.vx, h->P.vy, h->P.vz};
-        for (int d = 0; d < 3; ++d) {
-            for (int i = 0; i < N; ++i) {
-                tmp[i] = vs[3 * i + d];
-                if (!std::isfinite(tmp[i])) return fail(h, MD_ERR_INVALID_ARG, "non-finite velocity");
-            }
-            CU(cudaMemcpy(dst[d], tmp.data(), N * sizeof(double), cudaMemcpyHostToDevice));
-        }
+    const cudaStream_t s = h->stream;
+    if ((fields & MD_FIELD_V) && !in->v) return fail(h, MD_ERR_INVALID_ARG, "v buffer missing");
+    if ((fields & MD_FIELD_X) && !in->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
+    if ((fields & MD_FIELD_Q) && !in->q) return fail(h, MD_ERR_INVALID_ARG, "q buffer missing");
+    if ((fields & MD_FIELD_H) && !in->h) return fail(h, MD_ERR_INVALID_ARG, "h buffer missing");
+    // the arrays are copied as they are, checked and stored on the device; a field
+    // that fails its check, and the ones after it, are not stored
+    enum : unsigned { BAD_V = 1u, BAD_X = 2u, BAD_Q = 4u, BAD_H = 8u, BAD_XLIST = 16u };
+    const size_t nv = 3 * (size_t)N * sizeof(double);
+    CU(cudaMemsetAsync(h->d_bad, 0, sizeof(unsigned), s));
+    double* const vel[3] = {h->P.vx, h->P.vy, h->P.vz};
+    if (fields & MD_FIELD_V) {
+        CU(cudaMemcpyAsync(h->d_scratch, in->v, nv, cudaMemcpyHostToDevice, s));
+    } else {
+        // bring velocities to the integer step with the current forces first
+        launch_velocity_out(h->P, h->d_scratch, s);
     }
+    launch_store_vectors(h->d_scratch, N, vel, h->d_bad, BAD_V, s);
     if (fields & MD_FIELD_X) {
-        if (!in->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
-        std::vector<double> tmp(N);
-        double* dst[3] = {h->P.x, h->P.y, h->P.z};
-        for (int d = 0; d < 3; ++d) {
-            for (int i = 0; i < N; ++i) {
-                tmp[i] = in->x[3 * i + d];
-                if (!std::isfinite(tmp[i])) return fail(h, MD_ERR_INVALID_ARG, "non-finite position");
-            }
-            CU(cudaMemcpy(dst[d], tmp.data(), N * sizeof(double), cudaMemcpyHostToDevice));
-        }
+        double* const dst[3] = {h->P.x, h->P.y, h->P.z};
+        CU(cudaMemcpyAsync(h->d_scratch, in->x, nv, cudaMemcpyHostToDevice, s));
+        launch_store_vectors(h->d_scratch, N, dst, h->d_bad, BAD_X, s);
     }
+    uint8_t* const bytes = reinterpret_cast<uint8_t*>(h->d_scratch);
     if (fields & MD_FIELD_Q) {
-        if (!in->q) return fail(h, MD_ERR_INVALID_ARG, "q buffer missing");
-        std::vector<uint8_t> sp(N);
-        CU(cudaMemcpy(sp.data(), h->P.species, N, cudaMemcpyDeviceToHost));
-        for (int i = 0; i < N; ++i)
-            if (in->q[i] > h->z[sp[i]]) return fail(h, MD_ERR_INVALID_ARG, "q above Z");
-        CU(cudaMemcpy(h->P.q, in->q, N, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(bytes, in->q, N, cudaMemcpyHostToDevice, s));
+        launch_store_bytes(bytes, N, h->P.q, h->P.species, h->P.zs, h->d_bad, BAD_Q, s);
     }
     if (fields & MD_FIELD_H) {
-        if (!in->h) return fail(h, MD_ERR_INVALID_ARG, "h buffer missing");
-        for (int i = 0; i < N; ++i)
-            if (in->h[i] > 1) return fail(h, MD_ERR_INVALID_ARG, "h must be 0 or 1");
-        CU(cudaMemcpy(h->P.h, in->h, N, cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(bytes, in->h, N, cudaMemcpyHostToDevice, s));
+        launch_store_bytes(bytes, N, h->P.h, h->P.species, nullptr, h->d_bad, BAD_H, s);
     }
-    if (fields & (MD_FIELD_PLASMA | MD_FIELD_COUNTS)) {
-        std::vector<RepState> rs(R);
-        CU(cudaMemcpy(rs.data(), h->P.rs, R * sizeof(RepState), cudaMemcpyDeviceToHost));
+    CU(cudaGetLastError());
+    const bool rep_fields = (fields & (MD_FIELD_PLASMA | MD_FIELD_COUNTS)) != 0;
+    if (rep_fields) CU(cudaMemcpyAsync(h->h_rs, h->P.rs, R * sizeof(RepState), cudaMemcpyDeviceToHost, s));
+    CU(cudaMemcpyAsync(h->h_err, h->d_bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+    if (*h->h_err & BAD_V) return fail(h, MD_ERR_INVALID_ARG, "non-finite velocity");
+    if (*h->h_err & BAD_X) return fail(h, MD_ERR_INVALID_ARG, "non-finite position");
+    if (*h->h_err & BAD_Q) return fail(h, MD_ERR_INVALID_ARG, "q above Z");
+    if (*h->h_err & BAD_H) return fail(h, MD_ERR_INVALID_ARG, "h must be 0 or 1");
+    if (rep_fields) {
+        RepState* rs = h->h_rs;
         for (int r = 0; r < R; ++r) {
             if (fields & MD_FIELD_PLASMA) {
                 if (!in->n_e || !in->e_gas_mev) return fail(h, MD_ERR_INVALID_ARG, "plasma buffers missing");
@@ -1594,29 +1579,26 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
             if ((fields & MD_FIELD_COUNTS) && in->event_counts)
                 for (int k = 0; k < 4; ++k) rs[r].counts[k] = in->event_counts[4 * r + k];
         }
-        CU(cudaMemcpy(h->P.rs, rs.data(), R * sizeof(RepState), cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(h->P.rs, rs, R * sizeof(RepState), cudaMemcpyHostToDevice, s));
     }
     if (fields & MD_FIELD_STEP) {
         if (in->step < 0 || in->step > h->cfg.max_steps) return fail(h, MD_ERR_INVALID_ARG, "step out of range");
         h->host_step = in->step;
-        CU(cudaMemcpy(h->P.step, &in->step, sizeof(long long), cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(h->P.step, &h->host_step, sizeof(long long), cudaMemcpyHostToDevice, s));
     }
-    CU(cudaMemset(h->P.kick_full, 0, sizeof(int)));
-    CU(cudaMemset(h->P.err, 0, sizeof(unsigned)));
+    CU(cudaMemsetAsync(h->P.kick_full, 0, sizeof(int), s));
+    CU(cudaMemsetAsync(h->P.err, 0, sizeof(unsigned), s));
     h->poisoned = false;
     bool from_ref = false;
     if (fields & MD_FIELD_XLIST) {
         if (!in->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
         if (h->P.xr) {   // buffered list: rebuild it where the checkpointed run built it
-            std::vector<double> tmp(N);
-            double* dst[3] = {h->P.xr, h->P.yr, h->P.zr};
-            for (int d = 0; d < 3; ++d) {
-                for (int i = 0; i < N; ++i) {
-                    tmp[i] = in->x_list[3 * i + d];
-                    if (!std::isfinite(tmp[i])) return fail(h, MD_ERR_INVALID_ARG, "non-finite list position");
-                }
-                CU(cudaMemcpy(dst[d], tmp.data(), N * sizeof(double), cudaMemcpyHostToDevice));
-            }
+            double* const dst[3] = {h->P.xr, h->P.yr, h->P.zr};
+            CU(cudaMemcpyAsync(h->d_scratch, in->x_list, nv, cudaMemcpyHostToDevice, s));
+            launch_store_vectors(h->d_scratch, N, dst, h->d_bad, BAD_XLIST, s);
+            CU(cudaMemcpyAsync(h->h_err, h->d_bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+            CU(cudaStreamSynchronize(s));
+            if (*h->h_err & BAD_XLIST) return fail(h, MD_ERR_INVALID_ARG, "non-finite list position");
             from_ref = true;
         }
     }
