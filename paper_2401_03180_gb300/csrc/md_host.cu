@@ -1108,7 +1108,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
                 if (w > best) { best = w; h->pair_warps = wpb; }
             }
         }
-        const int maxb = pair_max_blocks_per_sm(fp64, false, c.screening != 0, h->pair_warps, h->NTS_LJ, h->N);
+        const int maxb = std::max(1, pair_max_blocks_per_sm(fp64, false, c.screening != 0, h->pair_warps, h->NTS_LJ, h->N));
         const int pin = std::max(maxb, pair_pin_limit(fp64, c.screening != 0, h->pair_warps, h->NTS_LJ));
         if (c.pair_blocks_per_sm > pin)
             return fail(h, MD_ERR_INVALID_ARG, "pair_blocks_per_sm exceeds the " + std::to_string(pin) +
