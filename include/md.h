@@ -322,8 +322,8 @@ typedef struct md_timing {
     int sort_threads;        /* cell-sort block size in use                 */
     int list_blocks_per_sm;  /* list-build blocks per SM in use             */
     int build_kernels;       /* kernels of one cell + list build in the step
-                                graph (5 to 12: the scans and the sort take
-                                one or several kernels by grid size)       */
+                                graph (5 to 12: the scans, the sort and the list
+                                take one or several kernels by size)       */
     int64_t list_unbuffered_builds; /* of list_builds, those without the skin
                                 (list_skin_adaptive)                         */
 } md_timing;

@@ -238,7 +238,8 @@ __device__ __forceinline__ void pair64(const double4_16a& xi, int row_off, int f
 //                 the SC's chunk descriptors.
 // An SC's range is split into 1, 2, 7 or 14 parts (list_parts): as few as keep
 // every warp of the grid busy, so that a system of many SCs stages each SC once
-// and a small one still spreads over the GPU.
+// and a smaller one still spreads over the GPU.  Systems of few SCs take
+// k_list_fused below instead.
 struct ListWarp {
     float4 lo[kSuperClusters], hi[kSuperClusters];   // the SC's i-cluster boxes (cell frame)
     int2 fr[kSuperClusters];                          // fragment range of each i-cluster
@@ -612,6 +613,24 @@ __device__ __forceinline__ uint4 list_entry(const Params& p, const ListWarp& w, 
     return make_uint4((unsigned)j.jc, (unsigned)j.nb | (share ? kEntryExcl : 0u), mlo, mhi);
 }
 
+// The SC's atoms in slot order (cluster k, atom a); absent clusters far away.
+__device__ __forceinline__ void list_stage_atoms(const Params& p, ListWarp& w, const ListSC& s, int t, int n_threads)
+{
+    for (int a = t; a < kSCAtoms; a += n_threads) {
+        float4 v = make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.0f);
+        if ((a >> 3) < s.ncl) {
+            const int slot = s.fc * kClusterSize + a;
+            if (p.precision == 0) {
+                v = p.xq[slot];
+            } else {
+                const double4_32a x = p.xq64[slot];
+                v = make_float4((float)x.x, (float)x.y, (float)x.z, 0.0f);
+            }
+        }
+        w.ip[a] = v;
+    }
+}
+
 __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
 {
     constexpr unsigned kFull = 0xffffffffu;
@@ -647,20 +666,7 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
             w.hi[lane] = p.bb_hi[s.fc + lane];
             w.fr[lane] = p.bb_frag[s.fc + lane];
         }
-        for (int a = lane; a < kSCAtoms; a += 32) {
-            // slot order (cluster k, atom a); absent clusters far away
-            float4 v = make_float4(1.0e6f, 1.0e6f, 1.0e6f, 0.0f);
-            if ((a >> 3) < s.ncl) {
-                const int slot = s.fc * kClusterSize + a;
-                if (p.precision == 0) {
-                    v = p.xq[slot];
-                } else {
-                    const double4_32a t = p.xq64[slot];
-                    v = make_float4((float)t.x, (float)t.y, (float)t.z, 0.0f);
-                }
-            }
-            w.ip[a] = v;
-        }
+        list_stage_atoms(p, w, s, lane, 32);
         __syncwarp();
         int off = e0 + pre;
         const int end = off + mine;
@@ -676,6 +682,111 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
         // `end`; should it fall short, pad with empty entries (a real cluster, no
         // i-atom in range) rather than leave slots unwritten
         for (int at = off + lane; at < end; at += 32) p.pl[at] = make_uint4((unsigned)s.fc, 0u, 0u, 0u);
+    }
+}
+
+// The same list in one kernel, for systems of few SCs (kListFusedScs): a block
+// per SC, its 8 warps sharing the SC's index range.  Each warp keeps the
+// j-clusters it found in range (compacted in shared memory, kFound of them; a
+// warp that finds more repeats the box tests), the block adds up its warps'
+// counts and reserves the SC's entries and chunks with one atomic each.  An
+// SC's entries and chunks are those of the three kernels above; only where they
+// lie in the list follows the order of the atomics, which no sum depends on.
+// Latency-bound: what the three kernels spend on their launches, on staging the
+// SC once per part and pass, and on entries of j-clusters out of range is saved.
+// Count, scan and write against this kernel, per build: 8,005 atoms (unbuffered)
+// 20.1 -> 8.9 us, 12,297 atoms 23.6 -> 11.6, 30,000 atoms 31.9 -> 17.3.
+constexpr int kListFusedScs = 8192;
+constexpr int kFound = 128;
+__global__ void __launch_bounds__(kListWarps * 32, 4) k_list_fused(Params p)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    __shared__ ListWarp w;
+    __shared__ uint2 s_found[kListWarps][kFound];   // (j-cluster, half-shell index | i-cluster mask << 8)
+    __shared__ int s_cnt[kListWarps], s_e0, s_c0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (*p.err & ERR_CELL) return;
+    const int n_sc = p.counters[0];
+    const float rcb = list_rlist_f(p) + kBBoxMargin;
+    const float rcb2 = rcb * rcb;
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.counters[2] = 0;   // work counter of the force kernel
+    for (int sc = blockIdx.x; sc < n_sc; sc += gridDim.x) {
+        const ListSC s = list_sc(p, sc);
+        int total;
+        const ListCell c = list_cells(p, s, lane, &total);
+        __syncthreads();   // the previous SC's reads are done
+        if ((int)threadIdx.x < s.ncl) {
+            w.lo[threadIdx.x] = p.bb_lo[s.fc + threadIdx.x];
+            w.hi[threadIdx.x] = p.bb_hi[s.fc + threadIdx.x];
+            w.fr[threadIdx.x] = p.bb_frag[s.fc + threadIdx.x];
+        }
+        list_stage_atoms(p, w, s, threadIdx.x, blockDim.x);
+        __syncthreads();
+        const int i0 = (int)((long long)total * warp / kListWarps), i1 = (int)((long long)total * (warp + 1) / kListWarps);
+        int cnt = 0;
+        for (int base = i0; base < i1; base += 32) {
+            const ListJ j = list_j(p, w, s, c, base + lane, i1, rcb2);
+            const unsigned bal = __ballot_sync(kFull, j.m != 0u);
+            const int at = cnt + __popc(bal & ((1u << lane) - 1u));
+            if (j.m && at < kFound) s_found[warp][at] = make_uint2((unsigned)j.jc, (unsigned)j.nb | (j.m << 8));
+            cnt += __popc(bal);
+        }
+        if (lane == 0) s_cnt[warp] = cnt;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int tot = 0;
+            for (int k = 0; k < kListWarps; ++k) tot += s_cnt[k];
+            const int nch = (tot + kChunk - 1) / kChunk;
+            int e0 = atomicAdd(&p.counters[6], tot), c0 = atomicAdd(&p.counters[7], nch);
+            if ((long long)e0 + tot > p.pl_cap || (long long)c0 + nch > p.chunk_cap) {
+                atomicOr(p.err, ERR_LIST);
+                e0 = -1;
+            }
+            s_e0 = e0;
+            s_c0 = c0;
+        }
+        __syncthreads();
+        const int e0 = s_e0;
+        if (e0 < 0) continue;   // uniform across the block
+        int off = e0, tot = 0;
+        for (int k = 0; k < kListWarps; ++k) {
+            if (k < warp) off += s_cnt[k];
+            tot += s_cnt[k];
+        }
+        for (int t = threadIdx.x; t * kChunk < tot; t += blockDim.x)
+            p.pl_chunk[s_c0 + t] = make_int4(s.fc, e0 + t * kChunk, min(kChunk, tot - t * kChunk) | (s.ncl << 16), s.rr);
+        if (cnt <= kFound) {
+            for (int b = 0; b < cnt; b += 32) {
+                ListJ j;
+                j.jc = 0;
+                j.nb = 0;
+                j.m = 0u;
+                j.jl = j.jh = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (b + lane < cnt) {
+                    const uint2 f = s_found[warp][b + lane];
+                    j.jc = (int)f.x;
+                    j.nb = (int)(f.y & 0xffu);
+                    j.m = f.y >> 8;
+                }
+                const float Dx = __shfl_sync(kFull, c.Dx, j.nb), Dy = __shfl_sync(kFull, c.Dy, j.nb),
+                            Dz = __shfl_sync(kFull, c.Dz, j.nb);
+                if (j.m) {
+                    const float4 lo = p.bb_lo[j.jc], hi = p.bb_hi[j.jc];
+                    j.jl = make_float4(lo.x + Dx, lo.y + Dy, lo.z + Dz, 0.0f);
+                    j.jh = make_float4(hi.x + Dx, hi.y + Dy, hi.z + Dz, 0.0f);
+                }
+                const uint4 e = list_entry(p, w, j, __reduce_or_sync(kFull, j.m), rcb2);
+                if (j.m) p.pl[off + b + lane] = e;
+            }
+        } else {
+            for (int base = i0; base < i1; base += 32) {
+                const ListJ j = list_j(p, w, s, c, base + lane, i1, rcb2);
+                const unsigned bal = __ballot_sync(kFull, j.m != 0u);
+                const uint4 e = list_entry(p, w, j, __reduce_or_sync(kFull, j.m), rcb2);
+                if (j.m) p.pl[off + __popc(bal & ((1u << lane) - 1u))] = e;
+                off += __popc(bal);
+            }
+        }
     }
 }
 
@@ -1780,8 +1891,12 @@ int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
     return std::max(1, std::min(24 / warps, (int)(233472 / block)));
 }
 
-int launch_pair_list(const Params& p, cudaStream_t s, int blocks)
+int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm)
 {
+    if (p.sc_cap <= kListFusedScs) {
+        k_list_fused<<<std::min(p.sc_cap, n_sm * 8), kListWarps * 32, 0, s>>>(p);
+        return 1;
+    }
     int n = 2;
     k_list_count<<<blocks, kListWarps * 32, 0, s>>>(p);
     if (p.sc_cap >= kScanScsMulti) {

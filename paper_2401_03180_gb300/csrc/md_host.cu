@@ -184,7 +184,7 @@ void enqueue_rebuild(md_handle* h, cudaStream_t s, bool energy)
 {
     launch_step_a(h->P, 0, s, h->grid_atoms);
     launch_cells(h->P, s, h->grid_atoms, h->grid_cells, h->sort_threads);
-    launch_pair_list(h->P, s, h->list_blocks);
+    launch_pair_list(h->P, s, h->list_blocks, h->n_sm);
     set_build_step(h, s, true);   // forces at the build positions: the list may be pruned
     launch_pair_forces(h->P, s, energy, h->pair_blocks, h->pair_warps);
     launch_probe(h->P, s, true);
@@ -204,7 +204,7 @@ void enqueue_rebuild_from_ref(md_handle* h, cudaStream_t s)
     }
     launch_step_a(P, 0, s, h->grid_atoms);
     launch_cells(P, s, h->grid_atoms, h->grid_cells, h->sort_threads);
-    launch_pair_list(P, s, h->list_blocks);
+    launch_pair_list(P, s, h->list_blocks, h->n_sm);
     // a force pass at the build positions trims the entries' masks as the step
     // of the original build did (its forces are discarded; the trimmed atoms
     // only add exact zeros, so the forces below are the same either way)
@@ -223,7 +223,7 @@ void enqueue_step(md_handle* h, cudaStream_t s, bool events)
     int mode = STEP_KICK_DRIFT | STEP_ADVANCE | (h->cfg.cr_enabled ? STEP_CR : 0);
     launch_step_a(h->P, mode, s, h->grid_atoms);
     h->build_kernels = launch_cells(h->P, s, h->grid_atoms, h->grid_cells, h->sort_threads) +
-                       launch_pair_list(h->P, s, h->list_blocks);
+                       launch_pair_list(h->P, s, h->list_blocks, h->n_sm);
     // external event nodes: the events are recorded on every graph replay
     if (events) cudaEventRecordWithFlags(h->ev_pair0, s, cudaEventRecordExternal);
     launch_pair_forces(h->P, s, false, h->pair_blocks, h->pair_warps);
@@ -319,7 +319,7 @@ md_status capture_buffered_step(md_handle* h, bool events)
     cudaGraph_t rebuild = cp.conditional.phGraph_out[0];
     CU(cudaStreamBeginCaptureToGraph(h->body_stream, rebuild, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     h->build_kernels = launch_cells(h->P, h->body_stream, h->grid_atoms, h->grid_cells, h->sort_threads) +
-                       launch_pair_list(h->P, h->body_stream, h->list_blocks);
+                       launch_pair_list(h->P, h->body_stream, h->list_blocks, h->n_sm);
     CU(cudaStreamEndCapture(h->body_stream, &rebuild));
     CU(cudaStreamUpdateCaptureDependencies(s, &cn, nullptr, 1, cudaStreamSetCaptureDependencies));
     if (events) cudaEventRecordWithFlags(h->ev_pair0, s, cudaEventRecordExternal);
@@ -461,7 +461,7 @@ md_status autotune(md_handle* h)
                 float ms = 0.0f;
                 md_status s = timed([&]() {
                     launch_cells(h->P, h->stream, h->grid_atoms, h->grid_cells, st);
-                    launch_pair_list(h->P, h->stream, lblocks);
+                    launch_pair_list(h->P, h->stream, lblocks, h->n_sm);
                 }, &ms);
                 if (s != MD_OK) return s;
                 if (ms < best) { best = ms; bs = st; bl = lb; }
