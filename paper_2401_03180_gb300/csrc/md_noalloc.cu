@@ -15,10 +15,10 @@
 // It runs the same kernels as a handle's initial force evaluation (cell
 // build, pair forces, read-out), so its forces equal those of md_init +
 // md_get_state(MD_FIELD_F) on the same input.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
-#include <vector>
 
 #include "md.h"
 #include "md_internal.cuh"
@@ -92,11 +92,37 @@ constexpr Layout kL = make_layout();
 __device__ __align__(256) unsigned char g_md_scratch[kL.total];
 
 unsigned char* g_base[64] = {nullptr};   // device address of the scratch, per device
+int g_n_sm[64] = {0};                    // multiprocessors, per device
 
 md_status fail(md_status s, const std::string& m)
 {
     set_global_error(m);   // read back through md_last_error(NULL)
     return s;
+}
+
+// The species tables of one call, by value.
+struct NaTables {
+    int ns, nts;
+    int z[MD_MAX_SPECIES], ts_off[MD_MAX_SPECIES + 1];
+    double sig0[MD_MAX_SPECIES], eps0[MD_MAX_SPECIES];
+};
+
+// LJ constants of a pair of type states: sigma scaled by 1 - q/Z,
+// arithmetic-mean sigma, geometric-mean epsilon.  Explicit roundings: the same
+// values as the host-built table of a handle.
+__device__ void lj_pair(const NaTables& t, int a, int b, double& c6, double& c12)
+{
+    int sa = 0, sb = 0;
+    while (sa + 1 < t.ns && a >= t.ts_off[sa + 1]) ++sa;
+    while (sb + 1 < t.ns && b >= t.ts_off[sb + 1]) ++sb;
+    const double ga = __dmul_rn(t.sig0[sa], __dsub_rn(1.0, __ddiv_rn((double)(a - t.ts_off[sa]), (double)t.z[sa])));
+    const double gb = __dmul_rn(t.sig0[sb], __dsub_rn(1.0, __ddiv_rn((double)(b - t.ts_off[sb]), (double)t.z[sb])));
+    const double sg = __dmul_rn(0.5, __dadd_rn(ga, gb));
+    const double ep = __dsqrt_rn(__dmul_rn(t.eps0[sa], t.eps0[sb]));
+    double s6 = sg;
+    for (int k = 1; k < 6; ++k) s6 = __dmul_rn(s6, sg);
+    c6 = __dmul_rn(__dmul_rn(4.0, ep), s6);
+    c12 = __dmul_rn(c6, s6);
 }
 
 // Reset of the per-call state and the copy of the caller's atoms into the
@@ -105,20 +131,37 @@ md_status fail(md_status s, const std::string& m)
 // index is not below n_species or whose charge exceeds its species' Z raises
 // ERR_INPUT (the call then returns MD_ERR_INVALID_ARG) and is stored as a
 // neutral atom of species 0, so that every later table lookup stays in bounds.
-// The error word is cleared on the stream before this kernel runs.
-__global__ void k_noalloc_prepare(Params p, const double* __restrict__ x, const uint8_t* __restrict__ sp,
-                                  const uint8_t* __restrict__ q, const int32_t* __restrict__ fr, int slot_cap,
-                                  int cell_cap)
+// The error word is cleared on the stream before this kernel runs.  The tables,
+// the grid and the small constants are kernel arguments and are written here:
+// as six host-to-device copies and a host-built LJ table they took 17 of the 162 us of a
+// call of 12,297 atoms.
+__global__ void k_noalloc_prepare(Params p, NaTables tb, Grid g, double volume, const double* __restrict__ x,
+                                  const uint8_t* __restrict__ sp, const uint8_t* __restrict__ q,
+                                  const int32_t* __restrict__ fr, int slot_cap, int cell_cap)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = p.n_atoms;
+    for (int k = t; k < tb.nts * tb.nts; k += gridDim.x * blockDim.x) {
+        double c6, c12;
+        lj_pair(tb, k / tb.nts, k % tb.nts, c6, c12);
+        if (p.precision == 0) const_cast<float2*>(p.lj_f)[k] = make_float2((float)__dmul_rn(6.0, c6), (float)__dmul_rn(6.0, c12));
+        else const_cast<double2*>(p.lj_d)[k] = make_double2(__dmul_rn(-6.0, c6), __dmul_rn(-kLn2, c12));
+    }
+    if (t <= tb.ns) const_cast<int*>(p.ts_off)[t] = tb.ts_off[t];
+    if (t < tb.ns) const_cast<int*>(p.zs)[t] = tb.z[t];
+    if (t == 0) {
+        p.grid[0] = g;
+        const_cast<double*>(p.volume)[0] = volume;
+        const_cast<int*>(p.rep_off)[0] = 0;
+        const_cast<int*>(p.rep_off)[1] = n;
+    }
     if (t < n) {
         p.x[t] = x[3 * t + 0];
         p.y[t] = x[3 * t + 1];
         p.z[t] = x[3 * t + 2];
         p.vx[t] = 0.0; p.vy[t] = 0.0; p.vz[t] = 0.0;
         int st = sp[t], qt = q[t];
-        if (st >= p.n_species || qt > p.zs[st]) {
+        if (st >= tb.ns || qt > tb.z[st]) {
             atomicOr(p.err, ERR_INPUT);
             st = 0;
             qt = 0;
@@ -258,49 +301,26 @@ extern "C" md_status md_forces_noalloc(const md_forces_input* in, double* d_f, v
     P.xr = P.yr = P.zr = nullptr;
     P.maxd2 = nullptr; P.builds = nullptr; P.cond = 0;
 
-    // host-built tables: LJ per pair of type states (sigma scaled by 1 - q/Z,
-    // arithmetic-mean sigma, geometric-mean epsilon), offsets, the grid
-    std::vector<double> sig(nts), eps(nts);
-    for (int k = 0; k < in->n_species; ++k)
-        for (int qq = 0; qq <= in->z[k]; ++qq) {
-            sig[ts_off[k] + qq] = in->lj_sigma0[k] * (1.0 - (double)qq / (double)in->z[k]);
-            eps[ts_off[k] + qq] = in->lj_eps0[k];
-        }
-    std::vector<double2> tab_d((size_t)nts * nts);
-    std::vector<float2> tab_f((size_t)nts * nts);
-    for (int a = 0; a < nts; ++a)
-        for (int b = 0; b < nts; ++b) {
-            const double sg = 0.5 * (sig[a] + sig[b]);
-            const double ep = std::sqrt(eps[a] * eps[b]);
-            const double s6 = sg * sg * sg * sg * sg * sg;
-            const double c6 = 4.0 * ep * s6, c12 = c6 * s6;
-            tab_d[(size_t)a * nts + b] = make_double2(-6.0 * c6, -kLn2 * c12);   // pair kernels take (-6 c6, -ln2 c12)
-            tab_f[(size_t)a * nts + b] = make_float2((float)(6.0 * c6), (float)(6.0 * c12));
-        }
-    const int zs[MD_MAX_SPECIES] = {in->z[0], in->z[1], in->z[2], in->z[3], in->z[4], in->z[5], in->z[6], in->z[7]};
-    const double one = 1.0;
-    const int rep_off[2] = {0, n};
+    NaTables tb{};
+    tb.ns = in->n_species;
+    tb.nts = nts;
+    for (int k = 0; k < in->n_species; ++k) {
+        tb.z[k] = in->z[k];
+        tb.sig0[k] = in->lj_sigma0[k];
+        tb.eps0[k] = in->lj_eps0[k];
+    }
+    for (int k = 0; k <= in->n_species; ++k) tb.ts_off[k] = ts_off[k];
 #define NA_CU(call)                                                                                 \
     do {                                                                                            \
         const cudaError_t e_ = (call);                                                              \
         if (e_ != cudaSuccess) return fail(MD_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
-    if (in->precision == MD_PREC_MIXED)
-        NA_CU(cudaMemcpyAsync(B + kL.lj, tab_f.data(), tab_f.size() * sizeof(float2), cudaMemcpyHostToDevice, s));
-    else
-        NA_CU(cudaMemcpyAsync(B + kL.lj, tab_d.data(), tab_d.size() * sizeof(double2), cudaMemcpyHostToDevice, s));
-    NA_CU(cudaMemcpyAsync(B + kL.zs, zs, sizeof(zs), cudaMemcpyHostToDevice, s));
-    NA_CU(cudaMemcpyAsync(B + kL.ts_off, ts_off, sizeof(ts_off), cudaMemcpyHostToDevice, s));
-    NA_CU(cudaMemcpyAsync(B + kL.volume, &one, sizeof(double), cudaMemcpyHostToDevice, s));
-    NA_CU(cudaMemcpyAsync(B + kL.rep_off, rep_off, sizeof(rep_off), cudaMemcpyHostToDevice, s));
-    NA_CU(cudaMemcpyAsync(B + kL.grid, &g, sizeof(Grid), cudaMemcpyHostToDevice, s));
-
     NA_CU(cudaMemsetAsync(P.err, 0, sizeof(unsigned), s));
     const int span = std::max(P.slot_cap, std::max(n, g.cell_cap));
-    k_noalloc_prepare<<<(span + 255) / 256, 256, 0, s>>>(P, in->d_x, in->d_species, in->d_q, in->d_fragment,
+    k_noalloc_prepare<<<(span + 255) / 256, 256, 0, s>>>(P, tb, g, 1.0, in->d_x, in->d_species, in->d_q, in->d_fragment,
                                                           P.slot_cap, g.cell_cap);
-    int n_sm = 0;
-    NA_CU(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    if (!g_n_sm[dev]) NA_CU(cudaDeviceGetAttribute(&g_n_sm[dev], cudaDevAttrMultiProcessorCount, dev));
+    const int n_sm = g_n_sm[dev];
     const int warps = 8;
     const int blocks = n_sm * std::max(1, pair_max_blocks_per_sm(in->precision == MD_PREC_FP64, false, false, warps, nts, n));
     launch_step_a(P, 0, s, (n + 255) / 256);                           // grid and screening
