@@ -304,30 +304,77 @@ __global__ void __launch_bounds__(256) k_cell_scatter(Params p)
     p.tmp_key[p.cell_start[c] + p.atom_rank[i]] = ((unsigned long long)key << 32) | (unsigned)i;
 }
 
-// One CTA per cell: rank sort of the cell's keys (Hilbert index, atom), with
-// up to 8 threads sharing the count of one element; then the packed arrays
-// and the cluster bounding boxes.  Launched with 1,024 threads when there are
-// few cells per SM (large cells, all sorted at once) and 256 when there are
-// many: a cell's phases are latency-bound, and seven 256-thread CTAs per SM
-// keep more cells in flight than two 1,024-thread ones.
-// Order-preserving integer image of a float (for min/max with integer atomics).
-__device__ __forceinline__ int ord_f(float f)
+// Packed records and cluster boxes of one cell from its atoms in slot order
+// (order[e]: the atom of slot ps + e, e < n): consecutive threads take
+// consecutive slots, so records are written coalesced, the FP64 subtractions
+// run in full warps, and a cluster's box is a shuffle reduction over its eight
+// lanes.  Threads t of n_threads (whole warps) take part.
+__device__ __forceinline__ void pack_cell(const Params& p, const int* order, int ps, int n, int npad, const double cen[3],
+                                          const Grid& g, int t, int n_threads)
 {
-    const int i = __float_as_int(f);
-    return i < 0 ? i ^ 0x7fffffff : i;
+    constexpr unsigned kFull = 0xffffffffu;
+    const int n32 = (npad + 31) & ~31;
+    for (int e = t; e < n32; e += n_threads) {
+        const int slot = ps + e;
+        float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
+        int fmin = 0x7fffffff, fmax = (int)0x80000000;
+        if (e < n) {
+            const int i = order[e];
+            p.atom_of[slot] = i;
+            p.slot_of[i] = slot;
+            const double xi[3] = {p.x[i], p.y[i], p.z[i]};
+            const int fr = p.frag[i];
+            const float4 v = pack_record(p, slot, xi, cen, g.periodic, g.box, p.species[i], p.q[i], fr);
+            lo[0] = hi[0] = v.x;
+            lo[1] = hi[1] = v.y;
+            lo[2] = hi[2] = v.z;
+            fmin = fmax = fr;
+        } else if (e < npad) {   // padding: far away, no charge
+            const double far = 1.0e6 + 1024.0 * (double)slot;
+            p.atom_of[slot] = -1;
+            if (p.precision == 0) p.xq[slot] = make_float4((float)far, 1.0e6f, 1.0e6f, 0.0f);
+            else p.xq64[slot] = make_double4_32a(far, 1.0e6, 1.0e6, 0.0);
+            p.tf[slot] = make_int2(0, -1 - slot);
+            p.fx[slot] = 0; p.fy[slot] = 0; p.fz[slot] = 0; p.epot[slot] = 0;
+        }
+#pragma unroll
+        for (int o = 1; o < kClusterSize; o <<= 1) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                lo[d] = fminf(lo[d], __shfl_xor_sync(kFull, lo[d], o));
+                hi[d] = fmaxf(hi[d], __shfl_xor_sync(kFull, hi[d], o));
+            }
+            fmin = min(fmin, __shfl_xor_sync(kFull, fmin, o));
+            fmax = max(fmax, __shfl_xor_sync(kFull, fmax, o));
+        }
+        if (e < npad && (e & (kClusterSize - 1)) == 0) {
+            const int cl = slot / kClusterSize;
+            p.cl_cen[cl] = make_double4_32a(cen[0], cen[1], cen[2], 0.0);
+            p.bb_lo[cl] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+            p.bb_hi[cl] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+            p.bb_frag[cl] = make_int2(fmin, fmax);
+        }
+    }
 }
-__device__ __forceinline__ float unord_f(int i) { return __int_as_float(i < 0 ? i ^ 0x7fffffff : i); }
 
+// One CTA per cell: rank sort of the cell's keys (Hilbert index, atom), with
+// up to 8 threads sharing the count of one element, into the cell's slot order;
+// then the packed records and the cluster boxes.  Launched with 1,024 threads
+// when there are few cells per SM (large cells, all sorted at once) and 256 when
+// there are many: a cell's phases are latency-bound, and several 256-thread CTAs
+// per SM keep more cells in flight than two 1,024-thread ones.  Packing by the
+// threads that ranked (every 4th or 8th lane active, scattered stores, eight
+// shared-memory atomics per atom for the boxes) took 15.5 us for 30,000 atoms in
+// 125 cells against 12.8 now, 13.7 against 10.8 for 12,297 in 64, and 69 against
+// 57 for 199,773 in 729.
+//
 // small_max < 0: every cell; else only the cells k_cell_sort_small listed as
 // larger than it could take (p.big_cells[0 .. counters[4])).
 __global__ void __launch_bounds__(kSortThreads) k_cell_sort_pack(Params p, int small_max)
 {
     const int nt = blockDim.x;
     __shared__ unsigned long long s_key[kSortMax];
-    // cluster boxes of a cell held in shared memory (ordered-integer min x, y, z,
-    // max x, y, z, min and max fragment), built with integer atomics as the
-    // atoms are packed
-    __shared__ int s_bb[kSortMax / kClusterSize][8];
+    __shared__ int s_order[kSortMax];
     if (*p.err & ERR_CELL) return;
     const int tid = threadIdx.x;
     const int n_cells = small_max < 0 ? p.cell_cap_total : p.counters[4];
@@ -358,16 +405,9 @@ __global__ void __launch_bounds__(kSortThreads) k_cell_sort_pack(Params p, int s
                                g.origin[2] + (cz + 0.5) * g.edge[2]};
         const bool in_smem = n <= kSortMax;
         const unsigned long long* keys = in_smem ? s_key : p.tmp_key + b;
-        const int ncl = npad / kClusterSize;
-        if (in_smem) {
+        int* order = in_smem ? s_order : p.atom_of + ps;
+        if (in_smem)
             for (int e = tid; e < n; e += nt) s_key[e] = p.tmp_key[b + e];
-            for (int k = tid; k < ncl; k += nt) {
-                s_bb[k][0] = s_bb[k][1] = s_bb[k][2] = 0x7fffffff;
-                s_bb[k][3] = s_bb[k][4] = s_bb[k][5] = (int)0x80000000;
-                s_bb[k][6] = 0x7fffffff;
-                s_bb[k][7] = (int)0x80000000;
-            }
-        }
         __syncthreads();
         int tpe = 1;
         while (tpe < 8 && 2 * tpe * n <= nt) tpe *= 2;
@@ -379,90 +419,31 @@ __global__ void __launch_bounds__(kSortThreads) k_cell_sort_pack(Params p, int s
             int rank = 0;
             if (e < n) {
                 ke = keys[e];
+#pragma unroll 4
                 for (int f = sub; f < n; f += tpe) rank += keys[f] < ke;
             }
             for (int o = 1; o < tpe; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-            if (e < n && sub == 0) {
-                const int i = (int)(ke & 0xffffffffu);
-                const int slot = ps + rank;
-                p.atom_of[slot] = i;
-                p.slot_of[i] = slot;
-                const float4 v = pack_slot(p, slot, i, cen, g);
-                if (in_smem) {
-                    int* bb = s_bb[rank / kClusterSize];
-                    atomicMin(bb + 0, ord_f(v.x)); atomicMin(bb + 1, ord_f(v.y)); atomicMin(bb + 2, ord_f(v.z));
-                    atomicMax(bb + 3, ord_f(v.x)); atomicMax(bb + 4, ord_f(v.y)); atomicMax(bb + 5, ord_f(v.z));
-                    const int fr = p.frag[i];
-                    atomicMin(bb + 6, fr);
-                    atomicMax(bb + 7, fr);
-                }
-            }
+            if (e < n && sub == 0) order[rank] = (int)(ke & 0xffffffffu);
         }
-        for (int e = n + tid; e < npad; e += nt) {     // padding: far away, no charge
-            const int slot = ps + e;
-            const double far = 1.0e6 + 1024.0 * (double)slot;
-            p.atom_of[slot] = -1;
-            if (p.precision == 0) p.xq[slot] = make_float4((float)far, 1.0e6f, 1.0e6f, 0.0f);
-            else p.xq64[slot] = make_double4_32a(far, 1.0e6, 1.0e6, 0.0);
-            p.tf[slot] = make_int2(0, -1 - slot);
-            p.fx[slot] = 0; p.fy[slot] = 0; p.fz[slot] = 0; p.epot[slot] = 0;
-        }
-        __syncthreads();
-        // cluster bounding boxes (real atoms only) and fragment ranges
-        if (in_smem) {
-            for (int k = tid; k < ncl; k += nt) {
-                const int cl = ps / kClusterSize + k;
-                p.cl_cen[cl] = make_double4_32a(cen[0], cen[1], cen[2], 0.0);
-                p.bb_lo[cl] = make_float4(unord_f(s_bb[k][0]), unord_f(s_bb[k][1]), unord_f(s_bb[k][2]), 0.0f);
-                p.bb_hi[cl] = make_float4(unord_f(s_bb[k][3]), unord_f(s_bb[k][4]), unord_f(s_bb[k][5]), 0.0f);
-                p.bb_frag[cl] = make_int2(s_bb[k][6], s_bb[k][7]);
-            }
-            __syncthreads();
-            continue;
-        }
-        for (int k = tid; k < ncl; k += nt) {
-            float lx = 3.0e38f, ly = 3.0e38f, lz = 3.0e38f, hx = -3.0e38f, hy = -3.0e38f, hz = -3.0e38f;
-            int fmin = 0x7fffffff, fmax = (int)0x80000000;
-            for (int a = 0; a < kClusterSize; ++a) {
-                const int slot = ps + k * kClusterSize + a;
-                if (a + k * kClusterSize >= n) break;
-                float vx, vy, vz;
-                if (p.precision == 0) {
-                    const float4 t = p.xq[slot];
-                    vx = t.x; vy = t.y; vz = t.z;
-                } else {
-                    const double4_32a t = p.xq64[slot];
-                    vx = (float)t.x; vy = (float)t.y; vz = (float)t.z;
-                }
-                lx = fminf(lx, vx); hx = fmaxf(hx, vx);
-                ly = fminf(ly, vy); hy = fmaxf(hy, vy);
-                lz = fminf(lz, vz); hz = fmaxf(hz, vz);
-                const int fr = p.tf[slot].y;
-                fmin = min(fmin, fr);
-                fmax = max(fmax, fr);
-            }
-            const int cl = ps / kClusterSize + k;
-            p.cl_cen[cl] = make_double4_32a(cen[0], cen[1], cen[2], 0.0);
-            p.bb_lo[cl] = make_float4(lx, ly, lz, 0.0f);
-            p.bb_hi[cl] = make_float4(hx, hy, hz, 0.0f);
-            p.bb_frag[cl] = make_int2(fmin, fmax);
-        }
+        __syncthreads();   // (cells beyond kSortMax: the order is in global memory, visible to the block)
+        pack_cell(p, order, ps, n, npad, cen, g, tid, nt);
         __syncthreads();
     }
 }
 
 // Cells of up to kSmallCell atoms: one warp per cell, with the same rank sort,
 // packed records and cluster boxes as k_cell_sort_pack but no block barrier,
-// so that many more (latency-bound) cells are in flight.  Keys and boxes live
+// so that many more (latency-bound) cells are in flight.  Keys and order live
 // in the warp's share of shared memory; every lane reads the cell's keys as
 // broadcasts.
 __global__ void __launch_bounds__(kSmallWarps * 32) k_cell_sort_small(Params p)
 {
     __shared__ unsigned long long s_key[kSmallWarps][kSmallCell];
-    __shared__ int s_bb[kSmallWarps][kSmallCell / kClusterSize][8];
+    __shared__ int s_order[kSmallWarps][kSmallCell];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (*p.err & ERR_CELL) return;
     unsigned long long* key = s_key[warp];
+    int* order = s_order[warp];
     for (int c = blockIdx.x * kSmallWarps + warp; c < p.cell_cap_total; c += gridDim.x * kSmallWarps) {
         const int b = p.cell_start[c];
         const int n = p.cell_start[c + 1] - b;
@@ -486,52 +467,18 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_cell_sort_small(Params p)
         const double cen[3] = {g.origin[0] + (cx + 0.5) * g.edge[0],
                                g.origin[1] + (cy + 0.5) * g.edge[1],
                                g.origin[2] + (cz + 0.5) * g.edge[2]};
-        const int ncl = npad / kClusterSize;
         __syncwarp();
         for (int e = lane; e < n; e += 32) key[e] = p.tmp_key[b + e];
-        for (int k = lane; k < ncl; k += 32) {
-            int* bb = s_bb[warp][k];
-            bb[0] = bb[1] = bb[2] = 0x7fffffff;
-            bb[3] = bb[4] = bb[5] = (int)0x80000000;
-            bb[6] = 0x7fffffff;
-            bb[7] = (int)0x80000000;
-        }
         __syncwarp();
         for (int e = lane; e < n; e += 32) {
             const unsigned long long ke = key[e];
             int rank = 0;
 #pragma unroll 4
             for (int f = 0; f < n; ++f) rank += key[f] < ke;
-            const int i = (int)(ke & 0xffffffffu);
-            const int slot = ps + rank;
-            p.atom_of[slot] = i;
-            p.slot_of[i] = slot;
-            const float4 v = pack_slot(p, slot, i, cen, g);
-            int* bb = s_bb[warp][rank / kClusterSize];
-            atomicMin(bb + 0, ord_f(v.x)); atomicMin(bb + 1, ord_f(v.y)); atomicMin(bb + 2, ord_f(v.z));
-            atomicMax(bb + 3, ord_f(v.x)); atomicMax(bb + 4, ord_f(v.y)); atomicMax(bb + 5, ord_f(v.z));
-            const int fr = p.frag[i];
-            atomicMin(bb + 6, fr);
-            atomicMax(bb + 7, fr);
-        }
-        for (int e = n + lane; e < npad; e += 32) {     // padding: far away, no charge
-            const int slot = ps + e;
-            const double far = 1.0e6 + 1024.0 * (double)slot;
-            p.atom_of[slot] = -1;
-            if (p.precision == 0) p.xq[slot] = make_float4((float)far, 1.0e6f, 1.0e6f, 0.0f);
-            else p.xq64[slot] = make_double4_32a(far, 1.0e6, 1.0e6, 0.0);
-            p.tf[slot] = make_int2(0, -1 - slot);
-            p.fx[slot] = 0; p.fy[slot] = 0; p.fz[slot] = 0; p.epot[slot] = 0;
+            order[rank] = (int)(ke & 0xffffffffu);
         }
         __syncwarp();
-        for (int k = lane; k < ncl; k += 32) {
-            const int* bb = s_bb[warp][k];
-            const int cl = ps / kClusterSize + k;
-            p.cl_cen[cl] = make_double4_32a(cen[0], cen[1], cen[2], 0.0);
-            p.bb_lo[cl] = make_float4(unord_f(bb[0]), unord_f(bb[1]), unord_f(bb[2]), 0.0f);
-            p.bb_hi[cl] = make_float4(unord_f(bb[3]), unord_f(bb[4]), unord_f(bb[5]), 0.0f);
-            p.bb_frag[cl] = make_int2(bb[6], bb[7]);
-        }
+        pack_cell(p, order, ps, n, npad, cen, g, lane, 32);
     }
 }
 
