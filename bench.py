@@ -417,6 +417,7 @@ def run_gpu(args, rank, world, local):
                "d2h_bytes_per_step": int(n_atoms + 104 * s.n_replicas + 4)}
 
     dt_fs = 5e-5 * 1000.0
+    wide_step = -(-n_atoms // 32) >= 16 * sms
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W_,
         "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -459,9 +460,11 @@ def run_gpu(args, rank, world, local):
         "e2e": e2e,
         # per step: step kernel + force kernel (the bonded terms run inside it) (+ the
         # probe kernel; + the warp-per-replica reduction above 4 replicas, the step
-        # kernel's inline limit), and the build's kernels (cells + list, 5 to 12 by
-        # grid size) in the steps whose list is rebuilt
-        "gpu_launches": (2 + bool(args.probe) + (s.n_replicas > 4)) * K + tim.build_kernels * int(tim.list_builds),
+        # kernel's inline limit; + the total rates and that reduction from 16 blocks of
+        # 32 atoms per SM on), and the build's kernels (cells + list, 5 to 12 by grid
+        # size) in the steps whose list is rebuilt
+        "gpu_launches": (2 + bool(args.probe) + (s.n_replicas > 4 or wide_step) + wide_step) * K
+                        + tim.build_kernels * int(tim.list_builds),
         "pair_list": {"skin_nm": args.skin, "skin_mode": args.skin_mode, "builds": int(tim.list_builds),
                       "unbuffered_builds": int(tim.list_unbuffered_builds), "steps": K,
                       "steps_per_build": (K / tim.list_builds) if tim.list_builds else None,

@@ -74,47 +74,6 @@ __device__ __forceinline__ double interp(const double* K, int i0, double w)
     return __dadd_rn(K[i0], __dmul_rn(w, __dsub_rn(K[i0 + 1], K[i0])));
 }
 
-// ---------------------------------------------------------------------------
-// Per-replica scalars for the step `step` (Eq. 3 and the CR helpers) and
-// the cell grid for the positions just reduced into the bounding box.
-// Executed by one thread per replica.
-// ---------------------------------------------------------------------------
-__device__ void plasma_scalars(const Params& p, int r, long long step, RepState& st)
-{
-    double te, ne;
-    if (p.plasma_mode == 1) {
-        long long idx = (long long)r * (p.max_steps + 1) + (step <= p.max_steps ? step : p.max_steps);
-        ne = p.pres_ne[idx];
-        te = p.pres_te[idx];
-    } else if (st.n_e > 0) {
-        te = __ddiv_rn((double)st.e_gas, __dmul_rn(1500.0, (double)st.n_e));
-        ne = __ddiv_rn((double)st.n_e, p.volume[r]);
-    } else {
-        te = 0.0;
-        ne = 0.0;
-    }
-    double kap = 0.0;
-    if (ne > 0.0) {
-        double tc = te > p.te_floor ? te : p.te_floor;
-        double k2 = __ddiv_rn(__dmul_rn(p.four_pi_f, ne), __dmul_rn(tc, kEvKJmol));
-        kap = __dsqrt_rn(k2);
-    }
-    st.te_ev = te;
-    st.n_dens = ne;
-    st.kappa = kap;
-    st.ne_dt = __dmul_rn(ne, p.dt);
-    double x = __dmul_rn(te, p.inv_dte);
-    if (x > (double)(p.n_te - 1)) x = (double)(p.n_te - 1);
-    if (x < 0.0) x = 0.0;
-    int i0 = (int)x;
-    if (i0 > p.n_te - 2) i0 = p.n_te - 2;
-    st.it0 = i0;
-    st.wt = __dsub_rn(x, (double)i0);
-    double kf = p.kappa_fixed >= 0.0 ? p.kappa_fixed : kap;
-    st.kappa_force = kf;
-    st.kappa_f = (float)kf;
-}
-
 // Adaptive skin: whether this step rebuilds (x) and whether the list it builds
 // carries the skin (y), from the step's largest displacement and the current
 // list.  A pure function, so that the warps sizing the grids and the thread
@@ -137,40 +96,6 @@ __device__ __forceinline__ double next_rlist(const Params& p, unsigned maxd2)
 {
     if (SETCOND && p.lc) return adapt_decision(p, maxd2).y ? p.r_list : p.r_cut;
     return list_rlist(p);
-}
-
-__device__ void make_grid(const Params& p, int r, const unsigned long long* mn,
-                          const unsigned long long* mx, double rl)
-{
-    Grid& g = p.grid[r];
-    if (g.periodic) return;   // periodic grids are fixed at init
-    double lo[3], hi[3];
-    for (int d = 0; d < 3; ++d) {
-        lo[d] = mn[d] == ~0ull ? 0.0 : from_ordered(mn[d]);
-        hi[d] = mx[d] == 0ull ? 0.0 : from_ordered(mx[d]);
-        if (!(hi[d] >= lo[d])) { lo[d] = 0.0; hi[d] = 0.0; }
-    }
-    double f = 1.0;   // cell edges >= rl, the radius of the list built on the grid
-    int n[3];
-    for (int it = 0; it < 400; ++it) {
-        long long prod = 1;
-        for (int d = 0; d < 3; ++d) {
-            double m = floor((hi[d] - lo[d]) / (rl * f));
-            n[d] = m < 1.0 ? 1 : (m > 1.0e6 ? 1000000 : (int)m);
-            prod *= n[d];
-        }
-        if (prod <= g.cell_cap) break;
-        f *= 1.125;
-    }
-    for (int d = 0; d < 3; ++d) {
-        double ext = hi[d] - lo[d];
-        double e = n[d] == 1 ? (ext > rl ? ext : rl) : ext / n[d];
-        g.origin[d] = lo[d];
-        g.edge[d] = e;
-        g.inv_edge[d] = 1.0 / e;
-        g.edge_f[d] = (float)e;
-        g.dims[d] = n[d];
-    }
 }
 
 // Velocity increment of a half kick, (dt/2m) F.  The mixed path forms it in
@@ -273,49 +198,146 @@ __device__ void hyb_table(const Params& p, int rr, int lane, double kap, double 
     }
 }
 
-// Replica rr's per-step reduction by one warp: lane c reads accumulator copy
-// c and clears it, the warp reduces, lane 0 updates the plasma scalars (Eq. 3)
-// and the next grid.
+// Replica rr's per-step reduction by one warp, the plasma scalars of the next
+// step (Eq. 3 and the helpers of the charge update) and, for a vacuum replica,
+// the cell grid for the positions just reduced into the bounding box.
+//
+// This runs at the end of every step with nothing else on the GPU, so its chain
+// of dependent operations counts: lane f < 12 loads field f of all accumulator
+// copies at once and reduces (and clears) them; the FP64 divisions, each some
+// hundreds of cycles on GB300's FP64 pipe, are issued once for several lanes:
+// T_e on lane 0, n_e on lane 1 and the grid's three dimensions on lanes 2 to 4.
+// One lane after the other (thirteen divisions and a square root in a row) the
+// step kernel took 15.9 us for 1,500 methane atoms in vacuum and 19.4 us for the
+// 45k-atom droplet; now 13.0 and 17.9 us.  Periodic boxes, whose grid stands, take
+// what they took (water box 14.4 us).
 __device__ void finalize_replica(const Params& p, int rr, int lane, long long next, double rl)
 {
-    RepAccum* a = p.acc + (size_t)rr * kAccCopies;
-    RepState st;
-    if (lane == 0) st = p.rs[rr];   // issued before the accumulators are read and cleared
-    long long v[6] = {0, 0, 0, 0, 0, 0};
-    unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
-    if (lane < kAccCopies) {
-        v[0] = __ldcg(&a[lane].dNe);
-        v[1] = __ldcg(&a[lane].dE);
-        for (int k = 0; k < 4; ++k) v[2 + k] = __ldcg(&a[lane].counts[k]);
-        for (int d = 0; d < 3; ++d) {
-            mn[d] = __ldcg(&a[lane].bmin[d]);
-            mx[d] = __ldcg(&a[lane].bmax[d]);
-        }
-        a[lane].dNe = 0;
-        a[lane].dE = 0;
-        for (int k = 0; k < 4; ++k) a[lane].counts[k] = 0;
-        for (int d = 0; d < 3; ++d) {
-            a[lane].bmin[d] = ~0ull;
-            a[lane].bmax[d] = 0ull;
+    constexpr unsigned kFull = 0xffffffffu;
+    static_assert(sizeof(RepAccum) == 12 * sizeof(long long), "twelve fields of eight bytes");
+    RepState st{};
+    double vol = 1.0, pne = 0.0, pte = 0.0;
+    if (lane == 0) {   // issued before the accumulators are read and cleared
+        st = p.rs[rr];
+        if (p.plasma_mode == 1) {
+            const long long idx = (long long)rr * (p.max_steps + 1) + (next <= p.max_steps ? next : p.max_steps);
+            pne = p.pres_ne[idx];
+            pte = p.pres_te[idx];
         }
     }
-    for (int o = kAccCopies / 2; o; o >>= 1) {   // lanes 0..kAccCopies-1 hold the copies
-        for (int k = 0; k < 6; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        for (int d = 0; d < 3; ++d) {
-            const unsigned long long x = __shfl_xor_sync(0xffffffffu, mn[d], o);
-            const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx[d], o);
-            mn[d] = x < mn[d] ? x : mn[d];
-            mx[d] = y > mx[d] ? y : mx[d];
+    if (lane == 1) vol = p.volume[rr];
+    Grid& g = p.grid[rr];
+    const int periodic = g.periodic, cell_cap = g.cell_cap;
+    // sums on lanes 0 to 5; the box's lower ends (as complements) and upper ends as
+    // maxima on lanes 6 to 11; both by a tree over the copies
+    unsigned long long sum = 0ull, mx = 0ull;
+    if (lane < 12) {
+        unsigned long long* f = reinterpret_cast<unsigned long long*>(p.acc + (size_t)rr * kAccCopies) + lane;
+        const unsigned long long flip = lane >= 6 && lane < 9 ? ~0ull : 0ull;
+        unsigned long long v[kAccCopies], m[kAccCopies];
+#pragma unroll
+        for (int c = 0; c < kAccCopies; ++c) v[c] = __ldcg(f + 12 * c);
+#pragma unroll
+        for (int c = 0; c < kAccCopies; ++c) {
+            m[c] = v[c] ^ flip;
+            f[12 * c] = flip;
+        }
+#pragma unroll
+        for (int o = kAccCopies / 2; o; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < o; ++c) {
+                v[c] += v[c + o];
+                m[c] = max(m[c], m[c + o]);
+            }
+        sum = v[0];
+        mx = m[0] ^ flip;
+    }
+    // lane 0: the electron gas; lanes 2 to 4: one dimension of the bounding box each
+    const long long dE = (long long)__shfl_sync(kFull, sum, 1);
+    long long dc[4];
+    for (int k = 0; k < 4; ++k) dc[k] = (long long)__shfl_sync(kFull, sum, 2 + k);
+    const int d = lane >= 2 && lane < 5 ? lane - 2 : 0;
+    const unsigned long long mn = __shfl_sync(kFull, mx, 6 + d);
+    mx = __shfl_sync(kFull, mx, 9 + d);
+    if (lane == 0) {
+        st.n_e += (long long)sum;
+        st.e_gas += dE;
+        if (st.e_gas < 0) st.e_gas = 0;
+        for (int k = 0; k < 4; ++k) st.counts[k] += dc[k];
+    }
+    double lo = mn == ~0ull ? 0.0 : from_ordered(mn), hi = mx == 0ull ? 0.0 : from_ordered(mx);
+    if (!(hi >= lo)) lo = hi = 0.0;
+    const double ext = hi - lo;
+    const long long n_e = __shfl_sync(kFull, st.n_e, 0);
+    double num = 1.0, den = 1.0, f = 1.0;   // f: cell edges >= f rl, rl the radius of the list built on the grid
+    if (lane == 0 && n_e > 0) {
+        num = (double)st.e_gas;
+        den = __dmul_rn(1500.0, (double)n_e);
+    } else if (lane == 1 && n_e > 0) {
+        num = (double)n_e;
+        den = vol;
+    } else if (!periodic && lane >= 2 && lane < 5) {   // (a zero numerator takes the division's slow path)
+        num = ext;
+        den = rl * f;
+    }
+    double quo = __ddiv_rn(num, den);
+    double te = 0.0, ne = 0.0;   // lane 0
+    const double n_dens = __shfl_sync(kFull, quo, 1);
+    if (p.plasma_mode == 1) {
+        ne = pne;
+        te = pte;
+    } else if (n_e > 0) {
+        te = quo;
+        ne = n_dens;
+    }
+    int n = 1;
+    if (!periodic) {
+        for (int it = 0; it < 400; ++it) {
+            const double m = floor(quo);
+            n = m < 1.0 ? 1 : (m > 1.0e6 ? 1000000 : (int)m);
+            const long long prod = (long long)__shfl_sync(kFull, n, 2) * __shfl_sync(kFull, n, 3) * __shfl_sync(kFull, n, 4);
+            if (prod <= cell_cap) break;
+            f *= 1.125;
+            quo = __ddiv_rn(ext, rl * f);
+        }
+    }
+    num = den = 1.0;
+    if (lane == 0 && ne > 0.0) {
+        const double tc = te > p.te_floor ? te : p.te_floor;
+        num = __dmul_rn(p.four_pi_f, ne);
+        den = __dmul_rn(tc, kEvKJmol);
+    } else if (!periodic && lane >= 2 && lane < 5) {
+        num = ext;
+        den = (double)n;
+    }
+    quo = __ddiv_rn(num, den);
+    if (!periodic) {
+        if (lane >= 2 && lane < 5) {
+            const double e = n == 1 ? (ext > rl ? ext : rl) : quo;
+            g.origin[d] = lo;
+            g.edge[d] = e;
+            g.inv_edge[d] = 1.0 / e;
+            g.edge_f[d] = (float)e;
+            g.dims[d] = n;
         }
     }
     if (lane == 0) {
-        st.n_e += v[0];
-        st.e_gas += v[1];
-        if (st.e_gas < 0) st.e_gas = 0;
-        for (int k = 0; k < 4; ++k) st.counts[k] += v[2 + k];
-        plasma_scalars(p, rr, next, st);
+        const double kap = ne > 0.0 ? __dsqrt_rn(quo) : 0.0;
+        st.te_ev = te;
+        st.n_dens = ne;
+        st.kappa = kap;
+        st.ne_dt = __dmul_rn(ne, p.dt);
+        double x = __dmul_rn(te, p.inv_dte);
+        if (x > (double)(p.n_te - 1)) x = (double)(p.n_te - 1);
+        if (x < 0.0) x = 0.0;
+        int i0 = (int)x;
+        if (i0 > p.n_te - 2) i0 = p.n_te - 2;
+        st.it0 = i0;
+        st.wt = __dsub_rn(x, (double)i0);
+        const double kf = p.kappa_fixed >= 0.0 ? p.kappa_fixed : kap;
+        st.kappa_force = kf;
+        st.kappa_f = (float)kf;
         p.rs[rr] = st;
-        make_grid(p, rr, mn, mx, rl);
     }
     if (p.screening) {
         const double kap = __shfl_sync(0xffffffffu, st.kappa_force, 0);
@@ -372,6 +394,318 @@ __device__ void finalize_step(const Params& p, int mode, long long next, unsigne
     }
 }
 
+// Smallest (largest) of the lanes' 64-bit keys: the high words by one warp
+// reduction, then the low words of the lanes that hold it.
+template <bool MAX>
+__device__ __forceinline__ unsigned long long warp_extreme(unsigned long long v)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+    const unsigned h = MAX ? __reduce_max_sync(kFull, hi) : __reduce_min_sync(kFull, hi);
+    const unsigned c = hi == h ? lo : (MAX ? 0u : 0xffffffffu);
+    const unsigned l = MAX ? __reduce_max_sync(kFull, c) : __reduce_min_sync(kFull, c);
+    return ((unsigned long long)h << 32) | l;
+}
+
+// Half kicks, Langevin update, drift and periodic wrap of atom i: (ax, ay, az)
+// is the half kick's velocity increment.
+__device__ __forceinline__ void kick_drift(const Params& p, const Grid& g, int r, int s, int i, long long step, int kick_full,
+                                           double ax, double ay, double az, double& vx, double& vy, double& vz, double& x,
+                                           double& y, double& z)
+{
+    // the state holds v_{n-1/2} once stepping has started: finish the
+    // previous step's half kick, then this step's (two separate adds,
+    // exactly as velocity Verlet rounds them)
+    if (kick_full) { vx = vx + ax; vy = vy + ay; vz = vz + az; }
+    vx = vx + ax; vy = vy + ay; vz = vz + az;
+    if (p.langevin) {
+        // electron-ion coupling (Eqs. 13-14): exact Ornstein-Uhlenbeck
+        // update with Philox stream 1 of (seed, atom, step)
+        const double2 cs = p.lgv[(size_t)r * kMaxSpecies + s];
+        const unsigned long long sd = p.seed[r];
+        const uint4 w4 = philox4x32_10(make_uint4((unsigned)p.local_id[i], (unsigned)step, 1u, 0u),
+                                       make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
+        double gx, gy, gz;
+        gauss3(w4, p.precision == 0, gx, gy, gz);
+        vx = cs.x * vx + cs.y * gx;
+        vy = cs.x * vy + cs.y * gy;
+        vz = cs.x * vz + cs.y * gz;
+    }
+    // x + dt v with one rounding (GB300 issues FP64 at 2 lanes per SM per clock)
+    x = __fma_rn(p.dt, vx, x);
+    y = __fma_rn(p.dt, vy, y);
+    z = __fma_rn(p.dt, vz, z);
+    if (g.periodic) {
+        // wrap only atoms that left the box (FP64 division is slow); the
+        // tests run on the bit patterns
+        const double L0 = g.box[0], L1 = g.box[1], L2 = g.box[2];
+        if (below_zero(x) || at_or_above(x, L0)) { x -= L0 * floor(x / L0); if (x >= L0) x -= L0; }
+        if (below_zero(y) || at_or_above(y, L1)) { y -= L1 * floor(y / L1); if (y >= L1) y -= L1; }
+        if (below_zero(z) || at_or_above(z, L2)) { z -= L2 * floor(z / L2); if (z >= L2) z -= L2; }
+    }
+    // finite check on the exponent bits (integer ops; FP64 compares are slow here)
+    if (((__double2hiint(x) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(y) & 0x7ff00000) == 0x7ff00000) ||
+        ((__double2hiint(z) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(vx) & 0x7ff00000) == 0x7ff00000) ||
+        ((__double2hiint(vy) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(vz) & 0x7ff00000) == 0x7ff00000))
+        atomicOr(p.err, ERR_NONFINITE);
+}
+
+// Squared displacement since the last list build (minimum image) as the bits of
+// an FP32 number: it only decides the rebuild, against half the skin.
+// Non-negative floats order like their bit patterns (NaN sorts high).
+__device__ __forceinline__ unsigned moved2(const Params& p, const Grid& g, int i, double x, double y, double z)
+{
+    double d[3] = {x - p.xr[i], y - p.yr[i], z - p.zr[i]};
+    if (g.periodic)
+        for (int k = 0; k < 3; ++k) {
+            const int o = beyond_half(d[k], g.box[k]);
+            if (o > 0) d[k] -= g.box[k];
+            else if (o < 0) d[k] += g.box[k];
+        }
+    const float e0 = (float)d[0], e1 = (float)d[1], e2 = (float)d[2];
+    return __float_as_uint(e0 * e0 + e1 * e1 + e2 * e2);
+}
+
+// Rates of one atom in type state ts (species s of nuclear charge Z, charge q)
+// with K-hole flag h: the running sums of the four channels (Sec. II.A).
+struct Rates {
+    double a_pi, a_a, a_ci, a_rec, c1, c2, lam;
+};
+__device__ __forceinline__ Rates cr_rates(const Params& p, const RepState& st, double dF, int ts, int s, int Z, int q, int h)
+{
+    Rates x;
+    x.a_pi = __dmul_rn(p.sigma_pi[2 * ts + h], dF);
+    x.a_a = h ? p.auger_dt[s] : 0.0;
+    x.a_ci = 0.0;
+    x.a_rec = 0.0;
+    if (q < Z) x.a_ci = __dmul_rn(st.ne_dt, interp(p.k_ci + (long long)ts * p.n_te, st.it0, st.wt));
+    if (q > 0 && h == 0) x.a_rec = __dmul_rn(st.ne_dt, interp(p.k_rec + (long long)ts * p.n_te, st.it0, st.wt));
+    x.c1 = __dadd_rn(x.a_pi, x.a_a);
+    x.c2 = __dadd_rn(x.c1, x.a_ci);
+    x.lam = __dadd_rn(x.c2, x.a_rec);
+    return x;
+}
+
+// The channel that t, uniform in [0, lam), falls into: 0 PI, 1 Auger, 2 CI, 3 REC.
+__device__ __forceinline__ int cr_channel(const Rates& x, double t)
+{
+    if (t < x.a_pi) return 0;
+    if (t < x.c1) return 1;
+    if (t < x.c2) return 2;
+    if (t < x.lam) return 3;
+    return x.a_rec > 0.0 ? 3 : (x.a_ci > 0.0 ? 2 : (x.a_a > 0.0 ? 1 : 0));
+}
+
+// Applies an event of channel ch to (q, h) of type state ts; returns the energy
+// given to the electron gas (meV).
+__device__ __forceinline__ long long cr_event(const Params& p, int ch, int ts, int s, int Z, int& q, int& h)
+{
+    long long de;
+    if (ch == 0) {
+        de = p.e_pi_mev[2 * ts + h];
+        q += 1;
+        if (q == Z) h = 0;
+        else if (Z >= 3 && h == 0 && Z - q >= 2) h = 1;
+    } else if (ch == 1) {
+        q += 1;
+        h = 0;
+        de = p.e_auger_mev[s];
+    } else if (ch == 2) {
+        q += 1;
+        if (q == Z) h = 0;
+        de = -p.ip_mev[ts];
+    } else {
+        q -= 1;
+        de = p.ip_mev[ts - 1];
+    }
+    return de;
+}
+
+// Total rate of every (replica, type state, K-hole flag) at the step about to be
+// taken, for the step kernel of large systems: an atom then tests its uniform
+// against one table entry, and only the few that may have an event evaluate
+// the rates (the same expressions, so the same values).
+__global__ void __launch_bounds__(128) k_rates(Params p)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= p.n_rep * p.n_ts * 2) return;
+    const int r = k / (2 * p.n_ts), h = k & 1, ts = (k >> 1) % p.n_ts;
+    int s = 0;
+    while (s + 1 < p.n_species && ts >= p.ts_off[s + 1]) ++s;
+    const long long step = *p.step;
+    const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
+    p.rate_tab[k] = cr_rates(p, p.rs[r], dF, ts, s, p.zs[s], ts - p.ts_off[s], h).lam;
+}
+
+// Bounding box of the vacuum replicas' atoms into the block's window of replicas
+// from r0 (whole warps; one atom per lane, r = -1: none).
+__device__ __forceinline__ void box_update(const Params& p, int r, int r0, bool vac, const double pos[3],
+                                           unsigned long long (*s_bmin)[3], unsigned long long (*s_bmax)[3])
+{
+    const unsigned full = 0xffffffffu;
+    const int rl0 = __shfl_sync(full, r, 0);
+    const bool uniform = __all_sync(full, r == rl0) && rl0 >= 0;
+    const bool any_vac = __any_sync(full, vac);
+    if (any_vac) {
+        if (uniform) {
+            if (__shfl_sync(full, (int)vac, 0)) {
+                for (int d = 0; d < 3; ++d) {
+                    const unsigned long long key = ordered_bits(pos[d]);
+                    const unsigned long long mn = warp_extreme<false>(key), mx = warp_extreme<true>(key);
+                    if ((threadIdx.x & 31) == 0) {
+                        const int w = rl0 - r0;
+                        if (w < kRepWindow) {
+                            atomicMin(&s_bmin[w][d], mn);
+                            atomicMax(&s_bmax[w][d], mx);
+                        } else {
+                            RepAccum* a = p.acc + (size_t)rl0 * kAccCopies + (blockIdx.x & (kAccCopies - 1));
+                            atomicMin(&a->bmin[d], mn);
+                            atomicMax(&a->bmax[d], mx);
+                        }
+                    }
+                }
+            }
+        } else if (vac) {
+            const int w = r - r0;
+            for (int d = 0; d < 3; ++d) {
+                unsigned long long o = ordered_bits(pos[d]);
+                if (w < kRepWindow) {
+                    atomicMin(&s_bmin[w][d], o);
+                    atomicMax(&s_bmax[w][d], o);
+                } else {
+                    RepAccum* a = p.acc + (size_t)r * kAccCopies + (blockIdx.x & (kAccCopies - 1));
+                    atomicMin(&a->bmin[d], o);
+                    atomicMax(&a->bmax[d], o);
+                }
+            }
+        }
+    }
+}
+
+// The block's sums and boxes of replicas r0 .. r0 + nw - 1 into the accumulators.
+__device__ __forceinline__ void flush_block(const Params& p, int r0, int nw, long long (*s_acc)[6],
+                                            unsigned long long (*s_bmin)[3], unsigned long long (*s_bmax)[3])
+{
+    for (int k = threadIdx.x; k < nw * 12; k += blockDim.x) {
+        const int w = k / 12, f = k % 12;
+        RepAccum* a = p.acc + (size_t)(r0 + w) * kAccCopies + (blockIdx.x & (kAccCopies - 1));
+        if (f < 6) {
+            const long long v = s_acc[w][f];
+            if (v != 0) {
+                unsigned long long* dst = f == 0 ? (unsigned long long*)&a->dNe
+                                        : f == 1 ? (unsigned long long*)&a->dE
+                                                 : (unsigned long long*)&a->counts[f - 2];
+                atomicAdd(dst, (unsigned long long)v);
+            }
+        } else if (f < 9) {
+            if (s_bmin[w][f - 6] != ~0ull) atomicMin(&a->bmin[f - 6], s_bmin[w][f - 6]);
+        } else {
+            if (s_bmax[w][f - 9] != 0ull) atomicMax(&a->bmax[f - 9], s_bmax[w][f - 9]);
+        }
+    }
+}
+
+// The full step of large systems with rates: a thread does an atom's kick, drift,
+// charge update (against the table of total rates) and re-pack, with all of its
+// loads issued before the first use and no barrier in between; k_step_fin
+// reduces the replicas.  Two threads per atom (k_step_a) shorten the chain of a
+// system that leaves the chip idle, but with many blocks per SM the instructions
+// count: FP64 runs at 2 lanes per SM and clock here, and evaluating the rates
+// was most of the charge role's work, for an event in one atom of some hundreds.
+// 2 M-atom droplet: 302.6 us -> 203 + 3.9 (k_rates) + 7.5 us (k_step_fin), 1.9 TB/s
+// of state; 1,024 x 1,500 methane: 188.1 + 16.3 -> 147.0 + 4.0 + 9.5 us.  Blocks of
+// 64 atoms took 1 % less than 128.
+constexpr int kWideAtoms = 64;
+__global__ void __launch_bounds__(kWideAtoms, 16) k_step_wide(Params p)
+{
+    __shared__ long long s_acc[kRepWindow][6];
+    __shared__ unsigned long long s_bmin[kRepWindow][3], s_bmax[kRepWindow][3];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int first = blockIdx.x * kWideAtoms;
+    const int last = min(first + kWideAtoms, p.n_atoms) - 1;
+    const int i = min(first + tid, last);
+    const bool live = first + tid <= last;
+    const unsigned err = *p.err;
+    const long long step = *p.step;
+    const int kick_full = *p.kick_full;
+    const int r0 = p.rep[first], r_last = p.rep[last], r = p.rep[i];
+    const int s = p.species[i], slot = p.slot_of[i], qi = p.q[i], hi = p.h[i], fr = p.frag[i], loc = p.local_id[i];
+    double x = p.x[i], y = p.y[i], z = p.z[i];
+    double vx = p.vx[i], vy = p.vy[i], vz = p.vz[i];
+    const bool repack = p.xr != nullptr;
+    double4_32a cen = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    if (repack) cen = p.cl_cen[slot / kClusterSize];
+    double ax, ay, az;
+    half_kick(p, s, slot, ax, ay, az);
+    const int Z = p.zs[s], ts = p.ts_off[s] + qi;
+    const unsigned long long sd = p.seed[r];
+    const double lam = p.rate_tab[((long long)r * p.n_ts + ts) * 2 + hi];
+    const Grid& g = p.grid[r];
+    const int nw = min(r_last - r0 + 1, kRepWindow);
+    for (int k = tid; k < nw * 6; k += kWideAtoms) (&s_acc[0][0])[k] = 0;
+    for (int k = tid; k < nw * 3; k += kWideAtoms) {
+        (&s_bmin[0][0])[k] = ~0ull;
+        (&s_bmax[0][0])[k] = 0ull;
+    }
+    // a cluster-pair list overflow freezes the state (see k_step_a)
+    if (err & ERR_LIST) return;
+    __syncthreads();
+    unsigned d2_bits = 0u;
+    double pos[3] = {0.0, 0.0, 0.0};
+    if (live) {
+        kick_drift(p, g, r, s, i, step, kick_full, ax, ay, az, vx, vy, vz, x, y, z);
+        if (repack) d2_bits = moved2(p, g, i, x, y, z);
+        p.vx[i] = vx; p.vy[i] = vy; p.vz[i] = vz;
+        p.x[i] = x; p.y[i] = y; p.z[i] = z;
+        pos[0] = x; pos[1] = y; pos[2] = z;
+        int qn = qi;
+        if (step >= p.max_steps) atomicOr(p.err, ERR_TABLE_END);
+        // the tests of k_step_a, on the table's total rate
+        if (__double_as_longlong(lam) > 0ll) {
+            const uint4 w4 = philox4x32_10(make_uint4((unsigned)loc, (unsigned)step, 0u, 0u),
+                                           make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
+            const double u0 = u53(w4.x, w4.y);
+            if ((unsigned long long)__double_as_longlong(u0) < (unsigned long long)__double_as_longlong(lam) &&
+                u0 < one_minus_exp_neg(lam, p.etab, p.inv12)) {
+                const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
+                const Rates c = cr_rates(p, p.rs[r], dF, ts, s, Z, qi, hi);
+                const int ch = cr_channel(c, __dmul_rn(u53(w4.z, w4.w), c.lam));
+                int hn = hi;
+                const long long de = cr_event(p, ch, ts, s, Z, qn, hn);
+                p.q[i] = (uint8_t)qn;
+                p.h[i] = (uint8_t)hn;
+                const int w = r - r0;
+                unsigned long long* acc[3];
+                if (w < kRepWindow) {
+                    acc[0] = (unsigned long long*)&s_acc[w][0];
+                    acc[1] = (unsigned long long*)&s_acc[w][1];
+                    acc[2] = (unsigned long long*)&s_acc[w][2 + ch];
+                } else {
+                    RepAccum* a = p.acc + (size_t)r * kAccCopies + (blockIdx.x & (kAccCopies - 1));
+                    acc[0] = (unsigned long long*)&a->dNe;
+                    acc[1] = (unsigned long long*)&a->dE;
+                    acc[2] = (unsigned long long*)&a->counts[ch];
+                }
+                atomicAdd(acc[0], (unsigned long long)(ch == 3 ? -1ll : 1ll));
+                atomicAdd(acc[1], (unsigned long long)de);
+                atomicAdd(acc[2], 1ull);
+            }
+        }
+        if (repack) {
+            const Grid& gb = p.grid_b[r];
+            const double c[3] = {cen.x, cen.y, cen.z};
+            pack_record(p, slot, pos, c, gb.periodic, gb.box, s, qn, fr);
+        }
+    }
+    if (repack) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, d2_bits);
+        if (lane == 0 && m) atomicMax(p.maxd2, m);
+    }
+    box_update(p, live ? r : -1, r0, live && !g.periodic, pos, s_bmin, s_bmax);
+    __syncthreads();
+    flush_block(p, r0, nw, s_acc, s_bmin, s_bmax);
+}
+
 // SETCOND: the Verlet-buffered variant that decides the rebuild and sets the
 // graph condition (ncu does not profile kernels that can set one, so the
 // every-step variant is a separate instantiation).  MINB: resident blocks per
@@ -379,7 +713,7 @@ __device__ void finalize_step(const Params& p, int mode, long long next, unsigne
 // per SM, where the FP64 pipe binds and more resident warps pay (2 M-atom
 // droplet: 3.80 -> 3.71 ms per step); 10 (96 registers) for small grids, which
 // are latency-bound (water box: 108.4 against 110.9 us per step with 16)
-template <bool SETCOND, int MINB>
+template <bool SETCOND, int MINB, bool FIN>
 __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mode)
 {
     __shared__ long long s_acc[kRepWindow][6];
@@ -414,6 +748,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
     int r = live ? p.rep[i] : -1;
     double pos[3] = {0.0, 0.0, 0.0};
     bool vac = false;
+    unsigned d2_bits = 0u;   // squared displacement since the last build
     // inputs of this atom's re-pack (Verlet-buffered list), loaded before the
     // charge update is waited for
     const bool repack = live && !cr_role && p.xr && (mode & STEP_KICK_DRIFT);
@@ -435,61 +770,15 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
             pk_q = p.q[i];
         }
         if (mode & STEP_KICK_DRIFT) {
-            // the state holds v_{n-1/2} once stepping has started: finish the
-            // previous step's half kick, then this step's (two separate adds,
-            // exactly as velocity Verlet rounds them)
             double ax, ay, az;
             half_kick(p, s, p.slot_of[i], ax, ay, az);
             double vx = p.vx[i], vy = p.vy[i], vz = p.vz[i];
-            if (kick_full) { vx = vx + ax; vy = vy + ay; vz = vz + az; }
-            vx = vx + ax; vy = vy + ay; vz = vz + az;
-            if (p.langevin) {
-                // electron-ion coupling (Eqs. 13-14): exact Ornstein-Uhlenbeck
-                // update with Philox stream 1 of (seed, atom, step)
-                const double2 cs = p.lgv[(size_t)r * kMaxSpecies + s];
-                const unsigned long long sd = p.seed[r];
-                const uint4 w4 = philox4x32_10(make_uint4((unsigned)p.local_id[i], (unsigned)step, 1u, 0u),
-                                               make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
-                double gx, gy, gz;
-                gauss3(w4, p.precision == 0, gx, gy, gz);
-                vx = cs.x * vx + cs.y * gx;
-                vy = cs.x * vy + cs.y * gy;
-                vz = cs.x * vz + cs.y * gz;
-            }
-            // x + dt v with one rounding (GB300 issues FP64 at 2 lanes per SM per clock)
-            x = __fma_rn(p.dt, vx, x);
-            y = __fma_rn(p.dt, vy, y);
-            z = __fma_rn(p.dt, vz, z);
             const Grid& g = p.grid[r];
-            if (g.periodic) {
-                // wrap only atoms that left the box (FP64 division is slow); the
-                // tests run on the bit patterns
-                const double L0 = g.box[0], L1 = g.box[1], L2 = g.box[2];
-                if (below_zero(x) || at_or_above(x, L0)) { x -= L0 * floor(x / L0); if (x >= L0) x -= L0; }
-                if (below_zero(y) || at_or_above(y, L1)) { y -= L1 * floor(y / L1); if (y >= L1) y -= L1; }
-                if (below_zero(z) || at_or_above(z, L2)) { z -= L2 * floor(z / L2); if (z >= L2) z -= L2; }
-            }
-            // finite check on the exponent bits (integer ops; FP64 compares are slow here)
-            if (((__double2hiint(x) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(y) & 0x7ff00000) == 0x7ff00000) ||
-                ((__double2hiint(z) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(vx) & 0x7ff00000) == 0x7ff00000) ||
-                ((__double2hiint(vy) & 0x7ff00000) == 0x7ff00000) || ((__double2hiint(vz) & 0x7ff00000) == 0x7ff00000))
-                atomicOr(p.err, ERR_NONFINITE);
+            kick_drift(p, g, r, s, i, step, kick_full, ax, ay, az, vx, vy, vz, x, y, z);
             p.vx[i] = vx; p.vy[i] = vy; p.vz[i] = vz;
             p.x[i] = x; p.y[i] = y; p.z[i] = z;
             if (p.xr) {
-                // displacement since the last list build (minimum image), squared
-                // in FP32: it only decides the rebuild, against half the skin
-                double d[3] = {x - p.xr[i], y - p.yr[i], z - p.zr[i]};
-                if (g.periodic)
-                    for (int k = 0; k < 3; ++k) {
-                        const int o = beyond_half(d[k], g.box[k]);
-                        if (o > 0) d[k] -= g.box[k];
-                        else if (o < 0) d[k] += g.box[k];
-                    }
-                const float e0 = (float)d[0], e1 = (float)d[1], e2 = (float)d[2];
-                const float d2 = e0 * e0 + e1 * e1 + e2 * e2;
-                // non-negative floats order like their bit patterns (NaN sorts high)
-                atomicMax(&s_maxd2, __float_as_uint(d2));
+                d2_bits = moved2(p, g, i, x, y, z);
             }
         }
         pos[0] = x; pos[1] = y; pos[2] = z;
@@ -497,50 +786,13 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
     }
 
     // ---- bounding box of vacuum replicas (warp-reduced when uniform) ----
-    {
+    if (!cr_role) {   // whole warps
         const unsigned full = 0xffffffffu;
-        const int rl0 = __shfl_sync(full, r, 0);
-        const bool uniform = __all_sync(full, r == rl0) && rl0 >= 0;
-        const bool any_vac = __any_sync(full, vac);
-        if (any_vac) {
-            if (uniform) {
-                if (__shfl_sync(full, (int)vac, 0)) {
-                    for (int d = 0; d < 3; ++d) {
-                        unsigned long long mn = ordered_bits(pos[d]), mx = mn;
-                        for (int o = 16; o; o >>= 1) {
-                            unsigned long long a = __shfl_xor_sync(full, mn, o);
-                            unsigned long long b = __shfl_xor_sync(full, mx, o);
-                            mn = a < mn ? a : mn;
-                            mx = b > mx ? b : mx;
-                        }
-                        if (lane == 0) {
-                            const int w = rl0 - r0;
-                            if (w < kRepWindow) {
-                                atomicMin(&s_bmin[w][d], mn);
-                                atomicMax(&s_bmax[w][d], mx);
-                            } else {
-                                RepAccum* a = p.acc + (size_t)rl0 * kAccCopies + (blockIdx.x & (kAccCopies - 1));
-                                atomicMin(&a->bmin[d], mn);
-                                atomicMax(&a->bmax[d], mx);
-                            }
-                        }
-                    }
-                }
-            } else if (vac) {
-                const int w = r - r0;
-                for (int d = 0; d < 3; ++d) {
-                    unsigned long long o = ordered_bits(pos[d]);
-                    if (w < kRepWindow) {
-                        atomicMin(&s_bmin[w][d], o);
-                        atomicMax(&s_bmax[w][d], o);
-                    } else {
-                        RepAccum* a = p.acc + (size_t)r * kAccCopies + (blockIdx.x & (kAccCopies - 1));
-                        atomicMin(&a->bmin[d], o);
-                        atomicMax(&a->bmax[d], o);
-                    }
-                }
-            }
+        if (p.xr && (mode & STEP_KICK_DRIFT)) {
+            const unsigned m = __reduce_max_sync(full, d2_bits);
+            if (lane == 0) s_maxd2 = m;   // one kick warp per block
         }
+        box_update(p, r, r0, vac, pos, s_bmin, s_bmax);
     }
 
     // ---- collisional-radiative update (reading of Sec. II.A) ----
@@ -589,58 +841,26 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
         const int qi = p.q[i], hi = p.h[i];
         s_q[i - first] = (uint8_t)qi;   // replaced below if an event changes it
         const int ts = p.ts_off[s] + qi;
-        const RepState st = p.rs[r];
-        double dF = 0.0;
-        if (step < p.max_steps) dF = p.dF[(long long)r * p.max_steps + step];
-        else atomicOr(p.err, ERR_TABLE_END);
-        const double a_pi = __dmul_rn(p.sigma_pi[2 * ts + hi], dF);
-        const double a_a = hi ? p.auger_dt[s] : 0.0;
-        double a_ci = 0.0, a_rec = 0.0;
-        if (qi < Z) a_ci = __dmul_rn(st.ne_dt, interp(p.k_ci + (long long)ts * p.n_te, st.it0, st.wt));
-        if (qi > 0 && hi == 0)
-            a_rec = __dmul_rn(st.ne_dt, interp(p.k_rec + (long long)ts * p.n_te, st.it0, st.wt));
-        const double c1 = __dadd_rn(a_pi, a_a);
-        const double c2 = __dadd_rn(c1, a_ci);
-        const double lam = __dadd_rn(c2, a_rec);
+        if (step >= p.max_steps) atomicOr(p.err, ERR_TABLE_END);
+        const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
+        const Rates x = cr_rates(p, p.rs[r], dF, ts, s, Z, qi, hi);
         int ch = -1;
         // lam and u0 are non-negative doubles, whose order is that of their
         // bit patterns: the tests run in the integer pipe
-        if (__double_as_longlong(lam) > 0ll) {
+        if (__double_as_longlong(x.lam) > 0ll) {
             const unsigned long long sd = p.seed[r];
             const uint4 w4 = philox4x32_10(make_uint4((unsigned)p.local_id[i], (unsigned)step, 0u, 0u),
                                            make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
             const double u0 = u53(w4.x, w4.y);
             // 1 - e^{-lam} <= lam, so u0 >= lam decides "no event" exactly
-            if ((unsigned long long)__double_as_longlong(u0) < (unsigned long long)__double_as_longlong(lam) &&
-                u0 < one_minus_exp_neg(lam, p.etab, p.inv12)) {
-                const double t = __dmul_rn(u53(w4.z, w4.w), lam);
-                if (t < a_pi) ch = 0;
-                else if (t < c1) ch = 1;
-                else if (t < c2) ch = 2;
-                else if (t < lam) ch = 3;
-                else ch = a_rec > 0.0 ? 3 : (a_ci > 0.0 ? 2 : (a_a > 0.0 ? 1 : 0));
+            if ((unsigned long long)__double_as_longlong(u0) < (unsigned long long)__double_as_longlong(x.lam) &&
+                u0 < one_minus_exp_neg(x.lam, p.etab, p.inv12)) {
+                ch = cr_channel(x, __dmul_rn(u53(w4.z, w4.w), x.lam));
             }
         }
         if (ch >= 0) {
             int qn = qi, hn = hi;
-            long long de;
-            if (ch == 0) {
-                qn = qi + 1;
-                de = p.e_pi_mev[2 * ts + hi];
-                if (qn == Z) hn = 0;
-                else if (Z >= 3 && hi == 0 && Z - qn >= 2) hn = 1;
-            } else if (ch == 1) {
-                qn = qi + 1;
-                hn = 0;
-                de = p.e_auger_mev[s];
-            } else if (ch == 2) {
-                qn = qi + 1;
-                if (qn == Z) hn = 0;
-                de = -p.ip_mev[ts];
-            } else {
-                qn = qi - 1;
-                de = p.ip_mev[ts - 1];
-            }
+            const long long de = cr_event(p, ch, ts, s, Z, qn, hn);
             p.q[i] = (uint8_t)qn;
             p.h[i] = (uint8_t)hn;
             s_q[i - first] = (uint8_t)qn;
@@ -672,30 +892,14 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
         const int last_atom = min(first + kStepAtoms, p.n_atoms) - 1;
         const int r_last = p.rep[last_atom];
         const int nw = min(r_last - r0 + 1, kRepWindow);
-        for (int k = tid; k < nw * 12; k += blockDim.x) {
-            const int w = k / 12, f = k % 12;
-            RepAccum* a = p.acc + (size_t)(r0 + w) * kAccCopies + (blockIdx.x & (kAccCopies - 1));
-            if (f < 6) {
-                const long long v = s_acc[w][f];
-                if (v != 0) {
-                    unsigned long long* dst = f == 0 ? (unsigned long long*)&a->dNe
-                                            : f == 1 ? (unsigned long long*)&a->dE
-                                                     : (unsigned long long*)&a->counts[f - 2];
-                    atomicAdd(dst, (unsigned long long)v);
-                }
-            } else if (f < 9) {
-                if (s_bmin[w][f - 6] != ~0ull) atomicMin(&a->bmin[f - 6], s_bmin[w][f - 6]);
-            } else {
-                if (s_bmax[w][f - 9] != 0ull) atomicMax(&a->bmax[f - 9], s_bmax[w][f - 9]);
-            }
-        }
+        flush_block(p, r0, nw, s_acc, s_bmin, s_bmax);
     }
 
     if (tid == 0 && s_maxd2) atomicMax(p.maxd2, s_maxd2);
 
     // ---- per-replica reduction (Eq. 3) and next grid: by this kernel's last
     // block for a few replicas, by k_step_fin (a warp per replica) for more ----
-    if (p.n_rep > kInlineReps) return;
+    if constexpr (FIN) return;
     __threadfence();
     __syncthreads();
     if (tid == 0) s_last = (atomicAdd(&p.counters[3], 1) == (int)gridDim.x - 1);
@@ -754,14 +958,24 @@ void launch_step_a(const Params& p, int mode, cudaStream_t s, int grid_atoms)
     const int blocks = (p.n_atoms + kStepAtoms - 1) / kStepAtoms;
     const int fin_blocks = (p.n_rep * 32 + 255) / 256;
     const bool wide = blocks >= kWide * n_sm;
-    if (mode & STEP_SETCOND) {
-        if (wide) k_step_a<true, kWide><<<blocks, kStepThreads, 0, s>>>(p, mode);
-        else k_step_a<true, 10><<<blocks, kStepThreads, 0, s>>>(p, mode);
-        if (p.n_rep > kInlineReps) k_step_fin<true><<<fin_blocks, 256, 0, s>>>(p, mode);
+    const bool full = wide && (mode & STEP_KICK_DRIFT) && (mode & STEP_CR) && p.charge_mode != kChargeTable && p.rate_tab;
+    const bool fin = wide || p.n_rep > kInlineReps;
+    const bool cond = (mode & STEP_SETCOND) != 0;
+    if (full) {
+        k_rates<<<(p.n_rep * p.n_ts * 2 + 127) / 128, 128, 0, s>>>(p);
+        k_step_wide<<<(p.n_atoms + kWideAtoms - 1) / kWideAtoms, kWideAtoms, 0, s>>>(p);
+    } else if (wide) {
+        k_step_a<false, kWide, true><<<blocks, kStepThreads, 0, s>>>(p, mode);
+    } else if (fin) {
+        k_step_a<false, 10, true><<<blocks, kStepThreads, 0, s>>>(p, mode);
+    } else if (cond) {
+        k_step_a<true, 10, false><<<blocks, kStepThreads, 0, s>>>(p, mode);
     } else {
-        if (wide) k_step_a<false, kWide><<<blocks, kStepThreads, 0, s>>>(p, mode);
-        else k_step_a<false, 10><<<blocks, kStepThreads, 0, s>>>(p, mode);
-        if (p.n_rep > kInlineReps) k_step_fin<false><<<fin_blocks, 256, 0, s>>>(p, mode);
+        k_step_a<false, 10, false><<<blocks, kStepThreads, 0, s>>>(p, mode);
+    }
+    if (fin) {
+        if (cond) k_step_fin<true><<<fin_blocks, 256, 0, s>>>(p, mode);
+        else k_step_fin<false><<<fin_blocks, 256, 0, s>>>(p, mode);
     }
 }
 
