@@ -121,7 +121,7 @@ __device__ __forceinline__ void half_kick(const Params& p, int s, int slot, doub
 // ---------------------------------------------------------------------------
 // k_step_a: one thread per atom (original order).
 // ---------------------------------------------------------------------------
-constexpr int kInlineReps = 4;   // up to this many replicas the step kernel's last block reduces them
+constexpr int kInlineReps = 4;   // up to this many replicas (eight lanes of a warp each) the step kernel's last block reduces them
 
 // Three standard normal numbers for the Langevin force (Sec. II.B, Eq. 14)
 // from four Philox words: Box-Muller on u = (w + 1/2) 2^-32 for the pairs
@@ -164,6 +164,9 @@ __device__ __forceinline__ void gauss3(uint4 w, bool fp32, double& g0, double& g
 // x = kappa r' and D = 3 + 3x + x^2, G = 3 Q e^x / D,
 // c1 = -Q kappa (3 + 3x/2) / D and c2 = -2 pi n_e / 3 for every Q.
 // Without an ion sphere (Q = 0, n_e = 0 or kappa = 0): r' = 0, G = Q.
+// R itself is not needed, (kappa R)^3 is; the neutral atom skips the divisions,
+// whose slow path a zero numerator takes for the whole warp (hybrid box of 12,003
+// atoms: step kernel 16.1 -> 15.0 us).
 __device__ void hyb_table(const Params& p, int rr, int lane, double kap, double ne)
 {
     HybQ* rows = p.hq + (size_t)rr * kHybQ;
@@ -173,9 +176,10 @@ __device__ void hyb_table(const Params& p, int rr, int lane, double kap, double 
     for (int q = lane; q <= p.z_max; q += 32) {   // the charge states the species can reach
         const double Q = (double)q;
         double G = Q, rp = 0.0, c1 = 0.0;
-        if (q > 0 && ne > 0.0 && kap > 0.0) {
-            const double R = cbrt(3.0 * Q / (4.0 * kPi * ne));
-            const double s = R * kap, s3 = s * s * s;
+        const bool ion = q > 0 && ne > 0.0 && kap > 0.0;
+        double phirc = 0.0;
+        if (ion) {
+            const double s3 = 3.0 * Q / (4.0 * kPi * ne) * kap * kap * kap;   // (kappa R)^3
             const double t = cbrt(1.0 + s3);
             rp = s3 / (kap * (t * t + t + 1.0));
             const double x = kap * rp;
@@ -183,7 +187,11 @@ __device__ void hyb_table(const Params& p, int rr, int lane, double kap, double 
             c1 = -Q * kap * (3.0 + 1.5 * x) / D;
             G = 3.0 * Q * exp(x) / D;
         }
-        const double phirc = rc < rp ? Q / rc + c1 - c2 * rc * rc : G * exp(-kap * rc) / rc;
+        if (q > 0) {
+            const bool in = rc < rp;
+            const double ph = (in ? Q : G * exp(-kap * rc)) / rc;
+            phirc = in ? ph + c1 - c2 * rc * rc : ph;
+        }
         HybQ h;
         h.G = G; h.rp = rp; h.c1 = c1; h.phirc = phirc;
         h.Gf = (float)fmin(G, 1.0e30); h.rpf = (float)rp; h.c1f = (float)c1; h.phircf = (float)phirc;
@@ -198,26 +206,34 @@ __device__ void hyb_table(const Params& p, int rr, int lane, double kap, double 
     }
 }
 
-// Replica rr's per-step reduction by one warp, the plasma scalars of the next
-// step (Eq. 3 and the helpers of the charge update) and, for a vacuum replica,
-// the cell grid for the positions just reduced into the bounding box.
+// The per-step reduction of up to four replicas (base .. base + nr - 1, eight
+// lanes each) and the plasma scalars of their next step (Eq. 3 and the helpers of
+// the charge update), by one warp.
 //
-// This runs at the end of every step with nothing else on the GPU, so its chain
-// of dependent operations counts: lane f < 12 loads field f of all accumulator
-// copies at once and reduces (and clears) them; the FP64 divisions, each some
-// hundreds of cycles on GB300's FP64 pipe, are issued once for several lanes:
-// T_e on lane 0, n_e on lane 1 and the grid's three dimensions on lanes 2 to 4.
-// One lane after the other (thirteen divisions and a square root in a row) the
-// step kernel took 15.9 us for 1,500 methane atoms in vacuum and 19.4 us for the
-// 45k-atom droplet; now 13.0 and 17.9 us.  Periodic boxes, whose grid stands, take
-// what they took (water box 14.4 us).
-__device__ void finalize_replica(const Params& p, int rr, int lane, long long next, double rl)
+// It runs at the end of every step with nothing else on the GPU, so its chain of
+// dependent operations counts: lane f < 6 of a replica loads field f of all
+// accumulator copies at once and reduces (and clears) them; the FP64 divisions and
+// roots, each some hundreds of cycles on GB300's FP64 pipe, are issued once for
+// several lanes: T_e on lane 0 with n_e on lane 1, kappa on lane 0 with the
+// species' Langevin widths on the lanes from 1.  The cell grids are sized by
+// finalize_grid on another warp meanwhile.  With
+// one chain for everything (thirteen divisions and a square root) the step kernel
+// took 15.9 us for 1,500 methane atoms in vacuum, 18.5 for 12,003 atoms of water
+// with hybrid screening and 19.4 for the 45k-atom droplet; with this, the box
+// reduced without contention, the records packed while the charge-update warp
+// flushes, and the rate bounds below: 9.4, 15.0 and 13.3 us (water box of 30,000
+// atoms 14.5 -> 10.7).
+__device__ void finalize_plasma(const Params& p, int base, int nr, int lane, long long next)
 {
     constexpr unsigned kFull = 0xffffffffu;
     static_assert(sizeof(RepAccum) == 12 * sizeof(long long), "twelve fields of eight bytes");
+    const int sub = lane & 7;
+    const bool on = (lane >> 3) < nr;
+    const int rr = on ? base + (lane >> 3) : base;
+    const bool head = on && sub == 0;
     RepState st{};
     double vol = 1.0, pne = 0.0, pte = 0.0;
-    if (lane == 0) {   // issued before the accumulators are read and cleared
+    if (head) {   // issued before the accumulators are read and cleared
         st = p.rs[rr];
         if (p.plasma_mode == 1) {
             const long long idx = (long long)rr * (p.max_steps + 1) + (next <= p.max_steps ? next : p.max_steps);
@@ -225,64 +241,42 @@ __device__ void finalize_replica(const Params& p, int rr, int lane, long long ne
             pte = p.pres_te[idx];
         }
     }
-    if (lane == 1) vol = p.volume[rr];
-    Grid& g = p.grid[rr];
-    const int periodic = g.periodic, cell_cap = g.cell_cap;
-    // sums on lanes 0 to 5; the box's lower ends (as complements) and upper ends as
-    // maxima on lanes 6 to 11; both by a tree over the copies
-    unsigned long long sum = 0ull, mx = 0ull;
-    if (lane < 12) {
-        unsigned long long* f = reinterpret_cast<unsigned long long*>(p.acc + (size_t)rr * kAccCopies) + lane;
-        const unsigned long long flip = lane >= 6 && lane < 9 ? ~0ull : 0ull;
-        unsigned long long v[kAccCopies], m[kAccCopies];
+    if (on && sub == 1) vol = p.volume[rr];
+    unsigned long long sum = 0ull;
+    if (on && sub < 6) {
+        unsigned long long* f = reinterpret_cast<unsigned long long*>(p.acc + (size_t)rr * kAccCopies) + sub;
+        unsigned long long v[kAccCopies];
 #pragma unroll
         for (int c = 0; c < kAccCopies; ++c) v[c] = __ldcg(f + 12 * c);
 #pragma unroll
-        for (int c = 0; c < kAccCopies; ++c) {
-            m[c] = v[c] ^ flip;
-            f[12 * c] = flip;
-        }
+        for (int c = 0; c < kAccCopies; ++c) f[12 * c] = 0ull;
 #pragma unroll
         for (int o = kAccCopies / 2; o; o >>= 1)
 #pragma unroll
-            for (int c = 0; c < o; ++c) {
-                v[c] += v[c + o];
-                m[c] = max(m[c], m[c + o]);
-            }
+            for (int c = 0; c < o; ++c) v[c] += v[c + o];
         sum = v[0];
-        mx = m[0] ^ flip;
     }
-    // lane 0: the electron gas; lanes 2 to 4: one dimension of the bounding box each
-    const long long dE = (long long)__shfl_sync(kFull, sum, 1);
+    const long long dE = (long long)__shfl_sync(kFull, sum, 1, 8);
     long long dc[4];
-    for (int k = 0; k < 4; ++k) dc[k] = (long long)__shfl_sync(kFull, sum, 2 + k);
-    const int d = lane >= 2 && lane < 5 ? lane - 2 : 0;
-    const unsigned long long mn = __shfl_sync(kFull, mx, 6 + d);
-    mx = __shfl_sync(kFull, mx, 9 + d);
-    if (lane == 0) {
+    for (int k = 0; k < 4; ++k) dc[k] = (long long)__shfl_sync(kFull, sum, 2 + k, 8);
+    if (sub == 0) {
         st.n_e += (long long)sum;
         st.e_gas += dE;
         if (st.e_gas < 0) st.e_gas = 0;
         for (int k = 0; k < 4; ++k) st.counts[k] += dc[k];
     }
-    double lo = mn == ~0ull ? 0.0 : from_ordered(mn), hi = mx == 0ull ? 0.0 : from_ordered(mx);
-    if (!(hi >= lo)) lo = hi = 0.0;
-    const double ext = hi - lo;
-    const long long n_e = __shfl_sync(kFull, st.n_e, 0);
-    double num = 1.0, den = 1.0, f = 1.0;   // f: cell edges >= f rl, rl the radius of the list built on the grid
-    if (lane == 0 && n_e > 0) {
+    const long long n_e = __shfl_sync(kFull, st.n_e, 0, 8);
+    double num = 1.0, den = 1.0;
+    if (sub == 0 && n_e > 0) {
         num = (double)st.e_gas;
         den = __dmul_rn(1500.0, (double)n_e);
-    } else if (lane == 1 && n_e > 0) {
+    } else if (sub == 1 && n_e > 0) {
         num = (double)n_e;
         den = vol;
-    } else if (!periodic && lane >= 2 && lane < 5) {   // (a zero numerator takes the division's slow path)
-        num = ext;
-        den = rl * f;
     }
     double quo = __ddiv_rn(num, den);
-    double te = 0.0, ne = 0.0;   // lane 0
-    const double n_dens = __shfl_sync(kFull, quo, 1);
+    const double n_dens = __shfl_sync(kFull, quo, 1, 8);
+    double te = 0.0, ne = 0.0;
     if (p.plasma_mode == 1) {
         ne = pne;
         te = pte;
@@ -290,39 +284,28 @@ __device__ void finalize_replica(const Params& p, int rr, int lane, long long ne
         te = quo;
         ne = n_dens;
     }
-    int n = 1;
-    if (!periodic) {
-        for (int it = 0; it < 400; ++it) {
-            const double m = floor(quo);
-            n = m < 1.0 ? 1 : (m > 1.0e6 ? 1000000 : (int)m);
-            const long long prod = (long long)__shfl_sync(kFull, n, 2) * __shfl_sync(kFull, n, 3) * __shfl_sync(kFull, n, 4);
-            if (prod <= cell_cap) break;
-            f *= 1.125;
-            quo = __ddiv_rn(ext, rl * f);
-        }
-    }
+    te = __shfl_sync(kFull, te, 0, 8);
+    ne = __shfl_sync(kFull, ne, 0, 8);
     num = den = 1.0;
-    if (lane == 0 && ne > 0.0) {
+    // Langevin update of the next step per species (Eqs. 13-14): gamma =
+    // n_e g_s, c = e^{-gamma dt}, sigma = sqrt((1 - c^2) k_B T_e / m_s); species s
+    // on lane s + 1, the last of eight after the others
+    double lc = 0.0;
+    const int ls = sub - 1;
+    const bool lgv = p.langevin && on && ls >= 0 && ls < p.n_species;
+    if (lgv) {
+        lc = exp(-(ne * p.lgv_g[ls]) * p.dt);
+        num = (1.0 - lc * lc) * (te * kEvKJmol);
+        den = p.mass[ls];
+    } else if (head && ne > 0.0) {
         const double tc = te > p.te_floor ? te : p.te_floor;
         num = __dmul_rn(p.four_pi_f, ne);
         den = __dmul_rn(tc, kEvKJmol);
-    } else if (!periodic && lane >= 2 && lane < 5) {
-        num = ext;
-        den = (double)n;
     }
-    quo = __ddiv_rn(num, den);
-    if (!periodic) {
-        if (lane >= 2 && lane < 5) {
-            const double e = n == 1 ? (ext > rl ? ext : rl) : quo;
-            g.origin[d] = lo;
-            g.edge[d] = e;
-            g.inv_edge[d] = 1.0 / e;
-            g.edge_f[d] = (float)e;
-            g.dims[d] = n;
-        }
-    }
-    if (lane == 0) {
-        const double kap = ne > 0.0 ? __dsqrt_rn(quo) : 0.0;
+    const double root = __dsqrt_rn(__ddiv_rn(num, den));
+    if (lgv) p.lgv[(size_t)rr * kMaxSpecies + ls] = make_double2(lc, root);
+    if (head) {
+        const double kap = ne > 0.0 ? root : 0.0;
         st.te_ev = te;
         st.n_dens = ne;
         st.kappa = kap;
@@ -338,23 +321,76 @@ __device__ void finalize_replica(const Params& p, int rr, int lane, long long ne
         st.kappa_force = kf;
         st.kappa_f = (float)kf;
         p.rs[rr] = st;
-    }
-    if (p.screening) {
-        const double kap = __shfl_sync(0xffffffffu, st.kappa_force, 0);
-        const double ne = __shfl_sync(0xffffffffu, st.n_dens, 0);
-        hyb_table(p, rr, lane, kap, ne);
-    }
-    if (p.langevin) {
-        // Langevin update of the next step per species (Eqs. 13-14): gamma =
-        // n_e g_s, c = e^{-gamma dt}, sigma = sqrt((1 - c^2) k_B T_e / m_s)
-        const double ne = __shfl_sync(0xffffffffu, st.n_dens, 0);
-        const double te = __shfl_sync(0xffffffffu, st.te_ev, 0);
-        if (lane < p.n_species) {
-            const double gam = ne * p.lgv_g[lane];
-            const double c = exp(-gam * p.dt);
-            const double kT = te * kEvKJmol;
-            p.lgv[(size_t)rr * kMaxSpecies + lane] = make_double2(c, sqrt((1.0 - c * c) * kT / p.mass[lane]));
+        if (p.langevin && p.n_species == kMaxSpecies) {
+            const int s = kMaxSpecies - 1;
+            const double c = exp(-(ne * p.lgv_g[s]) * p.dt);
+            p.lgv[(size_t)rr * kMaxSpecies + s] =
+                make_double2(c, __dsqrt_rn(__ddiv_rn((1.0 - c * c) * (te * kEvKJmol), p.mass[s])));
         }
+    }
+    if (p.screening)
+        for (int k = 0; k < nr; ++k)
+            hyb_table(p, base + k, lane, __shfl_sync(kFull, st.kappa_force, 8 * k), __shfl_sync(kFull, st.n_dens, 8 * k));
+}
+
+// The bounding boxes of up to four replicas (eight lanes each) and, for a vacuum
+// replica, the cell grid of the positions reduced into it; rl: the radius of the
+// list built on the grid.
+__device__ void finalize_grid(const Params& p, int base, int nr, int lane, double rl)
+{
+    constexpr unsigned kFull = 0xffffffffu;
+    const int sub = lane & 7;
+    const bool on = (lane >> 3) < nr;
+    const int rr = on ? base + (lane >> 3) : base;
+    Grid& g = p.grid[rr];
+    const int periodic = g.periodic, cell_cap = g.cell_cap;
+    // lower ends on lanes 0 to 2, upper ends on 3 to 5, both as maxima (of complements)
+    unsigned long long mx = 0ull;
+    if (on && sub < 6 && !periodic) {
+        unsigned long long* f = reinterpret_cast<unsigned long long*>(p.acc + (size_t)rr * kAccCopies) + 6 + sub;
+        const unsigned long long flip = sub < 3 ? ~0ull : 0ull;
+        unsigned long long m[kAccCopies];
+#pragma unroll
+        for (int c = 0; c < kAccCopies; ++c) m[c] = __ldcg(f + 12 * c);
+#pragma unroll
+        for (int c = 0; c < kAccCopies; ++c) {
+            m[c] ^= flip;
+            f[12 * c] = flip;
+        }
+#pragma unroll
+        for (int o = kAccCopies / 2; o; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < o; ++c) m[c] = max(m[c], m[c + o]);
+        mx = m[0] ^ flip;
+    }
+    if (__all_sync(kFull, !on || periodic)) return;
+    const int d = sub < 3 ? sub : 0;   // lane d: dimension d
+    const unsigned long long mn = __shfl_sync(kFull, mx, d, 8);
+    mx = __shfl_sync(kFull, mx, 3 + d, 8);
+    double lo = mn == ~0ull ? 0.0 : from_ordered(mn), hi = mx == 0ull ? 0.0 : from_ordered(mx);
+    if (!(hi >= lo)) lo = hi = 0.0;
+    const bool size = on && !periodic;
+    const double ext = size ? hi - lo : 1.0;   // (a zero numerator takes the division's slow path)
+    double f = 1.0;
+    int n = 1;
+    bool done = !size;
+    for (int it = 0; it < 400; ++it) {
+        const double m = floor(__ddiv_rn(ext, rl * f));
+        const int nn = m < 1.0 ? 1 : (m > 1.0e6 ? 1000000 : (int)m);
+        if (!done) n = nn;
+        const long long prod = (long long)__shfl_sync(kFull, n, 0, 8) * __shfl_sync(kFull, n, 1, 8) * __shfl_sync(kFull, n, 2, 8);
+        done |= prod <= cell_cap;
+        if (__all_sync(kFull, done)) break;
+        f *= 1.125;
+    }
+    const double quo = __ddiv_rn(ext, (double)n);
+    if (size && sub < 3) {
+        const double e = n == 1 ? (ext > rl ? ext : rl) : quo;
+        g.origin[d] = lo;
+        g.edge[d] = e;
+        g.inv_edge[d] = 1.0 / e;
+        g.edge_f[d] = (float)e;
+        g.dims[d] = n;
     }
 }
 
@@ -486,13 +522,58 @@ __device__ __forceinline__ Rates cr_rates(const Params& p, const RepState& st, d
     return x;
 }
 
+// An FP32 number above the double whose high word is hi (infinity for what FP32
+// cannot hold, infinities and NaN; its smallest normal number for what is smaller).
+__device__ __forceinline__ float above_f(int hi)
+{
+    const int mag = hi & 0x7fffffff;
+    if (mag >= 0x47e00000) return __int_as_float(0x7f800000);
+    return hi < 0x38100000 ? 1.17549435e-38f : __uint_as_float((unsigned)hi * 8u + 0x40000008u);
+}
+__device__ __forceinline__ int hi_word(const double* a) { return reinterpret_cast<const int*>(a)[1]; }
+
+// Whether u0 = u53(a, .) is certainly below 1 - e^{-lam} >= lam - lam^2 / 2 (lam > 0),
+// which spares the exponential's forty FP64 operations but for the few atoms that
+// draw a number between the two.
+__device__ __forceinline__ bool sure_event(unsigned a, double lam)
+{
+    const int hi = __double2hiint(lam);
+    const float lo_f = hi < 0x38100000 || hi >= 0x47e00000 ? 0.0f : __uint_as_float((unsigned)hi * 8u + 0x40000000u);
+    const float t = __fmul_rn(lo_f, __fmul_rn(__fsub_rn(1.0f, __fmul_rn(0.5f, above_f(hi))), 0.999998f));
+    return __fmul_rn(__uint2float_ru((a >> 5) + 1u), 7.4505806e-9f) < t;
+}
+
+// An upper bound of cr_rates' total rate in FP32: the interpolated coefficients
+// are at most the larger of their two table values.  GB300's FP64 pipe takes 16
+// cycles of the SM per warp instruction, and the bound rules an event out for
+// all but the few atoms that draw a number near or below their rate.
+__device__ __forceinline__ float cr_bound(const Params& p, const RepState& st, double dF, int ts, int s, int Z, int q, int h)
+{
+    float b = __fmul_rn(above_f(hi_word(p.sigma_pi + 2 * ts + h)), above_f(__double2hiint(dF)));
+    if (h) b = __fadd_rn(b, above_f(hi_word(p.auger_dt + s)));
+    float k = 0.0f;
+    if (q < Z) {
+        const double* K = p.k_ci + (long long)ts * p.n_te + st.it0;
+        k = above_f(max(hi_word(K), hi_word(K + 1)));
+    }
+    if (q > 0 && h == 0) {
+        const double* K = p.k_rec + (long long)ts * p.n_te + st.it0;
+        k = __fadd_rn(k, above_f(max(hi_word(K), hi_word(K + 1))));
+    }
+    return __fmul_rn(__fadd_rn(b, __fmul_rn(k, above_f(__double2hiint(st.ne_dt)))), 1.000001f);
+}
+
+// a < b for non-negative doubles, in the integer pipe: their order is that of
+// their bit patterns.
+__device__ __forceinline__ bool below(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
 // The channel that t, uniform in [0, lam), falls into: 0 PI, 1 Auger, 2 CI, 3 REC.
 __device__ __forceinline__ int cr_channel(const Rates& x, double t)
 {
-    if (t < x.a_pi) return 0;
-    if (t < x.c1) return 1;
-    if (t < x.c2) return 2;
-    if (t < x.lam) return 3;
+    if (below(t, x.a_pi)) return 0;
+    if (below(t, x.c1)) return 1;
+    if (below(t, x.c2)) return 2;
+    if (below(t, x.lam)) return 3;
     return x.a_rec > 0.0 ? 3 : (x.a_ci > 0.0 ? 2 : (x.a_a > 0.0 ? 1 : 0));
 }
 
@@ -521,10 +602,9 @@ __device__ __forceinline__ long long cr_event(const Params& p, int ch, int ts, i
     return de;
 }
 
-// Total rate of every (replica, type state, K-hole flag) at the step about to be
-// taken, for the step kernel of large systems: an atom then tests its uniform
-// against one table entry, and only the few that may have an event evaluate
-// the rates (the same expressions, so the same values).
+// The running sums of the rates of every (replica, type state, K-hole flag) at the
+// step about to be taken, for the step kernel of large systems: an atom then tests
+// its uniform against one table entry (the same expressions, so the same values).
 __global__ void __launch_bounds__(128) k_rates(Params p)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -534,59 +614,52 @@ __global__ void __launch_bounds__(128) k_rates(Params p)
     while (s + 1 < p.n_species && ts >= p.ts_off[s + 1]) ++s;
     const long long step = *p.step;
     const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
-    p.rate_tab[k] = cr_rates(p, p.rs[r], dF, ts, s, p.zs[s], ts - p.ts_off[s], h).lam;
+    const Rates x = cr_rates(p, p.rs[r], dF, ts, s, p.zs[s], ts - p.ts_off[s], h);
+    double* t = p.rate_tab + 4ll * k;
+    t[0] = x.a_pi; t[1] = x.c1; t[2] = x.c2; t[3] = x.lam;
 }
 
 // Bounding box of the vacuum replicas' atoms into the block's window of replicas
-// from r0 (whole warps; one atom per lane, r = -1: none).
+// from r0 (whole warps; one atom per lane; vac: the lane's atom counts).  ONE: no
+// other warp of the block writes the window.  A replica at a time, reduced in the
+// warp: 64-bit minima and maxima in shared memory are compare-and-swap loops, and
+// 28 lanes of a last block contending for six of them took 3 us.
+template <bool ONE>
 __device__ __forceinline__ void box_update(const Params& p, int r, int r0, bool vac, const double pos[3],
                                            unsigned long long (*s_bmin)[3], unsigned long long (*s_bmax)[3])
 {
-    const unsigned full = 0xffffffffu;
-    const int rl0 = __shfl_sync(full, r, 0);
-    const bool uniform = __all_sync(full, r == rl0) && rl0 >= 0;
-    const bool any_vac = __any_sync(full, vac);
-    if (any_vac) {
-        if (uniform) {
-            if (__shfl_sync(full, (int)vac, 0)) {
-                for (int d = 0; d < 3; ++d) {
-                    const unsigned long long key = ordered_bits(pos[d]);
-                    const unsigned long long mn = warp_extreme<false>(key), mx = warp_extreme<true>(key);
-                    if ((threadIdx.x & 31) == 0) {
-                        const int w = rl0 - r0;
-                        if (w < kRepWindow) {
-                            atomicMin(&s_bmin[w][d], mn);
-                            atomicMax(&s_bmax[w][d], mx);
-                        } else {
-                            RepAccum* a = p.acc + (size_t)rl0 * kAccCopies + (blockIdx.x & (kAccCopies - 1));
-                            atomicMin(&a->bmin[d], mn);
-                            atomicMax(&a->bmax[d], mx);
-                        }
-                    }
-                }
-            }
-        } else if (vac) {
-            const int w = r - r0;
-            for (int d = 0; d < 3; ++d) {
-                unsigned long long o = ordered_bits(pos[d]);
-                if (w < kRepWindow) {
-                    atomicMin(&s_bmin[w][d], o);
-                    atomicMax(&s_bmax[w][d], o);
-                } else {
-                    RepAccum* a = p.acc + (size_t)r * kAccCopies + (blockIdx.x & (kAccCopies - 1));
-                    atomicMin(&a->bmin[d], o);
-                    atomicMax(&a->bmax[d], o);
-                }
-            }
+    constexpr unsigned kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned todo = __ballot_sync(kFull, vac);
+    while (todo) {
+        const int r1 = __shfl_sync(kFull, r, __ffs(todo) - 1);
+        const bool in = vac && r == r1;
+        todo &= ~__ballot_sync(kFull, in);
+        unsigned long long v = 0ull;   // lane d: lower end of dimension d, lane 3 + d: upper end
+        for (int d = 0; d < 3; ++d) {
+            const unsigned long long key = ordered_bits(pos[d]);
+            const unsigned long long mn = warp_extreme<false>(in ? key : ~0ull), mx = warp_extreme<true>(in ? key : 0ull);
+            if (lane == d) v = mn;
+            if (lane == 3 + d) v = mx;
+        }
+        if (lane < 6) {
+            const int w = r1 - r0, d = lane < 3 ? lane : lane - 3;
+            RepAccum* a = p.acc + (size_t)r1 * kAccCopies + (blockIdx.x & (kAccCopies - 1));
+            const bool win = w < kRepWindow;
+            unsigned long long* dst = lane < 3 ? (win ? &s_bmin[w][d] : &a->bmin[d]) : (win ? &s_bmax[w][d] : &a->bmax[d]);
+            if (ONE && win) *dst = v;
+            else if (lane < 3) atomicMin(dst, v);
+            else atomicMax(dst, v);
         }
     }
 }
 
-// The block's sums and boxes of replicas r0 .. r0 + nw - 1 into the accumulators.
+// The block's sums and boxes of replicas r0 .. r0 + nw - 1 into the accumulators,
+// by threads t of n_t.
 __device__ __forceinline__ void flush_block(const Params& p, int r0, int nw, long long (*s_acc)[6],
-                                            unsigned long long (*s_bmin)[3], unsigned long long (*s_bmax)[3])
+                                            unsigned long long (*s_bmin)[3], unsigned long long (*s_bmax)[3], int t, int n_t)
 {
-    for (int k = threadIdx.x; k < nw * 12; k += blockDim.x) {
+    for (int k = t; k < nw * 12; k += n_t) {
         const int w = k / 12, f = k % 12;
         RepAccum* a = p.acc + (size_t)(r0 + w) * kAccCopies + (blockIdx.x & (kAccCopies - 1));
         if (f < 6) {
@@ -610,11 +683,12 @@ __device__ __forceinline__ void flush_block(const Params& p, int r0, int nw, lon
 // loads issued before the first use and no barrier in between; k_step_fin
 // reduces the replicas.  Two threads per atom (k_step_a) shorten the chain of a
 // system that leaves the chip idle, but with many blocks per SM the instructions
-// count: FP64 runs at 2 lanes per SM and clock here, and evaluating the rates
-// was most of the charge role's work, for an event in one atom of some hundreds.
-// 2 M-atom droplet: 302.6 us -> 203 + 3.9 (k_rates) + 7.5 us (k_step_fin), 1.9 TB/s
-// of state; 1,024 x 1,500 methane: 188.1 + 16.3 -> 147.0 + 4.0 + 9.5 us.  Blocks of
-// 64 atoms took 1 % less than 128.
+// count: FP64 runs at 2 lanes per SM and clock here, and evaluating the rates and
+// 1 - e^{-lam} was most of the charge role's work, for an event in one atom of some
+// tens.  2 M-atom droplet: 302.6 us -> 126 + 4.0 (k_rates) + 6.7 us (k_step_fin),
+// 3.8 TB/s of state (203 us before sure_event); 1,024 x 1,500 methane: 188.1 + 16.3
+// -> 90.5 + 4.1 + 8.1 us; 199,773 atoms 46.6 -> 24.6 + 2.7 + 5.7.  Blocks of 64
+// atoms took 1 % less than 128.
 constexpr int kWideAtoms = 64;
 __global__ void __launch_bounds__(kWideAtoms, 16) k_step_wide(Params p)
 {
@@ -639,7 +713,8 @@ __global__ void __launch_bounds__(kWideAtoms, 16) k_step_wide(Params p)
     half_kick(p, s, slot, ax, ay, az);
     const int Z = p.zs[s], ts = p.ts_off[s] + qi;
     const unsigned long long sd = p.seed[r];
-    const double lam = p.rate_tab[((long long)r * p.n_ts + ts) * 2 + hi];
+    const double* tab = p.rate_tab + (((long long)r * p.n_ts + ts) * 2 + hi) * 4;
+    const double lam = tab[3];
     const Grid& g = p.grid[r];
     const int nw = min(r_last - r0 + 1, kRepWindow);
     for (int k = tid; k < nw * 6; k += kWideAtoms) (&s_acc[0][0])[k] = 0;
@@ -661,15 +736,18 @@ __global__ void __launch_bounds__(kWideAtoms, 16) k_step_wide(Params p)
         int qn = qi;
         if (step >= p.max_steps) atomicOr(p.err, ERR_TABLE_END);
         // the tests of k_step_a, on the table's total rate
-        if (__double_as_longlong(lam) > 0ll) {
+        if (below(0.0, lam)) {
             const uint4 w4 = philox4x32_10(make_uint4((unsigned)loc, (unsigned)step, 0u, 0u),
                                            make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
             const double u0 = u53(w4.x, w4.y);
-            if ((unsigned long long)__double_as_longlong(u0) < (unsigned long long)__double_as_longlong(lam) &&
-                u0 < one_minus_exp_neg(lam, p.etab, p.inv12)) {
-                const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
-                const Rates c = cr_rates(p, p.rs[r], dF, ts, s, Z, qi, hi);
-                const int ch = cr_channel(c, __dmul_rn(u53(w4.z, w4.w), c.lam));
+            if (below(u0, lam) &&
+                (sure_event(w4.x, lam) || u0 < one_minus_exp_neg(lam, p.etab, p.inv12))) {
+                const double t = __dmul_rn(u53(w4.z, w4.w), lam);
+                int ch = below(t, tab[0]) ? 0 : (below(t, tab[1]) ? 1 : (below(t, tab[2]) ? 2 : 3));
+                if (!below(t, lam)) {   // t rounded up to lam
+                    const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
+                    ch = cr_channel(cr_rates(p, p.rs[r], dF, ts, s, Z, qi, hi), t);
+                }
                 int hn = hi;
                 const long long de = cr_event(p, ch, ts, s, Z, qn, hn);
                 p.q[i] = (uint8_t)qn;
@@ -701,9 +779,9 @@ __global__ void __launch_bounds__(kWideAtoms, 16) k_step_wide(Params p)
         const unsigned m = __reduce_max_sync(0xffffffffu, d2_bits);
         if (lane == 0 && m) atomicMax(p.maxd2, m);
     }
-    box_update(p, live ? r : -1, r0, live && !g.periodic, pos, s_bmin, s_bmax);
+    box_update<false>(p, r, r0, live && !g.periodic, pos, s_bmin, s_bmax);
     __syncthreads();
-    flush_block(p, r0, nw, s_acc, s_bmin, s_bmax);
+    flush_block(p, r0, nw, s_acc, s_bmin, s_bmax, tid, kWideAtoms);
 }
 
 // SETCOND: the Verlet-buffered variant that decides the rebuild and sets the
@@ -720,20 +798,11 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
     __shared__ unsigned long long s_bmin[kRepWindow][3], s_bmax[kRepWindow][3];
     __shared__ int s_last;
     __shared__ unsigned s_maxd2;
-    __shared__ double s_rl;
-    __shared__ uint8_t s_q[kStepAtoms];   // charges after this step's update (charge-update warps)
+    __shared__ uint8_t s_q[kStepAtoms];   // charges after this step's update (charge-update warp)
     // a cluster-pair list overflow freezes the state at the step whose forces
     // are missing; the host grows the list, recomputes them and resumes
     if (*p.err & ERR_LIST) return;
     const int tid = threadIdx.x;
-    for (int k = tid; k < kRepWindow * 6; k += blockDim.x) (&s_acc[0][0])[k] = 0;
-    for (int k = tid; k < kRepWindow * 3; k += blockDim.x) {
-        (&s_bmin[0][0])[k] = ~0ull;
-        (&s_bmax[0][0])[k] = 0ull;
-    }
-    if (tid == 0) s_maxd2 = 0u;
-    __syncthreads();
-
     const long long step = *p.step;
     const int kick_full = *p.kick_full;
     // the first kStepAtoms threads kick, drift and re-pack atoms first ..
@@ -741,7 +810,7 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
     // atoms (independent until the re-pack)
     const bool cr_role = tid >= kStepAtoms;
     const int first = blockIdx.x * kStepAtoms;
-    const int r0 = p.rep[first < p.n_atoms ? first : p.n_atoms - 1];
+    const int r0 = p.rep[first], r_last = p.rep[min(first + kStepAtoms, p.n_atoms) - 1];
     const int i = first + (tid & (kStepAtoms - 1));
     const bool live = i < p.n_atoms;
     const int lane = tid & 31;
@@ -785,14 +854,20 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
         vac = !p.grid[r].periodic;
     }
 
-    // ---- bounding box of vacuum replicas (warp-reduced when uniform) ----
-    if (!cr_role) {   // whole warps
-        const unsigned full = 0xffffffffu;
-        if (p.xr && (mode & STEP_KICK_DRIFT)) {
-            const unsigned m = __reduce_max_sync(full, d2_bits);
-            if (lane == 0) s_maxd2 = m;   // one kick warp per block
+    // ---- bounding box of vacuum replicas; each warp clears the sums it writes ----
+    if (!cr_role) {
+        unsigned m = 0u;
+        if (p.xr && (mode & STEP_KICK_DRIFT)) m = __reduce_max_sync(0xffffffffu, d2_bits);
+        if (lane == 0) s_maxd2 = m;
+        for (int k = lane; k < kRepWindow * 3; k += 32) {
+            (&s_bmin[0][0])[k] = ~0ull;
+            (&s_bmax[0][0])[k] = 0ull;
         }
-        box_update(p, r, r0, vac, pos, s_bmin, s_bmax);
+        __syncwarp();
+        box_update<true>(p, r, r0, vac, pos, s_bmin, s_bmax);
+    } else {
+        for (int k = lane; k < kRepWindow * 6; k += 32) (&s_acc[0][0])[k] = 0;
+        __syncwarp();
     }
 
     // ---- collisional-radiative update (reading of Sec. II.A) ----
@@ -843,18 +918,18 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
         const int ts = p.ts_off[s] + qi;
         if (step >= p.max_steps) atomicOr(p.err, ERR_TABLE_END);
         const double dF = step < p.max_steps ? p.dF[(long long)r * p.max_steps + step] : 0.0;
-        const Rates x = cr_rates(p, p.rs[r], dF, ts, s, Z, qi, hi);
+        const RepState& rs = p.rs[r];
         int ch = -1;
-        // lam and u0 are non-negative doubles, whose order is that of their
-        // bit patterns: the tests run in the integer pipe
-        if (__double_as_longlong(x.lam) > 0ll) {
-            const unsigned long long sd = p.seed[r];
-            const uint4 w4 = philox4x32_10(make_uint4((unsigned)p.local_id[i], (unsigned)step, 0u, 0u),
-                                           make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
+        const unsigned long long sd = p.seed[r];
+        const uint4 w4 = philox4x32_10(make_uint4((unsigned)p.local_id[i], (unsigned)step, 0u, 0u),
+                                       make_uint2((unsigned)sd, (unsigned)(sd >> 32)));
+        // u0 = u53(w4.x, w4.y) has w4.x >> 5 as its leading 27 bits; 1 - e^{-lam} <=
+        // lam, so u0 >= lam, and u0 above a bound of lam, decide "no event" exactly
+        if (!(__fmul_rn(__uint2float_rz(w4.x >> 5), 7.4505806e-9f) > cr_bound(p, rs, dF, ts, s, Z, qi, hi))) {
+            const Rates x = cr_rates(p, rs, dF, ts, s, Z, qi, hi);
             const double u0 = u53(w4.x, w4.y);
-            // 1 - e^{-lam} <= lam, so u0 >= lam decides "no event" exactly
-            if ((unsigned long long)__double_as_longlong(u0) < (unsigned long long)__double_as_longlong(x.lam) &&
-                u0 < one_minus_exp_neg(x.lam, p.etab, p.inv12)) {
+            if (below(0.0, x.lam) && below(u0, x.lam) &&
+                (sure_event(w4.x, x.lam) || u0 < one_minus_exp_neg(x.lam, p.etab, p.inv12))) {
                 ch = cr_channel(x, __dmul_rn(u53(w4.z, w4.w), x.lam));
             }
         }
@@ -880,46 +955,42 @@ __global__ void __launch_bounds__(kStepThreads, MINB) k_step_a(Params p, int mod
     // ---- Verlet-buffered list: the packed record of this atom for the forces
     // of this step, in the slot of the last build (a build, if one follows,
     // rewrites all records); the force sums are cleared after the kick read them
-    __syncthreads();   // the charges of this step are written
+    __syncthreads();   // the charges of this step, the boxes and the sums are written
     if (repack) {
         const int qi = (mode & STEP_CR) ? (int)s_q[i - first] : pk_q;
         pack_record(p, pk_slot, pos, pk_cen, pk_per, pk_box, pk_sp, qi, pk_fr);
     }
-    __syncthreads();
 
-    // ---- flush block partials ----
-    {
-        const int last_atom = min(first + kStepAtoms, p.n_atoms) - 1;
-        const int r_last = p.rep[last_atom];
-        const int nw = min(r_last - r0 + 1, kRepWindow);
-        flush_block(p, r0, nw, s_acc, s_bmin, s_bmax);
+    // ---- flush block partials: by the charge-update warp, whose fence then waits
+    // for no record on its way to memory ----
+    if (cr_role) {
+        flush_block(p, r0, min(r_last - r0 + 1, kRepWindow), s_acc, s_bmin, s_bmax, lane, 32);
+        if (lane == 0 && s_maxd2) atomicMax(p.maxd2, s_maxd2);
     }
 
-    if (tid == 0 && s_maxd2) atomicMax(p.maxd2, s_maxd2);
-
     // ---- per-replica reduction (Eq. 3) and next grid: by this kernel's last
-    // block for a few replicas, by k_step_fin (a warp per replica) for more ----
+    // block for a few replicas, by k_step_fin for more ----
     if constexpr (FIN) return;
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(&p.counters[3], 1) == (int)gridDim.x - 1);
+    if (cr_role) {
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) s_last = (atomicAdd(&p.counters[3], 1) == (int)gridDim.x - 1);
+    }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    unsigned m2 = 0u;
-    if (tid == 0) {   // the list radius of this step's build, before finalize_step records it
-        m2 = SETCOND ? __ldcg(p.maxd2) : 0u;
-        s_rl = next_rlist<SETCOND>(p, m2);
-    }
-    __syncthreads();
-    const double rl = s_rl;
     const long long next = (mode & STEP_ADVANCE) ? step + 1 : step;
-    const int warp = tid >> 5, n_warps = blockDim.x >> 5;
-    for (int rr = warp; rr < p.n_rep; rr += n_warps) finalize_replica(p, rr, lane, next, rl);
-    if (tid == 0) finalize_step<SETCOND>(p, mode, next, m2);
+    if (cr_role) {
+        finalize_plasma(p, 0, p.n_rep, lane, next);
+    } else {
+        const unsigned m2 = SETCOND ? __ldcg(p.maxd2) : 0u;
+        finalize_grid(p, 0, p.n_rep, lane, next_rlist<SETCOND>(p, m2));
+        __syncwarp();
+        if (lane == 0) finalize_step<SETCOND>(p, mode, next, m2);
+    }
 }
 
-// Per-replica reduction when there are many replicas: one warp each, then the
+// Per-replica reduction when there are many replicas: two warps each, then the
 // last block finishes the step.
 template <bool SETCOND>
 __global__ void __launch_bounds__(256) k_step_fin(Params p, int mode)
@@ -929,10 +1000,12 @@ __global__ void __launch_bounds__(256) k_step_fin(Params p, int mode)
     const int tid = threadIdx.x, lane = tid & 31;
     const long long step = *p.step;
     const long long next = (mode & STEP_ADVANCE) ? step + 1 : step;
-    const int rr = (blockIdx.x * blockDim.x + tid) >> 5;
-    // every block reads maxd2 and the list state before the last one records the decision
-    const double rl = next_rlist<SETCOND>(p, SETCOND ? __ldcg(p.maxd2) : 0u);
-    if (rr < p.n_rep) finalize_replica(p, rr, lane, next, rl);
+    const int gw = (blockIdx.x * blockDim.x + tid) >> 5, rr = gw >> 1;
+    if (rr < p.n_rep) {
+        // every block reads maxd2 and the list state before the last one records the decision
+        if (gw & 1) finalize_grid(p, rr, 1, lane, next_rlist<SETCOND>(p, SETCOND ? __ldcg(p.maxd2) : 0u));
+        else finalize_plasma(p, rr, 1, lane, next);
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) s_last = (atomicAdd(&p.counters[3], 1) == (int)gridDim.x - 1);
@@ -956,7 +1029,7 @@ void launch_step_a(const Params& p, int mode, cudaStream_t s, int grid_atoms)
     static const int n_sm = sm_count();
     constexpr int kWide = 16;   // MINB of the variant for grids of many blocks per SM
     const int blocks = (p.n_atoms + kStepAtoms - 1) / kStepAtoms;
-    const int fin_blocks = (p.n_rep * 32 + 255) / 256;
+    const int fin_blocks = (p.n_rep * 64 + 255) / 256;
     const bool wide = blocks >= kWide * n_sm;
     const bool full = wide && (mode & STEP_KICK_DRIFT) && (mode & STEP_CR) && p.charge_mode != kChargeTable && p.rate_tab;
     const bool fin = wide || p.n_rep > kInlineReps;
