@@ -824,9 +824,9 @@ __device__ __forceinline__ void bonded_prologue(const Params& p)
 // this one issues 1.28 G at 68 %, the FMA pipe 48 % busy.  Cluster masks evaluate 14 %
 // more pairs than per-atom queues did (33 against 38 % of the evaluations
 // within r_cut, water at a 0.12 nm skin), which the cheaper tiles more than
-// pay for.  Per launch, 500,001-atom droplet 851 -> 772 us, water box of
-// 30,000 atoms 68.6 -> 64.6, 1,500 atoms 22.0 -> 18.4; hybrid screening, 12,003
-// atoms, 46.4 -> 41.7.  96 registers (20 warps per SM): with 80 (24 warps) the
+// pay for.  Per launch, 500,001-atom droplet 851 -> 768 us, water box of
+// 30,000 atoms 68.9 -> 62.9, 1,500 atoms 19.0 -> 10.5; hybrid screening, 12,003
+// atoms, 46.2 -> 40.9.  96 registers (20 warps per SM): with 80 (24 warps) the
 // compiler recomputes and spills (963 us), with 128 (16 warps) too few warps
 // cover the latencies (947 us before the j sums moved to shared memory).
 // Two tiles per branch for more independent work: 852 us, the longer code is
@@ -976,13 +976,27 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
     int lane;
     asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
     WF& w = reinterpret_cast<WF*>(smem + tab)[warp];
+    // A warp's first chunk is its own index (neighbours in the list on different
+    // blocks), the rest come from the counter; its descriptor and entries are on
+    // their way while the block copies the LJ table.  With every warp's first
+    // chunk from the counter, 2,432 warps queued for one address, and the early
+    // ones took second chunks before the late ones had asked for a first: 1,500
+    // atoms 15.4 us against 10.5 now, 8,005 atoms (2,296 chunks) 21.8 against 15.4,
+    // 30,000 atoms 64.7 against 62.9.
+    const unsigned err = *p.err;
+    const int n_chunks = min(p.counters[7], p.chunk_cap);
+    const int n_warps = gridDim.x * (blockDim.x >> 5);
+    int item = warp * gridDim.x + blockIdx.x;
+    int4 ch = make_int4(0, 0, 0, 0);   // (first cluster, first entry, entries | clusters << 16, replica)
+    if (item < n_chunks) ch = p.pl_chunk[item];
     for (int k = threadIdx.x; k < nts * nts; k += blockDim.x) s_lj[k] = p.lj_f[k];
+    PairEntry e4 = make_uint4(0u, 0u, 0u, 0u);
+    if (!(err & (ERR_CELL | ERR_LIST)) && item < n_chunks && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
     __syncthreads();
-    if (*p.err & (ERR_CELL | ERR_LIST)) return;
+    if (err & (ERR_CELL | ERR_LIST)) return;
     bonded_prologue<false, ENERGY>(p);
 
     const int tx = lane & 7, ty = lane >> 3;
-    const int n_chunks = min(p.counters[7], p.chunk_cap);
     const int lj_addr = (int)__cvta_generic_to_shared(smem);
     // after the j-force reduction lane (tx, ty) holds component tx & 3 (3: none)
     // of j-atom 2 ty (tx < 4) or 2 ty + 1 (tx >= 4)
@@ -1010,18 +1024,9 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
     // The work items are fetched ahead: while a chunk is evaluated, the counter's
     // answer and the descriptor of the next one are on their way, and its entries
     // are asked for before the i forces of this one are summed.
-    int item = 0;
-    if (lane == 0) item = atomicAdd(&p.counters[2], 1);
-    item = __shfl_sync(kFull, item, 0);
-    int4 ch = make_int4(0, 0, 0, 0);
-    PairEntry e4 = make_uint4(0u, 0u, 0u, 0u);
-    if (item < n_chunks) {
-        ch = p.pl_chunk[item];          // (first cluster, first entry, entries | clusters << 16, replica)
-        if (lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
-    }
     while (item < n_chunks) {
-        int next = 0;
-        if (lane == 0) next = atomicAdd(&p.counters[2], 1);
+        int next = n_chunks;
+        if (n_chunks > n_warps && lane == 0) next = n_warps + atomicAdd(&p.counters[2], 1);
         const int fc = ch.x, ent0 = ch.y, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         const Grid& g = p.grid_b[rr];
         c.kap = p.rs[rr].kappa_f;
@@ -1804,7 +1809,7 @@ static size_t pair_smem(int n_ts, int warps)
 // Registers of the mixed-precision force kernel: 96 (20 warps per SM) where
 // chunks are plenty; 128 (16 warps, no recomputation) for the hybrid and the
 // energy instances, which spill otherwise, and for systems with too few chunks
-// to fill more warps: per launch 1,500 atoms 18.4 (96) and 15.6 us (128), 8,005
+// to fill more warps: per launch 1,500 atoms 18.4 (96) and 15.6 us (128; 10.5 since), 8,005
 // atoms in unbuffered lists 25.9 and 23.9, 30,000 atoms 64.6 and 65.0.
 constexpr int kFewChunksAtoms = 16384;
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
