@@ -1821,13 +1821,25 @@ static auto pair_kernel()
 
 constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
 
-// FP64 blocks of 8 warps leave 44 KB for the LJ table (53 type states; 38 with
-// hybrid screening); with more states two blocks of 4 warps take their place.
-// The launch shape changes no result.
-template <bool FP64, bool HYB>
+// Warps of the blocks that a launch shape of `warps` per block is launched with,
+// given the block's own LJ table; the shape changes no result.
+//   FP64: blocks of 8 warps leave 44 KB for the table (53 type states; 38 with
+//   hybrid screening); with more states two blocks of 4 warps take their place.
+//   Mixed, 96 registers: 20 warps fit an SM's registers, as five blocks of 4 while
+//   the five tables are small (up to 28 type states), then as two blocks of 10 (up
+//   to 47) or one of 20 (up to 67).  Protein crystal, 43 type states, 199,773
+//   atoms: 398.8 us with 16 warps, 363.4 with 20.
+template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int fit_warps(int warps, int n_ts)
 {
-    while (FP64 && warps > 4 && pair_smem<FP64, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
+    if (FP64) {
+        while (warps > 4 && pair_smem<FP64, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
+        return warps;
+    }
+    constexpr int kWarps96 = 20, kSmemSm = 228 * 1024, kSmemBlock = 1024;   // an SM's shared memory, and what a block takes besides its own
+    if (ENERGY || HYB || FEW || warps != 4) return warps;
+    for (int w : {4, 10, 20})
+        if (pair_smem<FP64, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
     return warps;
 }
 
@@ -1847,9 +1859,11 @@ template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static void launch_one(const Params& p, cudaStream_t s, int blocks, int warps)
 {
     set_smem_attr<FP64, ENERGY, HYB, FEW>();
-    const int fit = fit_warps<FP64, HYB>(warps, p.n_ts_lj);
-    blocks *= warps / fit;
-    warps = fit;
+    const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, p.n_ts_lj);
+    if (blocks * warps % fit == 0) {
+        blocks = blocks * warps / fit;
+        warps = fit;
+    }
     pair_kernel<FP64, ENERGY, HYB, FEW>()<<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
 }
 
@@ -1857,7 +1871,7 @@ template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int max_blocks(int warps, int n_ts)
 {
     set_smem_attr<FP64, ENERGY, HYB, FEW>();
-    const int fit = fit_warps<FP64, HYB>(warps, n_ts);
+    const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, n_ts);
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW>(), fit * 32,
                                                   pair_smem<FP64, HYB>(n_ts, fit));

@@ -1102,16 +1102,24 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
         if (c.pair_warps) {
             h->pair_warps = c.pair_warps;
         } else {
+            // (with the blocks per SM pinned, by the interface's limits, whose 8 or
+            // 12 warps a block decide which pins are accepted)
+            const bool pinned = c.pair_blocks_per_sm != 0;
+            auto most = [&](int w) {
+                return w * (pinned ? pair_pin_limit(fp64, c.screening != 0, w, h->NTS_LJ)
+                                   : pair_max_blocks_per_sm(fp64, false, c.screening != 0, w, h->NTS_LJ, h->N));
+            };
             h->pair_warps = 8;
-            int best = 8 * pair_max_blocks_per_sm(fp64, false, c.screening != 0, 8, h->NTS_LJ, h->N);
+            int best = most(8);
             for (int wpb : {4, 12}) {
                 if (fp64) break;
-                const int w = wpb * pair_max_blocks_per_sm(fp64, false, c.screening != 0, wpb, h->NTS_LJ, h->N);
+                if (pinned && wpb == 4) continue;
+                const int w = most(wpb);
                 if (w > best) { best = w; h->pair_warps = wpb; }
             }
         }
         const int maxb = std::max(1, pair_max_blocks_per_sm(fp64, false, c.screening != 0, h->pair_warps, h->NTS_LJ, h->N));
-        const int pin = std::max(maxb, pair_pin_limit(fp64, c.screening != 0, h->pair_warps, h->NTS_LJ));
+        const int pin = pair_pin_limit(fp64, c.screening != 0, h->pair_warps, h->NTS_LJ);
         if (c.pair_blocks_per_sm > pin)
             return fail(h, MD_ERR_INVALID_ARG, "pair_blocks_per_sm exceeds the " + std::to_string(pin) +
                                                    " blocks of " + std::to_string(h->pair_warps) +
