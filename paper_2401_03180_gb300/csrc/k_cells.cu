@@ -183,8 +183,10 @@ __device__ __forceinline__ void scan_cells_finish(const Params& p, int on, int o
     p.counters[1] = over ? 0 : op;
     p.counters[2] = 0;
     p.counters[4] = 0;   // cells too large for the one-warp sort
+    p.counters[5] = 0;
     p.counters[6] = 0;
     p.counters[7] = 0;
+    p.counters[8] = 0;
 }
 
 // The grid of this build stays with the list until the next build.

@@ -240,6 +240,25 @@ __device__ __forceinline__ void pair64(const double4_16a& xi, int row_off, int f
 // every warp of the grid busy, so that a system of many SCs stages each SC once
 // and a smaller one still spreads over the GPU.  Systems of few SCs take
 // k_list_fused below instead.
+constexpr int kListFusedScs = 8192;   // super-cluster capacities up to this build their list in one kernel (k_list_fused)
+// Whether the list of these parameters holds light chunks apart (k_list_fused, lists
+// that serve several steps).  The kernels that find them (LIGHT) cost large systems
+// and single calls more than they give: 500,001 atoms 768 us without, 786 with.
+constexpr int kLightScs = 8192;
+__host__ __forceinline__ bool has_light(const Params& p) { return p.sc_cap <= kLightScs && p.xr != nullptr; }
+// The list's chunks and how many of them are heavy.
+__device__ __forceinline__ int2 chunk_counts(const Params& p)
+{
+    const int n = min(p.counters[7], p.chunk_cap);
+    return make_int2(n, max(n - p.counters[5], 0));
+}
+// Where chunk `item` of the list is: the heavy ones from the start of the table, the
+// light ones (k_list_fused) from its end; -1 beyond the last.
+__device__ __forceinline__ int chunk_at(const Params& p, int item, int2 n)
+{
+    return item >= n.x ? -1 : (item < n.y ? item : p.chunk_cap - 1 - (item - n.y));
+}
+
 struct ListWarp {
     float4 lo[kSuperClusters], hi[kSuperClusters];   // the SC's i-cluster boxes (cell frame)
     int2 fr[kSuperClusters];                          // fragment range of each i-cluster
@@ -696,14 +715,27 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
 // SC once per part and pass, and on entries of j-clusters out of range is saved.
 // Count, scan and write against this kernel, per build: 8,005 atoms (unbuffered)
 // 20.1 -> 8.9 us, 12,297 atoms 23.6 -> 11.6, 30,000 atoms 31.9 -> 17.3.
-constexpr int kListFusedScs = 8192;
+//
+// ORDER (buffered lists of up to kLightScs): the chunks of fewer than kLightTiles
+// tiles (i-clusters in range of an entry, before trimming) go to the end of the chunk
+// table, from its last element down, and are taken last (chunk_at): a force kernel's
+// warps then end within a light chunk's time of one another instead of a heavy
+// chunk's (of 63 us for 30,000 atoms the warps idled 11 on average).  Per launch
+// 30,000 atoms 63.0 -> 60.0 us, 45,005 atoms 66.6 -> 63.2, 12,003 with hybrid
+// screening 41.1 -> 39.1, FP64 forces of 30,000 atoms 1,628 -> 1,550, for 0.5 us more
+// of list building; with 24, 40 and 48 tiles 30,000 atoms take 61, 60.8 and 61.2.  A
+// list used once does not pay for it: of the 1.0 us that 8,005 atoms gain per launch
+// a build at every step takes 0.6, and a single call on 12,297 atoms is 2 % slower.
+constexpr int kLightTiles = 32;
+constexpr int kTileChunks = 256;   // chunks of an SC whose tiles are counted; later ones count as heavy
 constexpr int kFound = 128;
+template <bool ORDER>
 __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_fused(Params p)
 {
     constexpr unsigned kFull = 0xffffffffu;
     __shared__ ListWarp w;
     __shared__ uint2 s_found[kListWarps][kFound];   // (j-cluster, half-shell index | i-cluster mask << 8)
-    __shared__ int s_cnt[kListWarps], s_e0, s_c0;
+    __shared__ int s_cnt[kListWarps], s_e0, s_c0, s_tiles[ORDER ? kTileChunks : 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (*p.err & ERR_CELL) return;
     const int n_sc = p.counters[0];
@@ -721,6 +753,8 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_fused(Params p)
             w.fr[threadIdx.x] = p.bb_frag[s.fc + threadIdx.x];
         }
         list_stage_atoms(p, w, s, threadIdx.x, blockDim.x);
+        if constexpr (ORDER)
+            for (int t = threadIdx.x; t < kTileChunks; t += blockDim.x) s_tiles[t] = 0;
         __syncthreads();
         const int i0 = (int)((long long)total * warp / kListWarps), i1 = (int)((long long)total * (warp + 1) / kListWarps);
         int cnt = 0;
@@ -733,7 +767,46 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_fused(Params p)
         }
         if (lane == 0) s_cnt[warp] = cnt;
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if constexpr (ORDER) {
+            int pre = 0, tot = 0;
+            bool counted = true;
+            for (int k = 0; k < kListWarps; ++k) {
+                if (k < warp) pre += s_cnt[k];
+                tot += s_cnt[k];
+                counted &= s_cnt[k] <= kFound;
+            }
+            for (int k = lane; k < min(cnt, kFound); k += 32) {   // the chunks' tiles
+                const int t = (pre + k) / kChunk;
+                if (t < kTileChunks) atomicAdd(&s_tiles[t], __popc(s_found[warp][k].y >> 8));
+            }
+            __syncthreads();
+            if (warp == 0) {   // the SC's entries and chunks: four reservations at once
+                const int nch = (tot + kChunk - 1) / kChunk;
+                auto light = [&](int t) { return counted && t < min(nch, kTileChunks) && s_tiles[t] < kLightTiles; };
+                int nl = 0;
+                for (int t = lane; t - lane < nch; t += 32) nl += __popc(__ballot_sync(kFull, light(t)));
+                const int slot = lane == 0 ? 6 : (lane == 1 ? 7 : (lane == 2 ? 8 : 5));
+                int got = 0;
+                if (lane < 4) got = atomicAdd(&p.counters[slot], lane == 0 ? tot : (lane == 1 ? nch : (lane == 2 ? nch - nl : nl)));
+                const int e0 = __shfl_sync(kFull, got, 0), c0 = __shfl_sync(kFull, got, 1);
+                int h0 = __shfl_sync(kFull, got, 2), l0 = __shfl_sync(kFull, got, 3);
+                const bool fits = (long long)e0 + tot <= p.pl_cap && (long long)c0 + nch <= p.chunk_cap;
+                if (lane == 0) {
+                    if (!fits) atomicOr(p.err, ERR_LIST);
+                    s_e0 = fits ? e0 : -1;
+                }
+                for (int t = lane; fits && t - lane < nch; t += 32) {
+                    const bool on = t < nch, lt = light(t);
+                    const unsigned bl = __ballot_sync(kFull, lt), bh = __ballot_sync(kFull, on && !lt), before = (1u << lane) - 1u;
+                    const int at = lt ? p.chunk_cap - 1 - (l0 + __popc(bl & before)) : h0 + __popc(bh & before);
+                    // (where some SC did not fit, the reservations may run past the table)
+                    if (on && at >= 0 && at < p.chunk_cap)
+                        p.pl_chunk[at] = make_int4(s.fc, e0 + t * kChunk, min(kChunk, tot - t * kChunk) | (s.ncl << 16), s.rr);
+                    l0 += __popc(bl);
+                    h0 += __popc(bh);
+                }
+            }
+        } else if (threadIdx.x == 0) {
             int tot = 0;
             for (int k = 0; k < kListWarps; ++k) tot += s_cnt[k];
             const int nch = (tot + kChunk - 1) / kChunk;
@@ -753,8 +826,9 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_fused(Params p)
             if (k < warp) off += s_cnt[k];
             tot += s_cnt[k];
         }
-        for (int t = threadIdx.x; t * kChunk < tot; t += blockDim.x)
-            p.pl_chunk[s_c0 + t] = make_int4(s.fc, e0 + t * kChunk, min(kChunk, tot - t * kChunk) | (s.ncl << 16), s.rr);
+        if constexpr (!ORDER)
+            for (int t = threadIdx.x; t * kChunk < tot; t += blockDim.x)
+                p.pl_chunk[s_c0 + t] = make_int4(s.fc, e0 + t * kChunk, min(kChunk, tot - t * kChunk) | (s.ncl << 16), s.rr);
         if (cnt <= kFound) {
             for (int b = 0; b < cnt; b += 32) {
                 ListJ j;
@@ -825,8 +899,8 @@ __device__ __forceinline__ void bonded_prologue(const Params& p)
 // more pairs than per-atom queues did (33 against 38 % of the evaluations
 // within r_cut, water at a 0.12 nm skin), which the cheaper tiles more than
 // pay for.  Per launch, 500,001-atom droplet 851 -> 768 us, water box of
-// 30,000 atoms 68.9 -> 62.9, 1,500 atoms 19.0 -> 10.5; hybrid screening, 12,003
-// atoms, 46.2 -> 40.9.  96 registers (20 warps per SM): with 80 (24 warps) the
+// 30,000 atoms 68.9 -> 60.1, 1,500 atoms 19.0 -> 10.5; hybrid screening, 12,003
+// atoms, 46.2 -> 39.1.  96 registers (20 warps per SM): with 80 (24 warps) the
 // compiler recomputes and spills (963 us), with 128 (16 warps) too few warps
 // cover the latencies (947 us before the j sums moved to shared memory).
 // Two tiles per branch for more independent work: 852 us, the longer code is
@@ -850,6 +924,7 @@ struct WarpF32 {
     int irow[kSCAtoms];            // shared-memory address of the SC atoms' LJ rows
     int ifr[kSCAtoms];             // and their fragments
     float jp[kChunk * 4 * kJpRow]; // j-force parts [entry][ty][component][tx]
+    int2 counts;                   // the list's chunks, and the heavy ones among them
     uint2 ent[kChunk];             // first slot of the j-cluster; i-cluster mask | kEntGen | kEntShare | cluster of the SC << 16
     JHyb<HYB> hy;
 };
@@ -962,7 +1037,7 @@ __device__ __forceinline__ void red_fix_if(long long* dst, float v, bool on, boo
     bad |= on && !ok;
 }
 
-template <bool ENERGY, bool HYB, int REGS>
+template <bool ENERGY, bool HYB, bool LIGHT, int REGS>
 __global__ void __maxnreg__(REGS) k_pair(Params p)
 {
     using P = Prec<false>;
@@ -987,11 +1062,17 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
     const int n_chunks = min(p.counters[7], p.chunk_cap);
     const int n_warps = gridDim.x * (blockDim.x >> 5);
     int item = warp * gridDim.x + blockIdx.x;
+    if constexpr (LIGHT) {
+        const int2 counts = chunk_counts(p);
+        item = chunk_at(p, item, counts);
+        if (lane == 0) w.counts = counts;   // (registers are short, and the counters' line is busy with the work counter)
+    }
+    auto any = [&](int it) { return LIGHT ? it >= 0 : it < n_chunks; };
     int4 ch = make_int4(0, 0, 0, 0);   // (first cluster, first entry, entries | clusters << 16, replica)
-    if (item < n_chunks) ch = p.pl_chunk[item];
+    if (any(item)) ch = p.pl_chunk[item];
     for (int k = threadIdx.x; k < nts * nts; k += blockDim.x) s_lj[k] = p.lj_f[k];
     PairEntry e4 = make_uint4(0u, 0u, 0u, 0u);
-    if (!(err & (ERR_CELL | ERR_LIST)) && item < n_chunks && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
+    if (!(err & (ERR_CELL | ERR_LIST)) && any(item) && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
     __syncthreads();
     if (err & (ERR_CELL | ERR_LIST)) return;
     bonded_prologue<false, ENERGY>(p);
@@ -1024,9 +1105,16 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
     // The work items are fetched ahead: while a chunk is evaluated, the counter's
     // answer and the descriptor of the next one are on their way, and its entries
     // are asked for before the i forces of this one are summed.
-    while (item < n_chunks) {
-        int next = n_chunks;
-        if (n_chunks > n_warps && lane == 0) next = n_warps + atomicAdd(&p.counters[2], 1);
+    while (any(item)) {
+        int next = LIGHT ? -1 : n_chunks;
+        if constexpr (LIGHT) {
+            if (lane == 0) {
+                const int warps = gridDim.x * (blockDim.x >> 5);
+                if (w.counts.x > warps) next = warps + atomicAdd(&p.counters[2], 1);
+            }
+        } else {
+            if (n_chunks > n_warps && lane == 0) next = n_warps + atomicAdd(&p.counters[2], 1);
+        }
         const int fc = ch.x, ent0 = ch.y, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         const Grid& g = p.grid_b[rr];
         c.kap = p.rs[rr].kappa_f;
@@ -1090,8 +1178,10 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
             fx[k] = fy[k] = fz[k] = 0.0f;
             if constexpr (ENERGY) ue[k] = 0.0f;
         }
+        if constexpr (LIGHT)
+            if (lane == 0 && next >= 0) next = chunk_at(p, next, w.counts);
         next = __shfl_sync(kFull, next, 0);
-        if (next < n_chunks) ch = p.pl_chunk[next];
+        if (any(next)) ch = p.pl_chunk[next];
         __syncwarp();
 
 #pragma unroll 1
@@ -1180,7 +1270,7 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
         }
         // the next chunk's entries
         e4 = make_uint4(0u, 0u, 0u, 0u);
-        if (next < n_chunks && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
+        if (any(next) && lane < (ch.z & 0xffff)) e4 = p.pl[ch.y + lane];
         item = next;
         // i forces: sum over the four lane rows, a transposing reduction that leaves
         // two i-clusters to each row; sums of exact zero (tiles never evaluated) add nothing
@@ -1270,7 +1360,7 @@ __global__ void __launch_bounds__(256, 1) k_pair64(Params p)
     bonded_prologue<true, ENERGY>(p);
 
     const int tx = lane & 7, ty = lane >> 3;
-    const int n_chunks = min(p.counters[7], p.chunk_cap);
+    const int2 counts = chunk_counts(p);
     // after the j-force reduction lane (tx, ty) holds component tx & 3 of atom
     // ty (tx < 4) or ty + 4 (tx >= 4) of the entry's j-cluster
     const int comp = tx & 3;
@@ -1289,9 +1379,9 @@ __global__ void __launch_bounds__(256, 1) k_pair64(Params p)
     while (true) {
         int item = 0;
         if (lane == 0) item = atomicAdd(&p.counters[2], 1);
-        item = __shfl_sync(kFull, item, 0);
-        if (item >= n_chunks) break;
-        const int4 ch = p.pl_chunk[item];          // (first cluster, first entry, entries | clusters << 16, replica)
+        item = chunk_at(p, __shfl_sync(kFull, item, 0), counts);
+        if (item < 0) break;
+        const int4 ch = p.pl_chunk[item];   // (first cluster, first entry, entries | clusters << 16, replica)
         const int fc = ch.x, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         __syncwarp();   // the previous chunk's reads of the staged entries are done
         if (lane < n_ent) w.ent[lane] = p.pl[ch.y + lane];
@@ -1633,7 +1723,7 @@ struct FragOp {
     __device__ void finish() {}
 };
 
-template <bool FP64, class Op>
+template <bool FP64, bool LIGHT, class Op>
 __global__ void __launch_bounds__(256) k_walk(Params p, Op op)
 {
     using P = Prec<FP64>;
@@ -1663,7 +1753,7 @@ __global__ void __launch_bounds__(256) k_walk(Params p, Op op)
     }
     __syncthreads();
     const int tx = lane & 7, ty = lane >> 3;
-    const int n_chunks = min(p.counters[7], p.chunk_cap);
+    const int n_chunks = min(p.counters[7], p.chunk_cap), n_heavy = LIGHT ? chunk_counts(p).y : n_chunks;
     const float reach = op.reach(p);
     const bool near_only = reach < list_rlist_f(p);   // the operation needs only pairs well inside the list's radius
     while (true) {
@@ -1671,6 +1761,7 @@ __global__ void __launch_bounds__(256) k_walk(Params p, Op op)
         if (lane == 0) item = atomicAdd(&p.counters[2], 1);
         item = __shfl_sync(kFull, item, 0);
         if (item >= n_chunks) break;
+        if (LIGHT) item = chunk_at(p, item, make_int2(n_chunks, n_heavy));
         const int4 ch = p.pl_chunk[item];
         const int fc = ch.x, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
         PairEntry ent = lane < n_ent ? p.pl[ch.y + lane] : make_uint4(0u, 0u, 0u, 0u);
@@ -1758,11 +1849,12 @@ template <bool FP64, class Op>
 static void launch_walk(const Params& p, cudaStream_t s, int n_sm, Op op, size_t op_smem)
 {
     const size_t smem = op_smem + 256 * sizeof(unsigned) + 8 * sizeof(WalkWarp<FP64>);
-    cudaFuncSetAttribute(k_walk<FP64, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const auto f = has_light(p) ? k_walk<FP64, true, Op> : k_walk<FP64, false, Op>;
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     // as many blocks as an SM holds: the walks wait on dependent loads
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk<FP64, Op>, 256, smem);
-    k_walk<FP64, Op><<<n_sm * std::max(per_sm, 1), 256, smem, s>>>(p, op);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem);
+    f<<<n_sm * std::max(per_sm, 1), 256, smem, s>>>(p, op);
 }
 
 template <bool FP64>
@@ -1812,11 +1904,11 @@ static size_t pair_smem(int n_ts, int warps)
 // to fill more warps: per launch 1,500 atoms 18.4 (96) and 15.6 us (128; 10.5 since), 8,005
 // atoms in unbuffered lists 25.9 and 23.9, 30,000 atoms 64.6 and 65.0.
 constexpr int kFewChunksAtoms = 16384;
-template <bool FP64, bool ENERGY, bool HYB, bool FEW>
+template <bool FP64, bool ENERGY, bool HYB, bool FEW, bool LIGHT>
 static auto pair_kernel()
 {
     if constexpr (FP64) return k_pair64<ENERGY, HYB>;
-    else return k_pair<ENERGY, HYB, ENERGY || HYB || FEW ? 128 : 96>;
+    else return k_pair<ENERGY, HYB, LIGHT, ENERGY || HYB || FEW ? 128 : 96>;
 }
 
 constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
@@ -1827,7 +1919,7 @@ constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
 //   hybrid screening); with more states two blocks of 4 warps take their place.
 //   Mixed, 96 registers: 20 warps fit an SM's registers, as five blocks of 4 while
 //   the five tables are small (up to 28 type states), then as two blocks of 10 (up
-//   to 47) or one of 20 (up to 67).  Protein crystal, 43 type states, 199,773
+//   to 46) or one of 20 (up to 67).  Protein crystal, 43 type states, 199,773
 //   atoms: 398.8 us with 16 warps, 363.4 with 20.
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int fit_warps(int warps, int n_ts)
@@ -1843,37 +1935,37 @@ static int fit_warps(int warps, int n_ts)
     return warps;
 }
 
-template <bool FP64, bool ENERGY, bool HYB, bool FEW>
+template <bool FP64, bool ENERGY, bool HYB, bool FEW, bool LIGHT>
 static void set_smem_attr()
 {
     static bool done = false;   // one per instantiation
     if (!done) {
-        const auto f = pair_kernel<FP64, ENERGY, HYB, FEW>();
+        const auto f = pair_kernel<FP64, ENERGY, HYB, FEW, LIGHT>();
         cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
         cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         done = true;
     }
 }
 
-template <bool FP64, bool ENERGY, bool HYB, bool FEW>
+template <bool FP64, bool ENERGY, bool HYB, bool FEW, bool LIGHT>
 static void launch_one(const Params& p, cudaStream_t s, int blocks, int warps)
 {
-    set_smem_attr<FP64, ENERGY, HYB, FEW>();
+    set_smem_attr<FP64, ENERGY, HYB, FEW, LIGHT>();
     const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, p.n_ts_lj);
     if (blocks * warps % fit == 0) {
         blocks = blocks * warps / fit;
         warps = fit;
     }
-    pair_kernel<FP64, ENERGY, HYB, FEW>()<<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
+    pair_kernel<FP64, ENERGY, HYB, FEW, LIGHT>()<<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
 }
 
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int max_blocks(int warps, int n_ts)
 {
-    set_smem_attr<FP64, ENERGY, HYB, FEW>();
+    set_smem_attr<FP64, ENERGY, HYB, FEW, true>();
     const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, n_ts);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW>(), fit * 32,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW, true>(), fit * 32,
                                                   pair_smem<FP64, HYB>(n_ts, fit));
     return n * fit / warps;
 }
@@ -1913,7 +2005,8 @@ int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
 int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm)
 {
     if (p.sc_cap <= kListFusedScs) {
-        k_list_fused<<<std::min(p.sc_cap, n_sm * 8), kListWarps * 32, 0, s>>>(p);
+        const auto f = has_light(p) ? k_list_fused<true> : k_list_fused<false>;
+        f<<<std::min(p.sc_cap, n_sm * 8), kListWarps * 32, 0, s>>>(p);
         return 1;
     }
     int n = 2;
@@ -1936,8 +2029,9 @@ void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks
 {
     with_instance(p.precision != 0, energy, p.screening != 0, p.n_atoms <= kFewChunksAtoms,
                   [&](auto fp64, auto en, auto hyb, auto few) {
-                      launch_one<decltype(fp64)::value, decltype(en)::value, decltype(hyb)::value, decltype(few)::value>(
-                          p, s, blocks, warps);
+                      constexpr bool D = decltype(fp64)::value, E = decltype(en)::value, H = decltype(hyb)::value, F = decltype(few)::value;
+                      if (D || has_light(p)) launch_one<D, E, H, F, true>(p, s, blocks, warps);
+                      else launch_one<D, E, H, F, D>(p, s, blocks, warps);
                   });
 }
 

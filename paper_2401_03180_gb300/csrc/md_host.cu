@@ -946,7 +946,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     DALLOC(P.cell_count, C); DALLOC(P.cell_start, C + 1); DALLOC(P.cell_pstart, C + 1);
     DALLOC(P.tmp_key, N);
     DALLOC(P.sc_cell, P.sc_cap); DALLOC(P.sc_first, P.sc_cap); DALLOC(P.sc_ncl, P.sc_cap);
-    DALLOC(P.counters, 8);
+    DALLOC(P.counters, kCounters);
     DALLOC(P.list_cnt, (size_t)P.sc_cap * kHalfShell);
     DALLOC(P.sc_tot, P.sc_cap); DALLOC(P.sc_eoff, P.sc_cap); DALLOC(P.sc_coff, P.sc_cap);
     DALLOC(P.scan_tmp, 3 * kScanCtasMax);
@@ -1074,7 +1074,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
         CU(cudaMemcpy(d_ljf, lj_f.data(), lj_f.size() * sizeof(float2), cudaMemcpyHostToDevice));
         CU(cudaMemcpy(d_ljd, lj_d.data(), lj_d.size() * sizeof(double2), cudaMemcpyHostToDevice));
         CU(cudaMemset(P.cell_count, 0, C * sizeof(int)));
-        CU(cudaMemset(P.counters, 0, 8 * sizeof(int)));
+        CU(cudaMemset(P.counters, 0, kCounters * sizeof(int)));
         {
             // the first cell assignment walks atoms in input order
             std::vector<int> ident(P.slot_cap, -1);

@@ -21,6 +21,7 @@ constexpr int kListMinPerCluster = 32;   // initial pair-list entries per cluste
 constexpr int kMaxSpecies = 8;
 constexpr int kMaxTS = 128;
 constexpr int kNEtab = 16 * 40;       // e^{-k/16} table, lambda < 40
+constexpr int kCounters = 9;
 constexpr int kRepWindow = 8;         // replicas per CTA kept in shared memory
 constexpr double kFixScale = 4294967296.0;        // 2^32
 constexpr double kFixInv = 1.0 / 4294967296.0;
@@ -189,7 +190,7 @@ struct Params {
     int* sc_cell;            // [sc_cap]
     int* sc_first;           // [sc_cap] first cluster
     int* sc_ncl;             // [sc_cap] clusters in the super-cluster
-    int* counters;           // [0] n_sc, [1] n_slots, [2] work, [3] ticket, [4] big cells, [6] list entries, [7] chunks
+    int* counters;           // [0] n_sc, [1] n_slots, [2] work, [3] ticket, [4] big cells, [5] light chunks, [6] list entries, [7] chunks, [8] heavy chunks placed
     int* big_cells;          // [cell_cap_total] cells too large for the one-warp sort (counters[4] of them)
     int* list_cnt;           // [sc_cap * kHalfShell] entries of each super-cluster in each half-shell cell
     int* sc_tot;             // [sc_cap] entries per super-cluster

@@ -65,7 +65,7 @@ constexpr Layout make_layout()
     L.cell_count = take(4 * kNcMax); L.cell_start = take(4 * (kNcMax + 1)); L.cell_pstart = take(4 * (kNcMax + 1));
     L.tmp_key = take(8 * kNaMax);
     L.sc_cell = take(4 * kClusterCap); L.sc_first = take(4 * kClusterCap); L.sc_ncl = take(4 * kClusterCap);
-    L.counters = take(4 * 8);
+    L.counters = take(4 * kCounters);
     L.list_cnt = take(4 * (size_t)kClusterCap * kHalfShell);
     L.sc_tot = take(4 * kClusterCap);
     L.sc_eoff = take(4 * kClusterCap); L.sc_coff = take(4 * kClusterCap);
@@ -186,7 +186,7 @@ __global__ void k_noalloc_prepare(Params p, NaTables tb, Grid g, double volume, 
         for (int d = 0; d < 3; ++d) { a.bmin[d] = ~0ull; a.bmax[d] = 0ull; }
     }
     if (t == 0) {
-        for (int k = 0; k < 8; ++k) p.counters[k] = 0;
+        for (int k = 0; k < kCounters; ++k) p.counters[k] = 0;
         p.counters[1] = n;
         *p.step = 0;
         *p.kick_full = 0;

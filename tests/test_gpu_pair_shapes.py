@@ -37,8 +37,8 @@ def _system(z):
     return s, W.atomic_data(8.0, z=z), kw
 
 
-# 27, 28, 29 type states; 47, 48; 67, 68; 128
-@pytest.mark.parametrize("z", [(17, 8), (18, 8), (19, 8), (30, 15), (31, 15), (32, 32), (32, 32, 1), (32, 32, 32, 28)])
+# 27, 28, 29 type states; 46, 47; 66, 68; 128
+@pytest.mark.parametrize("z", [(17, 8), (18, 8), (19, 8), (32, 12), (30, 15), (32, 32), (32, 32, 1), (32, 32, 32, 28)])
 def test_default_shape_equals_a_pinned_one(z):
     s, atom, kw = _system(z)
     out = []
