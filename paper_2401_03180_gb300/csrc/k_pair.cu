@@ -227,20 +227,20 @@ __device__ __forceinline__ void pair64(const double4_16a& xi, int row_off, int f
 // chunks of kChunk, the work items of the force kernel.  The j-clusters of an
 // SC's 14 half-shell cells form one index range, swept 32 at a time with every
 // lane busy (cell by cell would leave lanes idle and chain one load latency per
-// cell).  Three kernels, with no block-level barrier:
+// cell).  Five kernels, the box tests with no block-level barrier:
 //   k_list_count  a warp per (SC, part of its index range) item counts the
 //                 entries of its part;
-//   k_list_scan   one block sums each SC's parts and scans the totals into
-//                 entry and chunk offsets (and flags a list too small for them);
+//   k_list_scan_* three kernels sum each SC's parts and scan the totals into
+//                 entry and chunk offsets (and flag a list too small for them);
 //   k_list_write  a warp per item repeats the box tests in the same rounding
 //                 and writes its entries from its offset (the SC's plus the
 //                 counts of the SC's earlier parts); the SC's first item writes
 //                 the SC's chunk descriptors.
 // An SC's range is split into 1, 2, 7 or 14 parts (list_parts): as few as keep
 // every warp of the grid busy, so that a system of many SCs stages each SC once
-// and a smaller one still spreads over the GPU.  Systems of few SCs take
-// k_list_fused below instead.
-constexpr int kListFusedScs = 8192;   // super-cluster capacities up to this build their list in one kernel (k_list_fused)
+// and a smaller one still spreads over the GPU.  Systems of up to kListFusedScs
+// SCs take k_list_fused below instead.
+constexpr int kListFusedScs = 32768;   // super-cluster capacities up to this build their list in one kernel (k_list_fused)
 // Whether the list of these parameters holds light chunks apart (k_list_fused, lists
 // that serve several steps).  The kernels that find them (LIGHT) cost large systems
 // and single calls more than they give: 500,001 atoms 768 us without, 786 with.
@@ -265,7 +265,6 @@ struct ListWarp {
     float4 ip[kSCAtoms];                              // the SC's atoms, [cluster k][atom a] (write pass)
 };
 constexpr int kListWarps = 8;
-constexpr int kScanScsMulti = 32768;   // super-cluster capacities from this size are scanned by many CTAs
 
 // An SC's cell, in the grid of its replica.
 struct ListSC {
@@ -523,19 +522,7 @@ __device__ __forceinline__ void scan_scs_finish(const Params& p, long long E, lo
     if (E > p.pl_cap || Cn > p.chunk_cap) atomicOr(p.err, ERR_LIST);
 }
 
-// Few SCs: one block does both passes.
-__global__ void __launch_bounds__(1024) k_list_scan(Params p)
-{
-    __shared__ int s_tot[32][2], s_base[32][2];
-    const int n = (*p.err & ERR_CELL) ? 0 : p.counters[0];
-    const int zero[2] = {0, 0};
-    scan_scs<false>(p, 0, n, zero, s_tot, s_base);
-    scan_scs<true>(p, 0, n, zero, s_tot, s_base);
-    if (threadIdx.x == 0)
-        scan_scs_finish(p, (long long)s_base[31][0] + s_tot[31][0], (long long)s_base[31][1] + s_tot[31][1]);
-}
-
-// Many SCs: each CTA sums its range; one CTA scans the sums (and finishes);
+// Each CTA sums its range; one CTA scans the sums (and finishes);
 // each CTA scans its range from its base (p.scan_tmp: [CTA][2]).
 __device__ __forceinline__ void sc_cta_range(int n, int& lo, int& hi)
 {
@@ -709,12 +696,15 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
 // j-clusters it found in range (compacted in shared memory, kFound of them; a
 // warp that finds more repeats the box tests), the block adds up its warps'
 // counts and reserves the SC's entries and chunks with one atomic each.  An
-// SC's entries and chunks are those of the three kernels above; only where they
+// SC's entries and chunks are those of the kernels above; only where they
 // lie in the list follows the order of the atomics, which no sum depends on.
-// Latency-bound: what the three kernels spend on their launches, on staging the
+// Latency-bound: what the kernels above spend on their launches, on staging the
 // SC once per part and pass, and on entries of j-clusters out of range is saved.
 // Count, scan and write against this kernel, per build: 8,005 atoms (unbuffered)
-// 20.1 -> 8.9 us, 12,297 atoms 23.6 -> 11.6, 30,000 atoms 31.9 -> 17.3.
+// 20.1 -> 8.9 us, 12,297 atoms 23.6 -> 11.6, 30,000 atoms 31.9 -> 17.3, 199,773 atoms
+// of protein crystal 111 -> 80.  The line lies where staging the SC for one part
+// pays: 500,001 atoms take 194 us that way and 186 this way, 2 M atoms 647 and 739, a
+// batch of 300,000 93 and 96.
 //
 // ORDER (buffered lists of up to kLightScs): the chunks of fewer than kLightTiles
 // tiles (i-clusters in range of an entry, before trimming) go to the end of the chunk
@@ -2009,20 +1999,13 @@ int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm)
         f<<<std::min(p.sc_cap, n_sm * 8), kListWarps * 32, 0, s>>>(p);
         return 1;
     }
-    int n = 2;
     k_list_count<<<blocks, kListWarps * 32, 0, s>>>(p);
-    if (p.sc_cap >= kScanScsMulti) {
-        const int ctas = std::min(kScanCtasMax, (p.sc_cap + 2047) / 2048);
-        k_list_scan_sums<<<ctas, 1024, 0, s>>>(p);
-        k_list_scan_top<<<1, 1024, 0, s>>>(p, ctas);
-        k_list_scan_apply<<<ctas, 1024, 0, s>>>(p);
-        n += 3;
-    } else {
-        k_list_scan<<<1, 1024, 0, s>>>(p);
-        n += 1;
-    }
+    const int ctas = std::min(kScanCtasMax, (p.sc_cap + 2047) / 2048);
+    k_list_scan_sums<<<ctas, 1024, 0, s>>>(p);
+    k_list_scan_top<<<1, 1024, 0, s>>>(p, ctas);
+    k_list_scan_apply<<<ctas, 1024, 0, s>>>(p);
     k_list_write<<<blocks, kListWarps * 32, 0, s>>>(p);
-    return n;
+    return 5;
 }
 
 void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks, int warps)
