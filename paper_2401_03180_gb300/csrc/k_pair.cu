@@ -1366,10 +1366,22 @@ __global__ void __launch_bounds__(256, 1) k_pair64(Params p)
     const T irc = T(1.0 / p.r_cut);
     const T coulf = p.coulomb_f;
 
+    // A warp's first chunk is its own index, neighbours on different SMs, the rest
+    // come from the counter.  The FP64 pipe is the SM's: with every first chunk from
+    // the counter, the first SMs to ask took up to eight of a small system's chunks
+    // and others none.  Per launch 3,224 atoms 317 -> 252 us, 1,500 atoms 239 -> 232,
+    // 30,000 atoms 1,561 -> 1,551.
+    const int n_warps = gridDim.x * (blockDim.x >> 5);
+    bool first = true;
     while (true) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&p.counters[2], 1);
-        item = chunk_at(p, __shfl_sync(kFull, item, 0), counts);
+        int item = warp * gridDim.x + blockIdx.x;
+        if (!first) {
+            if (counts.x <= n_warps) break;
+            if (lane == 0) item = n_warps + atomicAdd(&p.counters[2], 1);
+            item = __shfl_sync(kFull, item, 0);
+        }
+        first = false;
+        item = chunk_at(p, item, counts);
         if (item < 0) break;
         const int4 ch = p.pl_chunk[item];   // (first cluster, first entry, entries | clusters << 16, replica)
         const int fc = ch.x, n_ent = ch.z & 0xffff, ncl = ch.z >> 16, rr = ch.w;
