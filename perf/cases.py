@@ -374,6 +374,15 @@ def _replica_forces(x, q, sp, frag, box, kap, ne, hybrid, topo):
     return F.cpu().numpy(), U, pairs
 
 
+def _own_terms(topo, a, b):
+    """The bonded terms of the replica of atoms a .. b - 1, by that replica's own atom indices."""
+    if topo is None:
+        return None
+    bonds, angles = (t[(t[:, 0] >= a) & (t[:, 0] < b)] for t in (topo.bonds, topo.angles))
+    return W.Topology(bonds=bonds - np.array([a, a, 0], bonds.dtype), bond_params=topo.bond_params,
+                      angles=angles - np.array([a, a, a, 0], angles.dtype), angle_params=topo.angle_params)
+
+
 def _forces(case, s, st):
     kap, ne, _ = _kappa(st, s)
     F, U, pairs = np.empty((s.n_atoms, 3)), np.zeros(s.n_replicas), 0
@@ -381,7 +390,7 @@ def _forces(case, s, st):
         a, b = int(s.replica_offset[r]), int(s.replica_offset[r + 1])
         F[a:b], U[r], k = _replica_forces(st["x"][a:b], st["q"][a:b], s.species[a:b], s.fragment[a:b],
                                           float(s.box[r, 0]), float(kap[r]), float(ne[r]),
-                                          case.get("screening") == "hybrid", s.topology)
+                                          case.get("screening") == "hybrid", _own_terms(s.topology, a, b))
         pairs += k
     return F, U, pairs
 
