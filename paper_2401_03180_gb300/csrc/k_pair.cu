@@ -1134,8 +1134,7 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
             unsigned im = e4.z | e4.w;             // i-clusters with some atom in the mask
             im |= im >> 16;
             im = (im | (im >> 8)) & 0xffu;
-            const bool self = (e4.y & 0xffu) == 0u;
-            const unsigned kd = self ? (e4.x - (unsigned)fc) & 0xffffu : 0xffffu;   // i-cluster equal to the j-cluster
+            const unsigned kd = self_cluster((e4.y & 0xffu) == 0u, e4.x, (unsigned)fc);   // i-cluster equal to the j-cluster
             const bool share = (e4.y & kEntryExcl) != 0u;
             w.ent[lane] = make_uint2(e4.x * kClusterSize, im | (kd < (unsigned)ncl || share ? kEntGen : 0u) |
                                                               (share ? kEntShare : 0u) | (kd << 16));

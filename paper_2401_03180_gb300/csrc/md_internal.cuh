@@ -7,13 +7,13 @@
 
 #include <cuda_runtime.h>
 
+#include "rules.cuh"
+
 namespace mdg {
 
-// Atoms are grouped in clusters of 8 consecutive slots of the cell-sorted
-// order; a warp processes one super-cluster of up to K_SC i-clusters against
-// one neighbour cell at a time.
-constexpr int kClusterSize = 8;
-constexpr int kSuperClusters = 8;     // K_SC
+// Atoms are grouped in clusters of kClusterSize consecutive slots of the
+// cell-sorted order; a warp processes one super-cluster of up to
+// kSuperClusters i-clusters against one neighbour cell at a time.
 constexpr int kHalfShell = 14;        // self cell + 13 neighbour cells
 constexpr int kSCAtoms = kSuperClusters * kClusterSize;   // atom slots of a super-cluster
 constexpr int kChunk = 8;             // cluster-pair list entries per force work item
