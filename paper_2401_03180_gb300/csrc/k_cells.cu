@@ -332,10 +332,9 @@ __device__ __forceinline__ void pack_cell(const Params& p, const int* order, int
             lo[2] = hi[2] = v.z;
             fmin = fmax = fr;
         } else if (e < npad) {   // padding: far away, no charge
-            const double far = 1.0e6 + 1024.0 * (double)slot;
             p.atom_of[slot] = -1;
-            if (p.precision == 0) p.xq[slot] = make_float4((float)far, 1.0e6f, 1.0e6f, 0.0f);
-            else p.xq64[slot] = make_double4_32a(far, 1.0e6, 1.0e6, 0.0);
+            if (p.precision == 0) p.xq[slot] = make_float4((float)pad_x(slot), (float)kPadFar, (float)kPadFar, kPadCharge);
+            else p.xq64[slot] = make_double4_32a(pad_x(slot), kPadFar, kPadFar, (double)kPadCharge);
             p.tf[slot] = make_int2(0, -1 - slot);
             p.fx[slot] = 0; p.fy[slot] = 0; p.fz[slot] = 0; p.epot[slot] = 0;
         }

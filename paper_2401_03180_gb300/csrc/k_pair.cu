@@ -1168,7 +1168,7 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
             if (a < ncl * kClusterSize) {
                 const float4 v = p.xq[fc * kClusterSize + a];
                 const int2 t = p.tf[fc * kClusterSize + a];
-                w.ix[a] = make_float4(v.x, v.y, v.z, (HYB ? c.hf : coulf) * v.w);
+                w.ix[a] = make_float4(staged_x(v.x, v.w), v.y, v.z, (HYB ? c.hf : coulf) * v.w);
                 w.irow[a] = lj_addr + t.x * nts * (int)sizeof(float2);
                 w.ifr[a] = t.y;
                 if constexpr (HYB) w.hy.iGr[a] = make_float2(c.hf * c.rows[(int)v.w].Gf, c.rows[(int)v.w].rpf);

@@ -2,6 +2,8 @@
 // the device, in the library's host code and in a plain C++ compiler.
 #pragma once
 
+#include <cmath>
+
 #if defined(__CUDACC__)
 #define MDG_HD __host__ __device__ __forceinline__
 #else
@@ -22,5 +24,17 @@ MDG_HD unsigned self_cluster(bool own_cell, unsigned jc, unsigned fc)
     const unsigned d = jc - fc;
     return own_cell && d < (unsigned)kSuperClusters ? d : kNoSelf;
 }
+
+// Padding slots fill a cell's last cluster.  Their records lie far from every atom,
+// 1,024 nm apart along x in 64 bits; in 32 bits neighbouring ones coincide from
+// slot 2^24 on (beyond 2^34 nm), and a cell's shift may bring those of two cells
+// together.  The mixed force kernel evaluates whole cluster tiles, pads included, so
+// it stages the pads of the i side on the other side of the origin, out of reach of
+// every j-atom and pad; they carry the charge -0, which no atom has.
+constexpr double kPadFar = 1.0e6, kPadStep = 1024.0;   // nm
+constexpr float kPadCharge = -0.0f;
+constexpr float kPadStaged = -1.0e18f;
+MDG_HD double pad_x(int slot) { return kPadFar + kPadStep * (double)slot; }
+MDG_HD float staged_x(float x, float q) { return std::signbit(q) ? kPadStaged : x; }
 
 }  // namespace mdg

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -32,3 +33,27 @@ def test_self_cluster_compares_the_whole_difference(rules, d, k):
         assert lib.f(1, fc + d, fc) == (lib.none() if k is None else k)
         assert lib.f(0, fc + d, fc) == lib.none()
     assert lib.none() >= 8
+
+
+@pytest.mark.parametrize("slot", [0, 8, 1 << 20, 1 << 24, (1 << 24) + 4096, 1 << 25, (1 << 30) - 8])
+def test_padding_is_out_of_reach_of_padding(rules, slot):
+    """Pads of a cluster, as the mixed force kernel stages them on the i side, against
+    the same cluster's and other cells' pads on the j side, in 32 bits: never within
+    the largest cutoff (1,000 nm), though the j side's coincide from slot 2^24 on."""
+    lib = rules("float x(int s) { return (float)pad_x(s); }\n"
+                "float staged(float x, float q) { return staged_x(x, q); }\n"
+                "float charge() { return kPadCharge; }\nfloat far_() { return (float)kPadFar; }")
+    for f in (lib.x, lib.staged, lib.charge, lib.far_):
+        f.restype = ctypes.c_float
+    lib.staged.argtypes = [ctypes.c_float, ctypes.c_float]
+    pads = np.array([lib.x(slot + k) for k in range(8)], np.float32)
+    assert (len(np.unique(pads)) < 8) == (slot >= 1 << 24)
+    i = np.array([lib.staged(v, lib.charge()) for v in pads], np.float32)
+    y = np.float32(lib.far_())
+    for shift in (0.0, 1.2, -8192.0, 1.0e6):
+        dx = i[:, None] - (pads + np.float32(shift))[None]
+        dy = y - (y + np.float32(shift))
+        r2 = dx * dx + np.float32(2) * dy * dy
+        assert np.isfinite(r2).all() and r2.min() > 1.0e6 ** 2
+    assert lib.staged(ctypes.c_float(3.5), ctypes.c_float(0.0)) == 3.5          # a neutral atom stays where it is
+    assert lib.staged(ctypes.c_float(3.5), ctypes.c_float(2.0)) == 3.5
