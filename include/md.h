@@ -190,8 +190,12 @@ typedef struct md_config {
      * value pins that axis (the autotuner then leaves it alone).            */
     int pair_warps;          /* warps per force-kernel block: 4, 8 or 12
                                 (FP64: 4 or 8)                                 */
-    int pair_blocks_per_sm;  /* force-kernel blocks per SM, >= 1, within the
-                                occupancy the shape allows                     */
+    int pair_blocks_per_sm;  /* force-kernel blocks per SM, >= 1: up to 24 / warps
+                                (FP64: 16 / warps), less where the blocks'
+                                tables fill 228 KB of shared memory: (type
+                                states)^2 * 8 bytes (FP64: 16) and about 8 to
+                                9.7 KB per warp (FP64: 15 to 18).  Blocks that
+                                are not resident at once run one after another */
     int sort_threads;        /* threads per cell-sort block: 256 or 1024       */
     int list_blocks_per_sm;  /* list-build blocks (8 warps) per SM: 1 .. 16    */
     int list_skin_adaptive;  /* 1 (with list_skin_nm > 0): the device drops the

@@ -1930,8 +1930,9 @@ constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
 
 // Warps of the blocks that a launch shape of `warps` per block is launched with,
 // given the block's own LJ table; the shape changes no result.
-//   FP64: blocks of 8 warps leave 44 KB for the table (53 type states; 38 with
-//   hybrid screening); with more states two blocks of 4 warps take their place.
+//   FP64: blocks of 8 warps leave 47 KB for the table (55 type states; 41 with
+//   hybrid screening), blocks of 4 take up to 93 (90), of 2 up to 107 (106) and of
+//   one up to 114 (113); more blocks of fewer warps replace those that do not fit.
 //   Mixed, 96 registers: 20 warps fit an SM's registers, as five blocks of 4 while
 //   the five tables are small (up to 28 type states), then as two blocks of 10 (up
 //   to 46) or one of 20 (up to 67).  Protein crystal, 43 type states, 199,773
@@ -1939,14 +1940,14 @@ constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int fit_warps(int warps, int n_ts)
 {
-    if (FP64) {
-        while (warps > 4 && pair_smem<FP64, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
-        return warps;
+    if constexpr (FP64) {
+        while (warps > 1 && pair_smem<FP64, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
+    } else if constexpr (!ENERGY && !HYB && !FEW) {
+        constexpr int kWarps96 = 20, kSmemSm = 228 * 1024, kSmemBlock = 1024;   // an SM's shared memory, and what a block takes besides its own
+        if (warps != 4) return warps;
+        for (int w : {4, 10, 20})
+            if (pair_smem<FP64, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
     }
-    constexpr int kWarps96 = 20, kSmemSm = 228 * 1024, kSmemBlock = 1024;   // an SM's shared memory, and what a block takes besides its own
-    if (ENERGY || HYB || FEW || warps != 4) return warps;
-    for (int w : {4, 10, 20})
-        if (pair_smem<FP64, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
     return warps;
 }
 
@@ -1982,7 +1983,7 @@ static int max_blocks(int warps, int n_ts)
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW, true>(), fit * 32,
                                                   pair_smem<FP64, HYB>(n_ts, fit));
-    return n * fit / warps;
+    return n > 0 ? std::max(1, n * fit / warps) : 0;
 }
 
 // Calls f with the force kernel's instance as compile-time constants.
@@ -2003,18 +2004,6 @@ static void with_instance(bool fp64, bool energy, bool hyb, bool few, F&& f)
     if (fp64) eh(T{}, N{});
     else if (few && !energy && !hyb) f(N{}, N{}, N{}, T{});
     else eh(N{}, N{});
-}
-
-// Largest pair_blocks_per_sm a caller may pin for `warps` warps per block: the
-// interface's limits (24 resident warps per SM, less where the LJ table fills
-// the shared memory).  More blocks than fit at once are correct as well: blocks
-// take chunks from a counter until none is left.
-int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
-{
-    if (fp64) return std::max(1, pair_max_blocks_per_sm(true, false, hyb, warps, n_ts, 0));
-    const size_t tab = ((size_t)n_ts * n_ts * sizeof(float2) + 127) / 128 * 128;
-    const size_t block = tab + 1024 + (size_t)warps * (hyb ? 9664 : 8272) + 1024;
-    return std::max(1, std::min(24 / warps, (int)(233472 / block)));
 }
 
 int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm)

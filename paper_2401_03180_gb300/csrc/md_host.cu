@@ -1102,12 +1102,12 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
         if (c.pair_warps) {
             h->pair_warps = c.pair_warps;
         } else {
-            // (with the blocks per SM pinned, by the interface's limits, whose 8 or
-            // 12 warps a block decide which pins are accepted)
+            // (with the blocks per SM pinned, by the interface's limits for blocks of 8 and
+            // 12 warps, which decide what pins are accepted; of the shapes that fit)
             const bool pinned = c.pair_blocks_per_sm != 0;
             auto most = [&](int w) {
-                return w * (pinned ? pair_pin_limit(fp64, c.screening != 0, w, h->NTS_LJ)
-                                   : pair_max_blocks_per_sm(fp64, false, c.screening != 0, w, h->NTS_LJ, h->N));
+                const int n = pair_max_blocks_per_sm(fp64, false, c.screening != 0, w, h->NTS_LJ, h->N);
+                return w * (pinned && n ? pair_pin_limit(fp64, c.screening != 0, w, h->NTS_LJ) : n);
             };
             h->pair_warps = 8;
             int best = most(8);
@@ -1123,7 +1123,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
         if (c.pair_blocks_per_sm > pin)
             return fail(h, MD_ERR_INVALID_ARG, "pair_blocks_per_sm exceeds the " + std::to_string(pin) +
                                                    " blocks of " + std::to_string(h->pair_warps) +
-                                                   " warps an SM holds for this system");
+                                                   " warps accepted for this system");
         h->pair_blocks = h->n_sm * (c.pair_blocks_per_sm ? c.pair_blocks_per_sm : maxb);
     }
     // list kernels: one warp per super-cluster (or per group of its cells), 8 warps per block

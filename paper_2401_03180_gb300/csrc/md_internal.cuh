@@ -353,7 +353,6 @@ void launch_frag_count(const Params& p, cudaStream_t s, const int* parent, int* 
                        const int* mass_number, int mass_max, int charge_max, unsigned long long* counts);
 // resident blocks per SM; 0: the shape does not fit
 int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms);
-int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts);
 // message returned by md_last_error(NULL) (host side)
 void set_global_error(const std::string& msg);
 

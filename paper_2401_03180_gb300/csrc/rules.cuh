@@ -37,4 +37,23 @@ constexpr float kPadStaged = -1.0e18f;
 MDG_HD double pad_x(int slot) { return kPadFar + kPadStep * (double)slot; }
 MDG_HD float staged_x(float x, float q) { return std::signbit(q) ? kPadStaged : x; }
 
+// Largest blocks per SM that a caller may pin for blocks of `warps` warps, beside an
+// LJ table of n_ts type states.  The limit is a promise of the interface and stands
+// apart from the kernels of the day: it is what an SM held (registers, then shared
+// memory) of the force kernels with which the interface was first given, whose warps
+// took the bytes below.  More blocks than an SM holds of the present ones are
+// correct as well: they run one after another and take chunks until none is left.
+constexpr int kPinWarpBytes[2][2] = {{8272, 9664}, {15312, 18112}};   // [FP64][hybrid electrostatics]
+constexpr int kPinSmWarps[2] = {24, 16};                              // resident warps by registers, [FP64]
+constexpr int kPinBlockBytes = 1024 + 1024;                           // a block's lookup table, and what the SM keeps per block
+constexpr int kPinSmBytes = 228 * 1024;
+inline int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
+{
+    const int table = (n_ts * n_ts * (fp64 ? 16 : 8) + 127) / 128 * 128;
+    const int by_smem = kPinSmBytes / (table + kPinBlockBytes + warps * kPinWarpBytes[fp64][hyb]);
+    const int by_regs = kPinSmWarps[fp64] / warps;
+    const int n = by_smem < by_regs ? by_smem : by_regs;
+    return n > 1 ? n : 1;
+}
+
 }  // namespace mdg

@@ -57,3 +57,16 @@ def test_padding_is_out_of_reach_of_padding(rules, slot):
         assert np.isfinite(r2).all() and r2.min() > 1.0e6 ** 2
     assert lib.staged(ctypes.c_float(3.5), ctypes.c_float(0.0)) == 3.5          # a neutral atom stays where it is
     assert lib.staged(ctypes.c_float(3.5), ctypes.c_float(2.0)) == 3.5
+
+
+# (FP64, hybrid, warps, type states, blocks): the shapes that the interface has always accepted
+PINS = [(0, 0, 4, 2, 6), (0, 0, 8, 2, 3), (0, 0, 12, 2, 2), (0, 0, 4, 46, 4), (0, 0, 8, 46, 2), (0, 0, 12, 46, 1),
+        (0, 0, 8, 128, 1), (0, 1, 4, 28, 4), (0, 1, 12, 10, 1),
+        (1, 0, 4, 28, 3), (1, 0, 4, 30, 3), (1, 0, 4, 31, 2), (1, 0, 4, 57, 2), (1, 0, 4, 58, 1), (1, 0, 4, 94, 1),
+        (1, 0, 8, 2, 1), (1, 1, 4, 14, 3), (1, 1, 4, 15, 2), (1, 1, 4, 51, 2), (1, 1, 4, 52, 1), (1, 1, 8, 2, 1)]
+
+
+@pytest.mark.parametrize("fp64,hyb,warps,n_ts,blocks", PINS)
+def test_pinned_blocks_per_sm_stay_accepted(rules, fp64, hyb, warps, n_ts, blocks):
+    lib = rules("int f(int d, int h, int w, int n) { return pair_pin_limit(d != 0, h != 0, w, n); }")
+    assert lib.f(fp64, hyb, warps, n_ts) == blocks
