@@ -1428,41 +1428,47 @@ md_status md_step(md_handle* h, int n_steps)
     return guarded(h, [&]() { return md_step_body(h, n_steps); });
 }
 
+// The first field of md_get_state whose buffer is missing (else null).
+static const char* missing_buffer(const md_state* out, unsigned fields)
+{
+    if ((fields & MD_FIELD_X) && !out->x) return "x";
+    if ((fields & MD_FIELD_XLIST) && !out->x_list) return "x_list";
+    if ((fields & MD_FIELD_V) && !out->v) return "v";
+    if ((fields & MD_FIELD_F) && !out->f) return "f";
+    if ((fields & MD_FIELD_Q) && !out->q) return "q";
+    if ((fields & MD_FIELD_H) && !out->h) return "h";
+    return nullptr;
+}
+
 // The copies of md_get_state (the replicas' plasma state goes into pinned
-// memory), enqueued on the handle's stream.
+// memory), enqueued on the handle's stream; the buffers have been checked.
 static md_status get_state_async(md_handle* h, md_state* out, unsigned fields)
 {
     const int N = h->N, R = h->R;
     const size_t nv = 3 * (size_t)N * sizeof(double);
     if (fields & MD_FIELD_X) {
-        if (!out->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
         const double* src[3] = {h->P.x, h->P.y, h->P.z};
         launch_join_vectors(src, N, h->d_scratch, h->stream);
         CU(cudaMemcpyAsync(out->x, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_XLIST) {
-        if (!out->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
         const bool buffered = h->P.xr != nullptr;
         const double* src[3] = {buffered ? h->P.xr : h->P.x, buffered ? h->P.yr : h->P.y, buffered ? h->P.zr : h->P.z};
         launch_join_vectors(src, N, h->d_scratch, h->stream);
         CU(cudaMemcpyAsync(out->x_list, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_V) {
-        if (!out->v) return fail(h, MD_ERR_INVALID_ARG, "v buffer missing");
         launch_velocity_out(h->P, h->d_scratch, h->stream);
         CU(cudaMemcpyAsync(out->v, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_F) {
-        if (!out->f) return fail(h, MD_ERR_INVALID_ARG, "f buffer missing");
         launch_force_out(h->P, h->d_scratch, h->stream);
         CU(cudaMemcpyAsync(out->f, h->d_scratch, nv, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_Q) {
-        if (!out->q) return fail(h, MD_ERR_INVALID_ARG, "q buffer missing");
         CU(cudaMemcpyAsync(out->q, h->P.q, N, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & MD_FIELD_H) {
-        if (!out->h) return fail(h, MD_ERR_INVALID_ARG, "h buffer missing");
         CU(cudaMemcpyAsync(out->h, h->P.h, N, cudaMemcpyDeviceToHost, h->stream));
     }
     if (fields & (MD_FIELD_PLASMA | MD_FIELD_COUNTS))
@@ -1492,6 +1498,8 @@ static md_status md_get_state_body(md_handle* h, md_state* out, unsigned fields)
 {
     if (!h) return fail(nullptr, MD_ERR_INVALID_ARG, "null handle");
     if (!out) return fail(h, MD_ERR_INVALID_ARG, "null state");
+    // before the first copy is enqueued: no buffer is written once an error is returned
+    if (const char* f = missing_buffer(out, fields)) return fail(h, MD_ERR_INVALID_ARG, std::string(f) + " buffer missing");
     // After steps still in flight the copies and the error flags are read in one
     // round trip.  Any flag set (a list overflow, an error) falls back to md_sync
     // and copies again.
