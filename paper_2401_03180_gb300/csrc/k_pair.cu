@@ -264,7 +264,6 @@ struct ListWarp {
     int2 fr[kSuperClusters];                          // fragment range of each i-cluster
     float4 ip[kSCAtoms];                              // the SC's atoms, [cluster k][atom a] (write pass)
 };
-constexpr int kListWarps = 8;
 
 // An SC's cell, in the grid of its replica.
 struct ListSC {
@@ -2006,11 +2005,13 @@ static void with_instance(bool fp64, bool energy, bool hyb, bool few, F&& f)
     else eh(N{}, N{});
 }
 
-int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm)
+int launch_pair_list(const Params& p, cudaStream_t s, int per_sm, int n_sm)
 {
-    if (p.sc_cap <= kListFusedScs) {
+    const bool fused = p.sc_cap <= kListFusedScs;
+    const int blocks = list_grid(fused, p.sc_cap, per_sm, n_sm);
+    if (fused) {
         const auto f = has_light(p) ? k_list_fused<true> : k_list_fused<false>;
-        f<<<std::min(p.sc_cap, n_sm * 8), kListWarps * 32, 0, s>>>(p);
+        f<<<blocks, kListWarps * 32, 0, s>>>(p);
         return 1;
     }
     k_list_count<<<blocks, kListWarps * 32, 0, s>>>(p);

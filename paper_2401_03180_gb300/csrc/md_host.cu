@@ -39,7 +39,7 @@ struct md_handle {
     int prof_next = 0;                                    // pairs in flight
     long long list_grows = 0;
     int grid_atoms = 1, grid_cells = 1, sort_threads = 1024;
-    int pair_blocks = 1, pair_warps = 8, list_blocks = 1, list_bps = 8;
+    int pair_blocks = 1, pair_warps = 8, list_bps = 8;
     int build_kernels = 0;               // kernels of one cell + list build in the step graph
     long long host_step = 0;             // steps enqueued
     long long pending = 0;               // enqueued steps whose status is not read yet
@@ -184,7 +184,7 @@ void enqueue_rebuild(md_handle* h, cudaStream_t s, bool energy)
 {
     launch_step_a(h->P, 0, s, h->grid_atoms);
     launch_cells(h->P, s, h->grid_atoms, h->grid_cells, h->sort_threads);
-    launch_pair_list(h->P, s, h->list_blocks, h->n_sm);
+    launch_pair_list(h->P, s, h->list_bps, h->n_sm);
     set_build_step(h, s, true);   // forces at the build positions: the list may be pruned
     launch_pair_forces(h->P, s, energy, h->pair_blocks, h->pair_warps);
     launch_probe(h->P, s, true);
@@ -204,7 +204,7 @@ void enqueue_rebuild_from_ref(md_handle* h, cudaStream_t s)
     }
     launch_step_a(P, 0, s, h->grid_atoms);
     launch_cells(P, s, h->grid_atoms, h->grid_cells, h->sort_threads);
-    launch_pair_list(P, s, h->list_blocks, h->n_sm);
+    launch_pair_list(P, s, h->list_bps, h->n_sm);
     // a force pass at the build positions trims the entries' masks as the step
     // of the original build did (its forces are discarded; the trimmed atoms
     // only add exact zeros, so the forces below are the same either way)
@@ -223,7 +223,7 @@ void enqueue_step(md_handle* h, cudaStream_t s, bool events)
     int mode = STEP_KICK_DRIFT | STEP_ADVANCE | (h->cfg.cr_enabled ? STEP_CR : 0);
     launch_step_a(h->P, mode, s, h->grid_atoms);
     h->build_kernels = launch_cells(h->P, s, h->grid_atoms, h->grid_cells, h->sort_threads) +
-                       launch_pair_list(h->P, s, h->list_blocks, h->n_sm);
+                       launch_pair_list(h->P, s, h->list_bps, h->n_sm);
     // external event nodes: the events are recorded on every graph replay
     if (events) cudaEventRecordWithFlags(h->ev_pair0, s, cudaEventRecordExternal);
     launch_pair_forces(h->P, s, false, h->pair_blocks, h->pair_warps);
@@ -319,7 +319,7 @@ md_status capture_buffered_step(md_handle* h, bool events)
     cudaGraph_t rebuild = cp.conditional.phGraph_out[0];
     CU(cudaStreamBeginCaptureToGraph(h->body_stream, rebuild, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     h->build_kernels = launch_cells(h->P, h->body_stream, h->grid_atoms, h->grid_cells, h->sort_threads) +
-                       launch_pair_list(h->P, h->body_stream, h->list_blocks, h->n_sm);
+                       launch_pair_list(h->P, h->body_stream, h->list_bps, h->n_sm);
     CU(cudaStreamEndCapture(h->body_stream, &rebuild));
     CU(cudaStreamUpdateCaptureDependencies(s, &cn, nullptr, 1, cudaStreamSetCaptureDependencies));
     if (events) cudaEventRecordWithFlags(h->ev_pair0, s, cudaEventRecordExternal);
@@ -456,12 +456,10 @@ md_status autotune(md_handle* h)
             if (h->cfg.sort_threads && st != h->cfg.sort_threads) continue;
             for (int lb : lb_c) {
                 if (h->cfg.list_blocks_per_sm && lb != h->cfg.list_blocks_per_sm) continue;
-                const int lblocks =
-                    (int)std::max(1LL, std::min(((long long)h->P.sc_cap + 7) / 8, (long long)lb * h->n_sm));
                 float ms = 0.0f;
                 md_status s = timed([&]() {
                     launch_cells(h->P, h->stream, h->grid_atoms, h->grid_cells, st);
-                    launch_pair_list(h->P, h->stream, lblocks, h->n_sm);
+                    launch_pair_list(h->P, h->stream, lb, h->n_sm);
                 }, &ms);
                 if (s != MD_OK) return s;
                 if (ms < best) { best = ms; bs = st; bl = lb; }
@@ -469,7 +467,6 @@ md_status autotune(md_handle* h)
         }
         h->sort_threads = bs;
         h->list_bps = bl;
-        h->list_blocks = (int)std::max(1LL, std::min(((long long)h->P.sc_cap + 7) / 8, (long long)bl * h->n_sm));
     }
     float best = 1e30f;
     int bw = h->pair_warps, bb = h->pair_blocks;
@@ -1126,9 +1123,8 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
                                                    " warps accepted for this system");
         h->pair_blocks = h->n_sm * (c.pair_blocks_per_sm ? c.pair_blocks_per_sm : maxb);
     }
-    // list kernels: one warp per super-cluster (or per group of its cells), 8 warps per block
+    // list kernels: a block per super-cluster, or a warp per super-cluster or part of one
     h->list_bps = c.list_blocks_per_sm ? c.list_blocks_per_sm : 8;
-    h->list_blocks = (int)std::max(1LL, std::min(((long long)P.sc_cap + 7) / 8, (long long)h->list_bps * h->n_sm));
     CU(cudaDeviceSynchronize());
 
     // ---- initial cell list, cluster-pair list and forces F_0 ----

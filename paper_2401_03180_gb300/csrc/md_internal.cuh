@@ -330,7 +330,7 @@ __device__ __forceinline__ float list_half_skin2(const Params& p) { return p.lc 
 void launch_step_a(const Params& p, int mode, cudaStream_t s, int grid_atoms);
 // launch_cells and launch_pair_list return the number of kernels they launched
 int launch_cells(const Params& p, cudaStream_t s, int grid_atoms, int grid_cells, int sort_threads);
-int launch_pair_list(const Params& p, cudaStream_t s, int blocks, int n_sm);
+int launch_pair_list(const Params& p, cudaStream_t s, int per_sm, int n_sm);
 void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks, int warps);
 void launch_velocity_out(const Params& p, double* d_v_out, cudaStream_t s);
 // energies: n_parts blocks of kEnergyAtoms atoms, replica r's from part_off[r]

@@ -325,7 +325,7 @@ extern "C" md_status md_forces_noalloc(const md_forces_input* in, double* d_f, v
     const int blocks = n_sm * std::max(1, pair_max_blocks_per_sm(in->precision == MD_PREC_FP64, false, false, warps, nts, n));
     launch_step_a(P, 0, s, (n + 255) / 256);                           // grid and screening
     launch_cells(P, s, (n + 255) / 256, std::max(1, std::min(g.cell_cap, n_sm * 8)), 1024);
-    launch_pair_list(P, s, std::max(1, std::min((P.sc_cap + 7) / 8, 8 * n_sm)), n_sm);
+    launch_pair_list(P, s, 8, n_sm);
     launch_pair_forces(P, s, false, blocks, warps);
     launch_force_out(P, d_f, s);
     NA_CU(cudaGetLastError());

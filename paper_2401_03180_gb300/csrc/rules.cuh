@@ -56,4 +56,15 @@ inline int pair_pin_limit(bool fp64, bool hyb, int warps, int n_ts)
     return n > 1 ? n : 1;
 }
 
+// Blocks of a list build at `per_sm` blocks per SM: at most a block per super-cluster
+// in the one-kernel build, a warp (of eight) per super-cluster in the kernels for
+// many of them.
+constexpr int kListWarps = 8;
+inline int list_grid(bool fused, int sc_cap, int per_sm, int n_sm)
+{
+    const long long most = fused ? sc_cap : ((long long)sc_cap + kListWarps - 1) / kListWarps;
+    const long long n = (long long)per_sm * n_sm;
+    return (int)(n < 1 || most < 1 ? 1 : (n < most ? n : most));
+}
+
 }  // namespace mdg

@@ -70,3 +70,10 @@ PINS = [(0, 0, 4, 2, 6), (0, 0, 8, 2, 3), (0, 0, 12, 2, 2), (0, 0, 4, 46, 4), (0
 def test_pinned_blocks_per_sm_stay_accepted(rules, fp64, hyb, warps, n_ts, blocks):
     lib = rules("int f(int d, int h, int w, int n) { return pair_pin_limit(d != 0, h != 0, w, n); }")
     assert lib.f(fp64, hyb, warps, n_ts) == blocks
+
+
+@pytest.mark.parametrize("fused,sc_cap,per_sm,blocks", [(1, 32_768, 1, 152), (1, 32_768, 8, 1216), (1, 32_768, 16, 2432), (1, 300, 2, 300),
+                                                        (1, 1, 16, 1), (0, 40_000, 1, 152), (0, 40_000, 16, 2432), (0, 40_000, 64, 5000)])
+def test_list_blocks_per_sm_set_the_grid_of_either_build(rules, fused, sc_cap, per_sm, blocks):
+    lib = rules("int f(int fused, int sc, int per, int sm) { return list_grid(fused != 0, sc, per, sm); }")
+    assert lib.f(fused, sc_cap, per_sm, 152) == blocks
