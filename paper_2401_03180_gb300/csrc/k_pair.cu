@@ -895,15 +895,21 @@ __device__ __forceinline__ void bonded_prologue(const Params& p)
 // Two tiles per branch for more independent work: 852 us, the longer code is
 // slower.  The hybrid instance needs 128 registers (112: 45.1 us, 96: 50.9).
 // ---------------------------------------------------------------------------
-template <bool HYB>
+// MODE: 0 Debye, 1 hybrid electrostatics, 2 hybrid with energies
+template <int MODE>
 struct JHyb {};
 template <>
-struct JHyb<true> {
+struct JHyb<1> {
     float4 Gr[kChunk * 4];         // G and r' of the two j-atoms: G0 G1 r'0 r'1
     float2 iGr[kSCAtoms];          // (f/2) G_i and r'_i of the SC's atoms
 };
+template <>
+struct JHyb<2> : JHyb<1> {
+    float4 ce[kChunk * 4];         // c1 and phi(r_cut) of the two j-atoms: c1_0 c1_1 phi_0 phi_1
+    float2 ice[kSCAtoms];          // (f/2) c1_i and (f/2) phi_i(r_cut) of the SC's atoms
+};
 constexpr int kJpRow = 52;         // floats per lane row of the j-force parts (padded: rows start on different banks)
-template <bool HYB>
+template <int MODE>
 struct WarpF32 {
     float4 xy[kChunk * 4];         // j-atom pairs of the chunk, [entry][ty]: x0 x1 y0 y1 (shifted)
     float4 zq[kChunk * 4];         // z0 z1 q0 q1
@@ -915,7 +921,7 @@ struct WarpF32 {
     float jp[kChunk * 4 * kJpRow]; // j-force parts [entry][ty][component][tx]
     int2 counts;                   // the list's chunks, and the heavy ones among them
     uint2 ent[kChunk];             // first slot of the j-cluster; i-cluster mask | kEntGen | kEntShare | cluster of the SC << 16
-    JHyb<HYB> hy;
+    JHyb<MODE> hy;
 };
 constexpr unsigned kEntGen = 0x100u;     // the self-cluster diagonal or pairs within one fragment are possible
 constexpr unsigned kEntShare = 0x200u;   // the entry's fragment flag
@@ -926,7 +932,6 @@ struct PairCtx {
     float rl2;                     // PRUNE: squared list radius
     float irc6, sh6, sh1;          // ENERGY: r_c^-6, and the shift's e^{-kappa r_c} r_c^-6 / 6 and e^{-kappa r_c} / r_c
     float c2, hf;                  // hybrid: c2 of the replica, f/2
-    const HybQ* rows;              // hybrid: the replica's charge states
 };
 
 __device__ __forceinline__ float2 lds_f2(int addr)
@@ -938,11 +943,12 @@ __device__ __forceinline__ float2 lds_f2(int addr)
 
 // Atom i against j-atoms 0 and 1.  r^-6 (12 c12 r^-6 - 6 c6 + kappa r (c12 r^-6
 // - c6)) is r^-6 ((2 + kappa r / 6) P + 6 c6) with P = 6 c12 r^-6 - 6 c6.
-// GEN: pairs may be dropped (ok) or lie within one fragment (no LJ).
+// GEN: pairs may be dropped (ok) or lie within one fragment (no LJ).  iGr, jGr, iCe and
+// jCe: the hybrid constants of the atoms (JHyb).
 template <bool GEN, bool ENERGY, bool HYB>
 __device__ __forceinline__ void pair2(const PairCtx& c, const float4& xi, const float2& iGr, int row, int fri, const float4& xy,
-                                      const float4& zq, const int2& off, const int2& frj, const float4& jGr, bool ok0,
-                                      bool ok1, float& fx, float& fy, float& fz, float& u, int& npair, float2& fjx,
+                                      const float4& zq, const int2& off, const int2& frj, const float4& jGr,
+                                      const float2& iCe, const float4& jCe, bool ok0, bool ok1, float& fx, float& fy, float& fz, float& u, int& npair, float2& fjx,
                                       float2& fjy, float2& fjz, float2& r2)
 {
     using P = Prec<false>;
@@ -993,36 +999,37 @@ __device__ __forceinline__ void pair2(const PairCtx& c, const float4& xi, const 
     fjx = __ffma2_rn(fs, dx, fjx);
     fjy = __ffma2_rn(fs, dy, fjy);
     fjz = __ffma2_rn(fs, dz, fjz);
-    if constexpr (ENERGY && !HYB) {
-        // out of range rinv and lj are zero, and so is the energy before the shift:
-        // selects instead of two branches a tile, the shift's constants once per chunk
-        // (million-atom frame 2,280 -> 2,032 us)
-        const float2 qq = __fmul2_rn(make_float2(xi.w, xi.w), make_float2(zq.z, zq.w));
+    if constexpr (ENERGY) {
+        // out of range rinv and lj are zero, and the rest is left out: selects instead of
+        // two branches a tile, the shift's constants once per chunk (million-atom frame
+        // 2,280 -> 2,032 us)
         const float2 lp = __fmul2_rn(make_float2(lj0, lj1), make_float2(P0, P1));
-        const float2 v = __fmul2_rn(e, __ffma2_rn(lp, make_float2(1.0f / 6.0f, 1.0f / 6.0f), __fmul2_rn(qq, rinv)));
         const float s0 = same0 ? 0.0f : __fmaf_rn(l0.y, c.irc6, -l0.x), s1 = same1 ? 0.0f : __fmaf_rn(l1.y, c.irc6, -l1.x);
-        const float h0 = __fmaf_rn(s0, c.sh6, qq.x * c.sh1), h1 = __fmaf_rn(s1, c.sh6, qq.y * c.sh1);
-        u += v.x - (in0 ? h0 : 0.0f);
-        u += v.y - (in1 ? h1 : 0.0f);
+        const float2 six = make_float2(1.0f / 6.0f, 1.0f / 6.0f);
+        if constexpr (HYB) {
+            // each ion's phi - phi(r_cut) from its own form, the constants staged with the
+            // atoms (read from the replica's table per pair in range, in a branch each,
+            // they took the pass for 30,000 atoms from 283 to 641 us)
+            const float2 q2 = make_float2(zq.z, zq.w), er = __fmul2_rn(e, rinv);
+            const float2 ii = __ffma2_rn(make_float2(xi.w, xi.w), rinv,
+                                         __ffma2_rn(make_float2(-c.hf * c.c2, -c.hf * c.c2), r2, make_float2(iCe.x, iCe.x)));
+            const float2 io = __fmul2_rn(make_float2(iGr.x, iGr.x), er);
+            const float2 ji = __ffma2_rn(q2, rinv, __ffma2_rn(make_float2(-c.c2, -c.c2), r2, make_float2(jCe.x, jCe.y)));
+            const float2 jo = __fmul2_rn(make_float2(jGr.x, jGr.y), er);
+            const float2 pi = make_float2((r.x < iGr.y ? ii.x : io.x) - iCe.y, (r.y < iGr.y ? ii.y : io.y) - iCe.y);
+            const float2 pj = make_float2((r.x < jGr.z ? ji.x : jo.x) - jCe.z, (r.y < jGr.w ? ji.y : jo.y) - jCe.w);
+            const float2 cl = __ffma2_rn(q2, pi, __fmul2_rn(make_float2(xi.w, xi.w), pj));
+            const float2 v = __ffma2_rn(__fmul2_rn(e, lp), six, cl);
+            u += in0 ? __fmaf_rn(-s0, c.sh6, v.x) : 0.0f;
+            u += in1 ? __fmaf_rn(-s1, c.sh6, v.y) : 0.0f;
+        } else {
+            const float2 qq = __fmul2_rn(make_float2(xi.w, xi.w), make_float2(zq.z, zq.w));
+            const float2 v = __fmul2_rn(e, __ffma2_rn(lp, six, __fmul2_rn(qq, rinv)));
+            const float h0 = __fmaf_rn(s0, c.sh6, qq.x * c.sh1), h1 = __fmaf_rn(s1, c.sh6, qq.y * c.sh1);
+            u += v.x - (in0 ? h0 : 0.0f);
+            u += v.y - (in1 ? h1 : 0.0f);
+        }
         npair += (in0 ? 1 : 0) + (in1 ? 1 : 0);
-    }
-    if constexpr (ENERGY && HYB) {
-        const float irc2 = c.irc * c.irc, irc6 = irc2 * irc2 * irc2;
-        auto energy = [&](float rr, float rsq, float ri, float ee, float lj, float Pp, const float2& l, bool on,
-                          float qj, float G) {
-            float v = ee * (lj * (Pp * (1.0f / 6.0f)));
-            if (on) v -= c.erc * (__fmaf_rn(l.y, irc6, -l.x) * (1.0f / 6.0f)) * irc6;
-            const float qi = rintf(xi.w / c.hf);
-            const HybQ& Ri = c.rows[(int)qi];
-            const HybQ& Rj = c.rows[(int)qj];
-            const float cr2 = c.c2 * rsq;
-            const float phi_i = rr < Ri.rpf ? qi * ri + Ri.c1f - cr2 : Ri.Gf * ee * ri;
-            const float phi_j = rr < Rj.rpf ? qj * ri + Rj.c1f - cr2 : G * ee * ri;
-            v += c.hf * (qj * (phi_i - Ri.phircf) + qi * (phi_j - Rj.phircf));
-            return v;
-        };
-        if (in0) { u += energy(r.x, r2.x, rinv.x, e.x, lj0, P0, l0, !same0, zq.z, jGr.x); npair += 1; }
-        if (in1) { u += energy(r.y, r2.y, rinv.y, e.y, lj1, P1, l1, !same1, zq.w, jGr.y); npair += 1; }
     }
 }
 
@@ -1039,7 +1046,7 @@ template <bool ENERGY, bool HYB, bool LIGHT, int REGS>
 __global__ void __maxnreg__(REGS) k_pair(Params p)
 {
     using P = Prec<false>;
-    using WF = WarpF32<HYB>;
+    using WF = WarpF32<HYB ? (ENERGY ? 2 : 1) : 0>;
     constexpr unsigned kFull = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     const int nts = p.n_ts_lj;
@@ -1097,7 +1104,6 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
     c.rl2 = rlb * rlb;
     c.hf = 0.5f * coulf;
     c.c2 = 0.0f;
-    c.rows = nullptr;
     bool bad = false;
 
     // The work items are fetched ahead: while a chunk is evaluated, the counter's
@@ -1118,13 +1124,14 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
         c.kap = p.rs[rr].kappa_f;
         c.kl = c.kap * -1.4426950408889634f;
         c.erc = ENERGY ? P::expneg(c.kap * (float)p.r_cut) : 0.0f;
-        if constexpr (ENERGY && !HYB) {
+        if constexpr (ENERGY) {
             c.irc6 = c.irc * c.irc * c.irc * c.irc * c.irc * c.irc;
             c.sh6 = c.erc * c.irc6 * (1.0f / 6.0f);
             c.sh1 = c.erc * c.irc;
         }
+        const HybQ* rows = nullptr;            // hybrid: the replica's charge states
         if constexpr (HYB) {
-            c.rows = p.hq + (size_t)rr * kHybQ;
+            rows = p.hq + (size_t)rr * kHybQ;
             const HybRep hr = p.hrep[rr];
             c.c2 = hr.c2f;
         }
@@ -1155,9 +1162,10 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
                 w.off[lane] = make_int2(t.x * (int)sizeof(float2), t.z * (int)sizeof(float2));
                 w.jfr[lane] = make_int2(t.y, t.w);
                 if constexpr (HYB) {
-                    const HybQ& Ra = c.rows[(int)a.w];
-                    const HybQ& Rb = c.rows[(int)b.w];
+                    const HybQ& Ra = rows[(int)a.w];
+                    const HybQ& Rb = rows[(int)b.w];
                     w.hy.Gr[lane] = make_float4(Ra.Gf, Rb.Gf, Ra.rpf, Rb.rpf);
+                    if constexpr (ENERGY) w.hy.ce[lane] = make_float4(Ra.c1f, Rb.c1f, Ra.phircf, Rb.phircf);
                 }
             }
         }
@@ -1170,7 +1178,11 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
                 w.ix[a] = make_float4(staged_x(v.x, v.w), v.y, v.z, (HYB ? c.hf : coulf) * v.w);
                 w.irow[a] = lj_addr + t.x * nts * (int)sizeof(float2);
                 w.ifr[a] = t.y;
-                if constexpr (HYB) w.hy.iGr[a] = make_float2(c.hf * c.rows[(int)v.w].Gf, c.rows[(int)v.w].rpf);
+                if constexpr (HYB) {
+                    const HybQ& Ri = rows[(int)v.w];
+                    w.hy.iGr[a] = make_float2(c.hf * Ri.Gf, Ri.rpf);
+                    if constexpr (ENERGY) w.hy.ice[a] = make_float2(c.hf * Ri.c1f, c.hf * Ri.phircf);
+                }
             }
         float ue[ENERGY ? kSuperClusters : 1];
         float fx[kSuperClusters], fy[kSuperClusters], fz[kSuperClusters];
@@ -1194,8 +1206,9 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
             if ((um & 0xffu) == 0u) continue;      // no i-cluster in range (or emptied by pruning)
             const float4 xy = w.xy[4 * v + ty], zq = w.zq[4 * v + ty];
             const int2 off = w.off[4 * v + ty];
-            float4 jGr = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 jGr = make_float4(0.f, 0.f, 0.f, 0.f), jCe = jGr;
             if constexpr (HYB) jGr = w.hy.Gr[4 * v + ty];
+            if constexpr (HYB && ENERGY) jCe = w.hy.ce[4 * v + ty];
             float2 fjx = make_float2(0.f, 0.f), fjy = fjx, fjz = fjx, r2;
             // GEN: the self-cluster diagonal (i < j) or pairs within one fragment are
             // possible; PRUNE: build step
@@ -1210,8 +1223,9 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
                     if (um & (1u << k)) {
                         const float4 xi = w.ix[k * kClusterSize + tx];
                         const int row = w.irow[k * kClusterSize + tx];
-                        float2 iGr = make_float2(0.f, 0.f);
+                        float2 iGr = make_float2(0.f, 0.f), iCe = iGr;
                         if constexpr (HYB) iGr = w.hy.iGr[k * kClusterSize + tx];
+                        if constexpr (HYB && ENERGY) iCe = w.hy.ice[k * kClusterSize + tx];
                         int fri = 0;
                         bool ok0 = true, ok1 = true;
                         if constexpr (GEN) {
@@ -1220,7 +1234,7 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
                             ok0 = !dg || tx < ty;
                             ok1 = !dg || tx < ty + 4;
                         }
-                        pair2<GEN, ENERGY, HYB>(c, xi, iGr, row, fri, xy, zq, off, frj, jGr, ok0, ok1, fx[k], fy[k], fz[k],
+                        pair2<GEN, ENERGY, HYB>(c, xi, iGr, row, fri, xy, zq, off, frj, jGr, iCe, jCe, ok0, ok1, fx[k], fy[k], fz[k],
                                                 ue[ENERGY ? k : 0], npair, fjx, fjy, fjz, r2);
                         if constexpr (PRUNE) {
                             const bool n0 = ok0 && r2.x < c.rl2, n1 = ok1 && r2.y < c.rl2;
@@ -1904,12 +1918,12 @@ void launch_frag_link(const Params& p, cudaStream_t s, int n_sm, double r_frag, 
     }
 }
 
-template <bool FP64, bool HYB>
+template <bool FP64, bool ENERGY, bool HYB>
 static size_t pair_smem(int n_ts, int warps)
 {
     const size_t tab = ((size_t)n_ts * n_ts * sizeof(typename Prec<FP64>::C2) + 127) / 128 * 128;
     if (FP64) return tab + 256 * sizeof(unsigned) + (size_t)warps * sizeof(Warp64<HYB>);
-    return tab + (size_t)warps * sizeof(WarpF32<HYB>);
+    return tab + (size_t)warps * sizeof(WarpF32<HYB ? (ENERGY ? 2 : 1) : 0>);
 }
 
 // Registers of the mixed-precision force kernel: 96 (20 warps per SM) where
@@ -1940,12 +1954,14 @@ template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int fit_warps(int warps, int n_ts)
 {
     if constexpr (FP64) {
-        while (warps > 1 && pair_smem<FP64, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
+        while (warps > 1 && pair_smem<FP64, ENERGY, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
+    } else if constexpr (ENERGY && HYB) {   // whose warps take 1 KB more than the forces' that chose the shape
+        while (warps % 2 == 0 && pair_smem<FP64, ENERGY, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
     } else if constexpr (!ENERGY && !HYB && !FEW) {
         constexpr int kWarps96 = 20, kSmemSm = 228 * 1024, kSmemBlock = 1024;   // an SM's shared memory, and what a block takes besides its own
         if (warps != 4) return warps;
         for (int w : {4, 10, 20})
-            if (pair_smem<FP64, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
+            if (pair_smem<FP64, ENERGY, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, ENERGY, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
     }
     return warps;
 }
@@ -1971,7 +1987,7 @@ static void launch_one(const Params& p, cudaStream_t s, int blocks, int warps)
         blocks = blocks * warps / fit;
         warps = fit;
     }
-    pair_kernel<FP64, ENERGY, HYB, FEW, LIGHT>()<<<blocks, warps * 32, pair_smem<FP64, HYB>(p.n_ts_lj, warps), s>>>(p);
+    pair_kernel<FP64, ENERGY, HYB, FEW, LIGHT>()<<<blocks, warps * 32, pair_smem<FP64, ENERGY, HYB>(p.n_ts_lj, warps), s>>>(p);
 }
 
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
@@ -1981,7 +1997,7 @@ static int max_blocks(int warps, int n_ts)
     const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, n_ts);
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW, true>(), fit * 32,
-                                                  pair_smem<FP64, HYB>(n_ts, fit));
+                                                  pair_smem<FP64, ENERGY, HYB>(n_ts, fit));
     return n > 0 ? std::max(1, n * fit / warps) : 0;
 }
 

@@ -1,0 +1,59 @@
+"""Energies with hybrid electrostatics (-m gpu): the constants of the atoms are staged with
+them, so samples whose clusters are mostly padding, charges up to the nucleus and cutoffs
+inside the ion spheres are compared with the oracle; and the pass costs little more than
+the Debye one."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_2401_03180_gb300 import md as M
+from paper_2401_03180_gb300 import workloads as W
+
+from gpu_common import methane, water
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    import torch
+    from paper_2401_03180_gb300 import build
+    build.build()
+    assert torch.cuda.is_available(), "GPU tests need a GPU"
+
+
+@pytest.mark.parametrize("prec,tol", [("mixed", 1e-5), ("fp64", 1e-10)])   # of sum |U_i|, as the hybrid parity tests
+@pytest.mark.parametrize("n_mol,full", [(2, False), (2, True), (9, False), (201, False), (201, True)])
+@pytest.mark.parametrize("r_cut", [0.25, 1.2])
+def test_energies_match_the_oracle(oracle_mod, prec, tol, n_mol, full, r_cut):
+    s = methane(n_mol, charge_frac=0.6, seed=n_mol)
+    if full:
+        s.q0[::3] = W.Z[s.species[::3]]              # bare nuclei among them
+    s.q0[0] = 1                                       # (some charge in every sample)
+    atom = W.atomic_data(8.0)
+    kw = dict(r_cut=r_cut, cr_enabled=False, screening="hybrid")
+    ora = oracle_mod.OracleMD(s, atom, **kw)
+    g = M.IonisingMD(s, atom, precision=prec, max_steps=2, **kw)
+    ep, pairs = g.energies()[1:]
+    g.close()
+    ne, kap = ora.scal[0]["n_e"], ora.scal[0]["kappa"]
+    rp = [oracle_mod.hybrid_coeffs(q, ne, kap)[0] for q in np.unique(s.q0) if q > 0]
+    assert max(rp) > 0 and pairs > 0
+    assert abs(ep[0] - ora.potential()[0]) <= tol * np.abs(ora.U).sum()
+
+
+def test_the_pass_costs_little_more_than_the_debye_one():
+    """Without a table read per pair: 1.3 times the Debye pass; with one, 3.4 times."""
+    s, rc = water(6000)
+    best = {}
+    for screening in ("debye", "hybrid"):
+        g = M.IonisingMD(s, W.atomic_data(8.0), r_cut=rc, cr_enabled=False, max_steps=2, screening=screening)
+        t = []
+        for _ in range(20):
+            t0 = time.perf_counter()
+            g.energies()                              # reads its result back
+            t.append(time.perf_counter() - t0)
+        g.close()
+        best[screening] = min(t)
+    assert best["hybrid"] <= 2.0 * best["debye"], best
