@@ -1158,8 +1158,11 @@ void launch_store_bytes(const uint8_t* a, int n, uint8_t* dst, const uint8_t* sp
 // batch): blocks of kEnergyAtoms atoms, then a block per replica over their
 // sums.  Bound by memory (about 60 bytes per atom, the slot gathers through
 // L2); one block per replica left all but one SM idle: 3,950 us for a million
-// atoms in one replica, 26 us in blocks of 1,024 atoms.
-__global__ void __launch_bounds__(256) k_energy_parts(Params p, const int* part_off, double* ekin_part, long long* epot_part)
+// atoms in one replica, 26 us in blocks of 1,024 atoms.  A replica of one block has
+// its energies from the first pass, and where all are such the second is not
+// launched.
+__global__ void __launch_bounds__(256) k_energy_parts(Params p, const int* part_off, double* ekin_part, long long* epot_part,
+                                                      double* ekin, long long* epot)
 {
     __shared__ double s_k[256];
     __shared__ long long s_u[256];
@@ -1196,8 +1199,9 @@ __global__ void __launch_bounds__(256) k_energy_parts(Params p, const int* part_
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        ekin_part[blockIdx.x] = s_k[0];
-        epot_part[blockIdx.x] = s_u[0];
+        const bool whole = part_off[r + 1] - part_off[r] == 1;
+        *(whole ? ekin + r : ekin_part + blockIdx.x) = s_k[0];
+        *(whole ? epot + r : epot_part + blockIdx.x) = s_u[0];
     }
 }
 
@@ -1207,6 +1211,7 @@ __global__ void __launch_bounds__(256) k_energy_sum(const int* part_off, const d
     __shared__ double s_k[256];
     __shared__ long long s_u[256];
     const int r = blockIdx.x;
+    if (part_off[r + 1] - part_off[r] == 1) return;
     double k = 0.0;
     long long u = 0;
     for (int b = part_off[r] + threadIdx.x; b < part_off[r + 1]; b += blockDim.x) {
@@ -1247,8 +1252,8 @@ void launch_force_out(const Params& p, double* d_f_out, cudaStream_t s)
 void launch_energy(const Params& p, int n_parts, const int* part_off, double* ekin_part, long long* epot_part, double* d_ekin,
                    long long* d_epot, cudaStream_t s)
 {
-    k_energy_parts<<<n_parts, 256, 0, s>>>(p, part_off, ekin_part, epot_part);
-    k_energy_sum<<<p.n_rep, 256, 0, s>>>(part_off, ekin_part, epot_part, d_ekin, d_epot);
+    k_energy_parts<<<n_parts, 256, 0, s>>>(p, part_off, ekin_part, epot_part, d_ekin, d_epot);
+    if (n_parts > p.n_rep) k_energy_sum<<<p.n_rep, 256, 0, s>>>(part_off, ekin_part, epot_part, d_ekin, d_epot);
 }
 void launch_philox(unsigned long long seed, const uint32_t* ctr, long long n, uint32_t* out,
                    cudaStream_t s)
