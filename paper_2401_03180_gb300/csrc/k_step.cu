@@ -1161,18 +1161,13 @@ void launch_store_bytes(const uint8_t* a, int n, uint8_t* dst, const uint8_t* sp
 // atoms in one replica, 26 us in blocks of 1,024 atoms.  A replica of one block has
 // its energies from the first pass, and where all are such the second is not
 // launched.
-__global__ void __launch_bounds__(256) k_energy_parts(Params p, const int* part_off, double* ekin_part, long long* epot_part,
+__global__ void __launch_bounds__(256) k_energy_parts(Params p, const int4* part, double* ekin_part, long long* epot_part,
                                                       double* ekin, long long* epot)
 {
     __shared__ double s_k[256];
     __shared__ long long s_u[256];
-    int r = 0, hi = p.n_rep - 1;
-    while (r < hi) {
-        const int mid = (r + hi + 1) >> 1;
-        if (part_off[mid] <= (int)blockIdx.x) r = mid; else hi = mid - 1;
-    }
-    const int a0 = p.rep_off[r] + ((int)blockIdx.x - part_off[r]) * kEnergyAtoms;
-    const int a1 = min(a0 + kEnergyAtoms, p.rep_off[r + 1]);
+    const int4 me = part[blockIdx.x];   // (first atom, one past the last, replica, the replica's only block)
+    const int a0 = me.x, a1 = me.y, r = me.z;
     const int full = *p.kick_full;
     double k = 0.0;
     long long u = 0;
@@ -1199,7 +1194,7 @@ __global__ void __launch_bounds__(256) k_energy_parts(Params p, const int* part_
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const bool whole = part_off[r + 1] - part_off[r] == 1;
+        const bool whole = me.w != 0;
         *(whole ? ekin + r : ekin_part + blockIdx.x) = s_k[0];
         *(whole ? epot + r : epot_part + blockIdx.x) = s_u[0];
     }
@@ -1249,10 +1244,10 @@ void launch_force_out(const Params& p, double* d_f_out, cudaStream_t s)
 {
     k_force_out<<<(p.n_atoms + 255) / 256, 256, 0, s>>>(p, d_f_out);
 }
-void launch_energy(const Params& p, int n_parts, const int* part_off, double* ekin_part, long long* epot_part, double* d_ekin,
-                   long long* d_epot, cudaStream_t s)
+void launch_energy(const Params& p, int n_parts, const int4* part, const int* part_off, double* ekin_part,
+                   long long* epot_part, double* d_ekin, long long* d_epot, cudaStream_t s)
 {
-    k_energy_parts<<<n_parts, 256, 0, s>>>(p, part_off, ekin_part, epot_part, d_ekin, d_epot);
+    k_energy_parts<<<n_parts, 256, 0, s>>>(p, part, ekin_part, epot_part, d_ekin, d_epot);
     if (n_parts > p.n_rep) k_energy_sum<<<p.n_rep, 256, 0, s>>>(part_off, ekin_part, epot_part, d_ekin, d_epot);
 }
 void launch_philox(unsigned long long seed, const uint32_t* ctr, long long n, uint32_t* out,

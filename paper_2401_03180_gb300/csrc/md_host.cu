@@ -54,6 +54,7 @@ struct md_handle {
     long long* d_epot = nullptr;
     int energy_parts = 0;                // blocks of the energy sums, replica r's from d_part_off[r]
     int* d_part_off = nullptr;
+    int4* d_part = nullptr;
     double* d_ekin_part = nullptr;
     long long* d_epot_part = nullptr;
     std::vector<long long> n_of_species;   // [R][NS] atoms per replica and species
@@ -984,6 +985,13 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
             off[r + 1] = off[r] + (h->rep_off[r + 1] - h->rep_off[r] + kEnergyAtoms - 1) / kEnergyAtoms;
         h->energy_parts = off[R];
         DALLOC(h->d_part_off, R + 1);
+        std::vector<int4> part;
+        part.reserve(off[R]);
+        for (int r = 0; r < R; ++r)
+            for (int a = h->rep_off[r]; a < h->rep_off[r + 1]; a += kEnergyAtoms)
+                part.push_back(make_int4(a, std::min(a + kEnergyAtoms, h->rep_off[r + 1]), r, off[r + 1] - off[r] == 1));
+        DALLOC(h->d_part, h->energy_parts);
+        CU(cudaMemcpy(h->d_part, part.data(), part.size() * sizeof(int4), cudaMemcpyHostToDevice));
         DALLOC(h->d_ekin_part, h->energy_parts);
         DALLOC(h->d_epot_part, h->energy_parts);
         CU(cudaMemcpy(h->d_part_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -1849,7 +1857,7 @@ static md_status md_get_energies_body(md_handle* h, double* e_kin, double* e_pot
     launch_refresh(h->P, h->stream);
     set_build_step(h, h->stream, false);
     launch_pair_forces(h->P, h->stream, true, h->pair_blocks, h->pair_warps);
-    launch_energy(h->P, h->energy_parts, h->d_part_off, h->d_ekin_part, h->d_epot_part, h->d_ekin, h->d_epot, h->stream);
+    launch_energy(h->P, h->energy_parts, h->d_part, h->d_part_off, h->d_ekin_part, h->d_epot_part, h->d_ekin, h->d_epot, h->stream);
     CU(cudaGetLastError());
     std::vector<double> ek(R);
     std::vector<long long> ep(R);

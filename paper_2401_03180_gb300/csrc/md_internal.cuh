@@ -333,8 +333,9 @@ int launch_cells(const Params& p, cudaStream_t s, int grid_atoms, int grid_cells
 int launch_pair_list(const Params& p, cudaStream_t s, int per_sm, int n_sm);
 void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks, int warps);
 void launch_velocity_out(const Params& p, double* d_v_out, cudaStream_t s);
-// energies: n_parts blocks of kEnergyAtoms atoms, replica r's from part_off[r]
-void launch_energy(const Params& p, int n_parts, const int* part_off, double* ekin_part, long long* epot_part, double* d_ekin,
+// energies: n_parts blocks of up to kEnergyAtoms atoms, replica r's from part_off[r]; part: each block's
+// (first atom, one past the last, replica, 1: the replica's only block)
+void launch_energy(const Params& p, int n_parts, const int4* part, const int* part_off, double* ekin_part, long long* epot_part, double* d_ekin,
                    long long* d_epot, cudaStream_t s);
 void launch_philox(unsigned long long seed, const uint32_t* ctr, long long n, uint32_t* out,
                    cudaStream_t s);
