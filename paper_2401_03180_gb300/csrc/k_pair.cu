@@ -238,14 +238,13 @@ __device__ __forceinline__ void pair64(const double4_16a& xi, int row_off, int f
 //                 the SC's chunk descriptors.
 // An SC's range is split into 1, 2, 7 or 14 parts (list_parts): as few as keep
 // every warp of the grid busy, so that a system of many SCs stages each SC once
-// and a smaller one still spreads over the GPU.  Systems of up to kListFusedScs
-// SCs take k_list_fused below instead.
-constexpr int kListFusedScs = 32768;   // super-cluster capacities up to this build their list in one kernel (k_list_fused)
+// and a smaller one still spreads over the GPU.  Systems of few SCs take
+// k_list_fused below instead (list_in_one_kernel).
 // Whether the list of these parameters holds light chunks apart (k_list_fused, lists
 // that serve several steps).  The kernels that find them (LIGHT) cost large systems
 // and single calls more than they give: 500,001 atoms 768 us without, 786 with.
 constexpr int kLightScs = 8192;
-__host__ __forceinline__ bool has_light(const Params& p) { return p.sc_cap <= kLightScs && p.xr != nullptr; }
+__host__ __forceinline__ bool has_light(const Params& p) { return p.list_fused && p.sc_cap <= kLightScs && p.xr != nullptr; }
 // The list's chunks and how many of them are heavy.
 __device__ __forceinline__ int2 chunk_counts(const Params& p)
 {
@@ -690,7 +689,7 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
     }
 }
 
-// The same list in one kernel, for systems of few SCs (kListFusedScs): a block
+// The same list in one kernel, for systems of few SCs (list_in_one_kernel): a block
 // per SC, its 8 warps sharing the SC's index range.  Each warp keeps the
 // j-clusters it found in range (compacted in shared memory, kFound of them; a
 // warp that finds more repeats the box tests), the block adds up its warps'
@@ -701,9 +700,7 @@ __global__ void __launch_bounds__(kListWarps * 32, 4) k_list_write(Params p)
 // SC once per part and pass, and on entries of j-clusters out of range is saved.
 // Count, scan and write against this kernel, per build: 8,005 atoms (unbuffered)
 // 20.1 -> 8.9 us, 12,297 atoms 23.6 -> 11.6, 30,000 atoms 31.9 -> 17.3, 199,773 atoms
-// of protein crystal 111 -> 80.  The line lies where staging the SC for one part
-// pays: 500,001 atoms take 194 us that way and 186 this way, 2 M atoms 647 and 739, a
-// batch of 300,000 93 and 96.
+// of protein crystal 111 -> 80.
 //
 // ORDER (buffered lists of up to kLightScs): the chunks of fewer than kLightTiles
 // tiles (i-clusters in range of an entry, before trimming) go to the end of the chunk
@@ -2023,9 +2020,8 @@ static void with_instance(bool fp64, bool energy, bool hyb, bool few, F&& f)
 
 int launch_pair_list(const Params& p, cudaStream_t s, int per_sm, int n_sm)
 {
-    const bool fused = p.sc_cap <= kListFusedScs;
-    const int blocks = list_grid(fused, p.sc_cap, per_sm, n_sm);
-    if (fused) {
+    const int blocks = list_grid(p.list_fused, p.sc_cap, per_sm, n_sm);
+    if (p.list_fused) {
         const auto f = has_light(p) ? k_list_fused<true> : k_list_fused<false>;
         f<<<blocks, kListWarps * 32, 0, s>>>(p);
         return 1;

@@ -783,9 +783,10 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     h->rep_off.assign(sys->replica_offset, sys->replica_offset + h->R + 1);
     h->grid0.assign(h->R, Grid{});
     const double r_list = c.r_cut + c.list_skin_nm;   // cell edge and list cutoff
-    long long cells_total = 0;
+    long long cells_total = 0, cells_filled = 0;   // reserved; filled by the sample, a vacuum one somewhat expanded
     for (int r = 0; r < h->R; ++r) {
         Grid& g = h->grid0[r];
+        const long long atoms_r = h->rep_off[r + 1] - h->rep_off[r];
         const double* L = sys->box + 3 * r;
         g.periodic = (L[0] > 0 || L[1] > 0 || L[2] > 0) ? 1 : 0;
         if (g.periodic) {
@@ -802,6 +803,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
                 prod *= n;
             }
             g.cell_cap = (int)prod;
+            cells_filled += std::min(prod, atoms_r);
         } else {
             double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
             for (int i = h->rep_off[r]; i < h->rep_off[r + 1]; ++i)
@@ -824,6 +826,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
             long long cap = std::max(64LL, 4 * prod);
             cap = std::min(cap, (long long)(1 << 22));
             g.cell_cap = (int)cap;
+            cells_filled += std::min(std::min(2 * prod, cap), atoms_r);
         }
         g.cell_off = (int)cells_total;
         cells_total += g.cell_cap;
@@ -842,6 +845,7 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     P.slot_cap = (int)slot_cap;
     P.cluster_cap = P.slot_cap / kClusterSize + 1;
     P.sc_cap = P.cluster_cap;
+    P.list_fused = list_in_one_kernel(cells_filled, h->N, P.sc_cap);
     P.precision = c.precision; P.cr_enabled = c.cr_enabled; P.plasma_mode = c.plasma_mode;
     P.dt = c.dt_ps; P.r_cut = c.r_cut; P.rc2 = c.r_cut * c.r_cut; P.kappa_fixed = c.kappa_fixed;
     P.te_floor = c.te_floor_ev; P.coulomb_f = c.coulomb_f;

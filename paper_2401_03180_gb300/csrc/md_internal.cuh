@@ -200,6 +200,7 @@ struct Params {
     PairEntry* pl;           // [pl_cap] cluster-pair list (j-cluster, half-shell index, i-atom mask)
     int4* pl_chunk;          // [chunk_cap] (SC, first entry, entries, replica)
     int pl_cap, chunk_cap;
+    int list_fused;          // 1: the list is built by one kernel (list_in_one_kernel)
 
     // packed, cell-sorted arrays (slot order)
     float4* xq;              // (x, y, z) relative to the cell centre, q

@@ -296,6 +296,8 @@ extern "C" md_status md_forces_noalloc(const md_forces_input* in, double* d_f, v
     P.err = (unsigned*)(B + kL.err); P.step = (long long*)(B + kL.step); P.kick_full = (int*)(B + kL.kick);
     P.pl = (PairEntry*)(B + kL.pl); P.pl_chunk = (int4*)(B + kL.pl_chunk);
     P.pl_cap = kPlCap; P.chunk_cap = kChunkCap;
+    static_assert(kNcMax <= 4096 && kClusterCap <= kListFusedScs, "few super-clusters, and no graph to hide five launches in");
+    P.list_fused = 1;
     P.cl_cen = (double4_32a*)(B + kL.cl_cen);
     P.grid_b = P.grid;                 // one build: the build grid is the grid
     P.xr = P.yr = P.zr = nullptr;

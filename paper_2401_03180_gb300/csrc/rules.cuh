@@ -67,4 +67,23 @@ inline int list_grid(bool fused, int sc_cap, int per_sm, int n_sm)
     return (int)(n < 1 || most < 1 ? 1 : (n < most ? n : most));
 }
 
+// Whether the list is built by one kernel, a block per super-cluster (SC), or by five
+// that give a warp an SC or a part of one.  The first saves launches and staging, the
+// second keeps eight times as many SCs in flight: of `scs` SCs, estimated from the
+// cells that the sample fills and its atoms, up to 7,000 take the first where cells hold
+// 16 atoms or more, and up to 3,500 where they hold fewer, whose SCs are one cluster of
+// work each.  us per step, five kernels and one, lists built at every step: one atom a
+// cell 66.4 and 65.2 at 3,427 SCs, 79.6 and 80.3 at 4,989, 174 and 278 at 30,256; eight
+// a cell 61.7 and 57.0 at 1,944, 75.2 and 77.1 at 3,796; 27 a cell 161.7 and 143.4 at
+// 4,798, 219.7 and 253.6 at 9,752; 64 a cell 253.8 and 235.8 at 6,750; water (170 a
+// cell) 572.7 and 547.8 at 5,081.  Beyond a capacity of 32,768 SCs the kernels count
+// SCs that a batch's empty cells reserve; 500,001 atoms take 194 us a build in one
+// kernel and 186 in five, 2 M atoms 739 and 647, a batch of 300,000 96 and 93.
+constexpr int kListFusedScs = 32768;
+inline bool list_in_one_kernel(long long cells, long long atoms, int sc_cap)
+{
+    const long long scs = (cells < atoms ? cells : atoms) + atoms / (kSuperClusters * kClusterSize);
+    return sc_cap <= kListFusedScs && scs <= (atoms >= 16 * cells ? 7000 : 3500);
+}
+
 }  // namespace mdg

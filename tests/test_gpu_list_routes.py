@@ -1,6 +1,6 @@
 """Both list builds (-m gpu): the one-kernel build, a block per super-cluster, and the
-kernels that give a warp a part of one, taken from 32,768 super-clusters of capacity on.
-A vacuum replica reserves about 56 of them, so a batch of some hundred small replicas
+kernels that give a warp a part of one, taken by samples of many super-clusters and from
+32,768 of capacity on.  A vacuum replica reserves about 56 of them, so a batch of some hundred small replicas
 takes the second route with few real super-clusters, split into 1, 2, 7 or 14 parts by
 the warps of its grid.  Trajectories are those of the replicas alone, bit for bit."""
 import dataclasses
@@ -11,7 +11,7 @@ import pytest
 from paper_2401_03180_gb300 import md as M
 from paper_2401_03180_gb300 import workloads as W
 
-from gpu_common import methane, water
+from gpu_common import force_errors, methane, water
 
 pytestmark = pytest.mark.gpu
 FIELDS = M.MD_FIELD_X | M.MD_FIELD_F | M.MD_FIELD_Q
@@ -82,3 +82,30 @@ def test_a_cell_of_many_clusters(prec):
     a = _run(one, **kw)
     b = _run(W.concat([one] + [_molecule(k) for k in range(600)]), **kw)
     assert all(np.array_equal(a[k], b[k][:one.n_atoms]) for k in ("x", "f", "q"))
+
+
+@pytest.mark.parametrize("prec,tol", [("mixed", 1e-5), ("fp64", 1e-9)])      # the tolerances of the parity tests
+@pytest.mark.parametrize("m", [15, 16])
+def test_a_gas_on_both_sides_of_the_line(oracle_mod, prec, tol, m):
+    """One atom a cell, 3,375 and 4,096 super-clusters: one kernel and five."""
+    rng = np.random.default_rng(m)
+    n, a = m ** 3, 1.26
+    x = (np.indices((m, m, m)).reshape(3, -1).T + 0.5) * a + rng.uniform(-0.3, 0.3, (n, 3))
+    s = W.Sample(x=x, v=np.zeros((n, 3)), species=rng.integers(0, len(W.Z), n).astype(np.uint8), fragment=np.arange(n, dtype=np.int32),
+                 q0=(rng.random(n) < 0.5).astype(np.uint8), replica_offset=np.array([0, n], np.int32), seed=np.array([5], np.uint64),
+                 box=np.full((1, 3), m * a), volume=np.array([(m * a) ** 3]))
+    atom = W.atomic_data(8.0)
+    ora = oracle_mod.OracleMD(s, atom, r_cut=1.2, cr_enabled=False, kappa_fixed=1.0)
+    out = []
+    for per_sm in (0, 1, 16):
+        g = M.IonisingMD(s, atom, r_cut=1.2, precision=prec, cr_enabled=False, kappa_fixed=1.0, max_steps=4,
+                         launch_shape=dict(list_blocks_per_sm=per_sm))
+        out.append(g.get_state(M.MD_FIELD_F)["f"])
+        g.step(3)
+        out.append(g.get_state(M.MD_FIELD_X)["x"])
+        assert g.timing().build_kernels in ((5, 6, 7, 8) if m == 15 else (9, 10, 11, 12))
+        g.close()
+    rms, mx = force_errors(out[0], ora.F)
+    assert rms <= tol, (rms, mx)
+    for k in (2, 4):
+        assert np.array_equal(out[0], out[k]) and np.array_equal(out[1], out[k + 1])

@@ -77,3 +77,16 @@ def test_pinned_blocks_per_sm_stay_accepted(rules, fp64, hyb, warps, n_ts, block
 def test_list_blocks_per_sm_set_the_grid_of_either_build(rules, fused, sc_cap, per_sm, blocks):
     lib = rules("int f(int fused, int sc, int per, int sm) { return list_grid(fused != 0, sc, per, sm); }")
     assert lib.f(fused, sc_cap, per_sm, 152) == blocks
+
+
+# (filled cells, atoms, capacity in super-clusters, one kernel)
+@pytest.mark.parametrize("cells,atoms,sc_cap,one", [
+    (125, 30_000, 3_860, True), (729, 199_773, 25_611, True), (1331, 240_000, 31_166, True),      # liquids
+    (3_375, 3_375, 3_376, True), (4_913, 4_913, 4_914, False), (27_000, 27_000, 27_001, False),   # an atom a cell
+    (1_728, 13_824, 3_241, True), (15_625, 125_000, 29_298, False),                               # eight a cell
+    (3_375, 91_125, 14_344, True), (6_859, 185_193, 29_151, False),                               # 27 a cell
+    (400, 4_000, 22_901, True),                                                                   # a batch of molecules
+    (2_000, 300_000, 39_013, False), (600, 3_000, 33_976, False)])                                # beyond the capacity
+def test_lists_of_few_super_clusters_are_built_by_one_kernel(rules, cells, atoms, sc_cap, one):
+    lib = rules("int f(int cells, int atoms, int cap) { return list_in_one_kernel(cells, atoms, cap); }")
+    assert bool(lib.f(cells, atoms, sc_cap)) == one
