@@ -418,6 +418,7 @@ def run_gpu(args, rank, world, local):
 
     dt_fs = 5e-5 * 1000.0
     wide_step = -(-n_atoms // 32) >= 16 * sms
+    rate_table = wide_step and 2 * s.n_replicas * int((atom.z + 1).sum()) <= n_atoms
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W_,
         "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -463,7 +464,7 @@ def run_gpu(args, rank, world, local):
         # kernel's inline limit; + the total rates and that reduction from 16 blocks of
         # 32 atoms per SM on), and the build's kernels (cells + list, 5 to 12 by grid
         # size) in the steps whose list is rebuilt
-        "gpu_launches": (2 + bool(args.probe) + (s.n_replicas > 4 or wide_step) + wide_step) * K
+        "gpu_launches": (2 + bool(args.probe) + (s.n_replicas > 4 or wide_step) + rate_table) * K
                         + tim.build_kernels * int(tim.list_builds),
         "pair_list": {"skin_nm": args.skin, "skin_mode": args.skin_mode, "builds": int(tim.list_builds),
                       "unbuffered_builds": int(tim.list_unbuffered_builds), "steps": K,

@@ -12,11 +12,10 @@
 namespace mdg {
 
 constexpr int kAccCopies = 16;   // accumulator copies per replica (spread contention)
-// atoms per block of the step kernel: one warp of each role.  Blocks this
+// kStepAtoms atoms per block of the step kernel: one warp of each role.  Blocks this
 // small wait at their barriers for two warps only, so the SM keeps issuing
 // from the other blocks (water box: 1.8 us less per step than 128 atoms per
 // block; 2 M-atom droplet: 87 us less)
-constexpr int kStepAtoms = 32;
 constexpr int kStepThreads = 2 * kStepAtoms;   // two threads per atom: kick/drift and charge update
 
 // ---------------------------------------------------------------------------
@@ -1027,10 +1026,10 @@ void launch_step_a(const Params& p, int mode, cudaStream_t s, int grid_atoms)
 {
     (void)grid_atoms;
     static const int n_sm = sm_count();
-    constexpr int kWide = 16;   // MINB of the variant for grids of many blocks per SM
+    constexpr int kWide = kWideBlocks;   // MINB of the variant for grids of many blocks per SM
     const int blocks = (p.n_atoms + kStepAtoms - 1) / kStepAtoms;
     const int fin_blocks = (p.n_rep * 64 + 255) / 256;
-    const bool wide = blocks >= kWide * n_sm;
+    const bool wide = step_is_wide(p.n_atoms, n_sm);
     const bool full = wide && (mode & STEP_KICK_DRIFT) && (mode & STEP_CR) && p.charge_mode != kChargeTable && p.rate_tab;
     const bool fin = wide || p.n_rep > kInlineReps;
     const bool cond = (mode & STEP_SETCOND) != 0;

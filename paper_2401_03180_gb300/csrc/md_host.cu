@@ -896,7 +896,8 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
     }
     P.charge_mode = c.charge_mode;
     P.rate_tab = nullptr;
-    if (c.cr_enabled && c.charge_mode != MD_CHARGE_TABLE) DALLOC(P.rate_tab, (size_t)R * nts * 2 * 4);
+    if (c.cr_enabled && c.charge_mode != MD_CHARGE_TABLE && rates_by_table(N, R, nts, h->n_sm))
+        DALLOC(P.rate_tab, (size_t)R * nts * 2 * 4);
     if (c.charge_mode == MD_CHARGE_TABLE) {
         // every atom neutral until a table is set: running sums of 1 everywhere
         const size_t n = (size_t)R * (c.max_steps + 1) * nts;

@@ -176,7 +176,7 @@ struct Params {
     double* qcum;            // [n_rep][max_steps + 1][n_ts] running sums of the charge-state fractions
     const unsigned long long* seed;
     const double* dF;        // [n_rep][max_steps]
-    double* rate_tab;        // [n_rep][n_ts][2][4] running sums of the rates of the step (rates only, else null)
+    double* rate_tab;        // [n_rep][n_ts][2][4] running sums of the rates of the step (rates_by_table, else null)
     const double* pres_ne;   // [n_rep][max_steps + 1]
     const double* pres_te;
     const double* volume;

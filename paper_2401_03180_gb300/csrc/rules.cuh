@@ -86,4 +86,17 @@ inline bool list_in_one_kernel(long long cells, long long atoms, int sc_cap)
     return sc_cap <= kListFusedScs && scs <= (atoms >= 16 * cells ? 7000 : 3500);
 }
 
+// The step kernel of large systems: `wide` from kWideBlocks blocks of kStepAtoms atoms
+// per SM on, and there the charge update against a table of the total rates where the
+// table (two entries per replica and type state) is no larger than the sample; an
+// atom's own rates cost about as much as an entry.  8,000 replicas of 10 atoms, 43
+// type states: the table alone took 20 us of a step kernel of 31, 12 without it.
+constexpr int kStepAtoms = 32;
+constexpr int kWideBlocks = 16;
+inline bool step_is_wide(long long atoms, int n_sm) { return (atoms + kStepAtoms - 1) / kStepAtoms >= (long long)kWideBlocks * n_sm; }
+inline bool rates_by_table(long long atoms, long long replicas, int n_ts, int n_sm)
+{
+    return step_is_wide(atoms, n_sm) && 2 * replicas * n_ts <= atoms;
+}
+
 }  // namespace mdg

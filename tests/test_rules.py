@@ -90,3 +90,15 @@ def test_list_blocks_per_sm_set_the_grid_of_either_build(rules, fused, sc_cap, p
 def test_lists_of_few_super_clusters_are_built_by_one_kernel(rules, cells, atoms, sc_cap, one):
     lib = rules("int f(int cells, int atoms, int cap) { return list_in_one_kernel(cells, atoms, cap); }")
     assert bool(lib.f(cells, atoms, sc_cap)) == one
+
+
+# (atoms, replicas, type states, a table of the rates) at 152 multiprocessors
+@pytest.mark.parametrize("atoms,replicas,n_ts,table", [
+    (1_999_998, 1, 43, True), (199_773, 1, 43, True), (1_400_000, 256, 43, True), (77_793, 1, 43, True),   # large samples
+    (77_792, 1, 43, False), (30_000, 1, 43, False),                                                         # few blocks per SM
+    (80_000, 8_000, 43, False), (688_000, 8_000, 43, True), (687_999, 8_000, 43, False),                    # small replicas
+    (1 << 30, 1 << 29, 128, False)])
+def test_rates_come_from_a_table_no_larger_than_the_sample(rules, atoms, replicas, n_ts, table):
+    lib = rules("int f(long long n, long long r, int ts, int sm) { return rates_by_table(n, r, ts, sm); }")
+    lib.f.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    assert bool(lib.f(atoms, replicas, n_ts, 152)) == table
