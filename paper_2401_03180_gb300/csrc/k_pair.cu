@@ -1946,7 +1946,8 @@ constexpr size_t kSmemMax = 227 * 1024;   // shared memory a block may ask for
 //   Mixed, 96 registers: 20 warps fit an SM's registers, as five blocks of 4 while
 //   the five tables are small (up to 28 type states), then as two blocks of 10 (up
 //   to 46) or one of 20 (up to 67).  Protein crystal, 43 type states, 199,773
-//   atoms: 398.8 us with 16 warps, 363.4 with 20.
+//   atoms: 398.8 us with 16 warps, 363.4 with 20.  The same for blocks of 12, of
+//   which an SM would hold one; of 8 it holds two, nearly as good as 20 warps.
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
 static int fit_warps(int warps, int n_ts)
 {
@@ -1956,7 +1957,7 @@ static int fit_warps(int warps, int n_ts)
         while (warps % 2 == 0 && pair_smem<FP64, ENERGY, HYB>(n_ts, warps) > kSmemMax) warps /= 2;
     } else if constexpr (!ENERGY && !HYB && !FEW) {
         constexpr int kWarps96 = 20, kSmemSm = 228 * 1024, kSmemBlock = 1024;   // an SM's shared memory, and what a block takes besides its own
-        if (warps != 4) return warps;
+        if (warps == 8) return warps;
         for (int w : {4, 10, 20})
             if (pair_smem<FP64, ENERGY, HYB>(n_ts, w) <= kSmemMax && kWarps96 / w * (pair_smem<FP64, ENERGY, HYB>(n_ts, w) + kSmemBlock) <= kSmemSm) return w;
     }
@@ -1980,22 +1981,22 @@ static void launch_one(const Params& p, cudaStream_t s, int blocks, int warps)
 {
     set_smem_attr<FP64, ENERGY, HYB, FEW, LIGHT>();
     const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, p.n_ts_lj);
-    if (blocks * warps % fit == 0) {
-        blocks = blocks * warps / fit;
+    if (fit < warps || blocks * warps % fit == 0) {   // (not fewer, larger blocks than the caller's warps fill)
+        blocks = (blocks * warps + fit - 1) / fit;
         warps = fit;
     }
     pair_kernel<FP64, ENERGY, HYB, FEW, LIGHT>()<<<blocks, warps * 32, pair_smem<FP64, ENERGY, HYB>(p.n_ts_lj, warps), s>>>(p);
 }
 
 template <bool FP64, bool ENERGY, bool HYB, bool FEW>
-static int max_blocks(int warps, int n_ts)
+static int resident_warps(int warps, int n_ts)
 {
     set_smem_attr<FP64, ENERGY, HYB, FEW, true>();
     const int fit = fit_warps<FP64, ENERGY, HYB, FEW>(warps, n_ts);
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair_kernel<FP64, ENERGY, HYB, FEW, true>(), fit * 32,
                                                   pair_smem<FP64, ENERGY, HYB>(n_ts, fit));
-    return n > 0 ? std::max(1, n * fit / warps) : 0;
+    return n * fit;
 }
 
 // Calls f with the force kernel's instance as compile-time constants.
@@ -2045,13 +2046,18 @@ void launch_pair_forces(const Params& p, cudaStream_t s, bool energy, int blocks
                   });
 }
 
-int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms)
+int pair_resident_warps(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms)
 {
     int n = 0;
     with_instance(fp64, energy, hyb, n_atoms <= kFewChunksAtoms, [&](auto d, auto en, auto h, auto few) {
-        n = max_blocks<decltype(d)::value, decltype(en)::value, decltype(h)::value, decltype(few)::value>(warps, n_ts);
+        n = resident_warps<decltype(d)::value, decltype(en)::value, decltype(h)::value, decltype(few)::value>(warps, n_ts);
     });
     return n;
+}
+
+int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms)
+{
+    return (pair_resident_warps(fp64, energy, hyb, warps, n_ts, n_atoms) + warps - 1) / warps;
 }
 
 }  // namespace mdg

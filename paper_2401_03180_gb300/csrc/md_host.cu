@@ -1116,8 +1116,8 @@ static md_status init_impl(md_handle* h, const md_config* cfg, const md_system* 
             // 12 warps, which decide what pins are accepted; of the shapes that fit)
             const bool pinned = c.pair_blocks_per_sm != 0;
             auto most = [&](int w) {
-                const int n = pair_max_blocks_per_sm(fp64, false, c.screening != 0, w, h->NTS_LJ, h->N);
-                return w * (pinned && n ? pair_pin_limit(fp64, c.screening != 0, w, h->NTS_LJ) : n);
+                const int n = pair_resident_warps(fp64, false, c.screening != 0, w, h->NTS_LJ, h->N);
+                return pinned && n ? w * pair_pin_limit(fp64, c.screening != 0, w, h->NTS_LJ) : n;
             };
             h->pair_warps = 8;
             int best = most(8);

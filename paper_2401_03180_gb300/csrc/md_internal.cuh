@@ -353,7 +353,9 @@ void launch_frag_link(const Params& p, cudaStream_t s, int n_sm, double r_frag, 
 void launch_frag_init(const Params& p, cudaStream_t s, int* parent, int* mass, int* charge);
 void launch_frag_count(const Params& p, cudaStream_t s, const int* parent, int* label, int* mass, int* charge,
                        const int* mass_number, int mass_max, int charge_max, unsigned long long* counts);
-// resident blocks per SM; 0: the shape does not fit
+// resident warps per SM of the blocks that a shape is launched with, and the blocks of
+// the shape that have as many; 0: the shape does not fit
+int pair_resident_warps(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms);
 int pair_max_blocks_per_sm(bool fp64, bool energy, bool hyb, int warps, int n_ts, int n_atoms);
 // message returned by md_last_error(NULL) (host side)
 void set_global_error(const std::string& msg);
