@@ -1100,10 +1100,11 @@ __global__ void __launch_bounds__(256) k_check_vectors(const double* __restrict_
 }
 
 __global__ void __launch_bounds__(256) k_split_vectors(const double* __restrict__ a, int n, double* x, double* y, double* z,
-                                                       const unsigned* bad)
+                                                       const unsigned* bad, int* flag)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || *bad) return;
+    if (flag && i == 0) *flag = 0;
     x[i] = a[3 * (size_t)i];
     y[i] = a[3 * (size_t)i + 1];
     z[i] = a[3 * (size_t)i + 2];
@@ -1134,11 +1135,12 @@ __global__ void __launch_bounds__(256) k_store_bytes(const uint8_t* __restrict__
     if (i < n && !*bad) dst[i] = a[i];
 }
 
-void launch_store_vectors(const double* a, int n, double* const dst[3], unsigned* bad, unsigned bit, cudaStream_t s)
+void launch_store_vectors(const double* a, int n, double* const dst[3], unsigned* bad, unsigned bit, cudaStream_t s,
+                          int* flag)
 {
     const int blocks = (n + 255) / 256;
     if (bit) k_check_vectors<<<blocks, 256, 0, s>>>(a, n, bad, bit);
-    k_split_vectors<<<blocks, 256, 0, s>>>(a, n, dst[0], dst[1], dst[2], bad);
+    k_split_vectors<<<blocks, 256, 0, s>>>(a, n, dst[0], dst[1], dst[2], bad, flag);
 }
 void launch_join_vectors(const double* const src[3], int n, double* a, cudaStream_t s)
 {

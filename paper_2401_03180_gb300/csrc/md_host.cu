@@ -1558,8 +1558,27 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
     if ((fields & MD_FIELD_X) && !in->x) return fail(h, MD_ERR_INVALID_ARG, "x buffer missing");
     if ((fields & MD_FIELD_Q) && !in->q) return fail(h, MD_ERR_INVALID_ARG, "q buffer missing");
     if ((fields & MD_FIELD_H) && !in->h) return fail(h, MD_ERR_INVALID_ARG, "h buffer missing");
+    if ((fields & MD_FIELD_XLIST) && !in->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
+    if (fields & MD_FIELD_PLASMA) {
+        if (!in->n_e || !in->e_gas_mev) return fail(h, MD_ERR_INVALID_ARG, "plasma buffers missing");
+        for (int r = 0; r < R; ++r)
+            if (in->n_e[r] < 0 || in->e_gas_mev[r] < 0) return fail(h, MD_ERR_INVALID_ARG, "negative plasma counter");
+    }
+    if ((fields & MD_FIELD_STEP) && (in->step < 0 || in->step > h->cfg.max_steps))
+        return fail(h, MD_ERR_INVALID_ARG, "step out of range");
     // the arrays are copied as they are, checked and stored on the device; a field
-    // that fails its check, and the ones after it, are not stored
+    // that fails its check, and the ones after it, are not stored, and the forces and
+    // lists are brought in line with the ones before it
+    auto refuse = [&](const char* why, bool stored) -> md_status {
+        if (stored && !h->poisoned) {
+            if (h->P.lc) CU(reset_list_ctl(h));
+            bool grown = false;
+            md_status st = rebuild_checked(h, &grown);
+            if (st == MD_OK && grown) st = capture_graph(h);
+            if (st != MD_OK) return st;
+        }
+        return fail(h, MD_ERR_INVALID_ARG, why);
+    };
     enum : unsigned { BAD_V = 1u, BAD_X = 2u, BAD_Q = 4u, BAD_H = 8u, BAD_XLIST = 16u };
     const size_t nv = 3 * (size_t)N * sizeof(double);
     CU(cudaMemsetAsync(h->d_bad, 0, sizeof(unsigned), s));
@@ -1570,7 +1589,7 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
         // bring velocities to the integer step with the current forces first
         launch_velocity_out(h->P, h->d_scratch, s);
     }
-    launch_store_vectors(h->d_scratch, N, vel, h->d_bad, BAD_V, s);
+    launch_store_vectors(h->d_scratch, N, vel, h->d_bad, BAD_V, s, h->P.kick_full);   // (at the integer step now)
     if (fields & MD_FIELD_X) {
         double* const dst[3] = {h->P.x, h->P.y, h->P.z};
         CU(cudaMemcpyAsync(h->d_scratch, in->x, nv, cudaMemcpyHostToDevice, s));
@@ -1590,16 +1609,14 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
     if (rep_fields) CU(cudaMemcpyAsync(h->h_rs, h->P.rs, R * sizeof(RepState), cudaMemcpyDeviceToHost, s));
     CU(cudaMemcpyAsync(h->h_err, h->d_bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    if (*h->h_err & BAD_V) return fail(h, MD_ERR_INVALID_ARG, "non-finite velocity");
-    if (*h->h_err & BAD_X) return fail(h, MD_ERR_INVALID_ARG, "non-finite position");
-    if (*h->h_err & BAD_Q) return fail(h, MD_ERR_INVALID_ARG, "q above Z");
-    if (*h->h_err & BAD_H) return fail(h, MD_ERR_INVALID_ARG, "h must be 0 or 1");
+    if (*h->h_err & BAD_V) return refuse("non-finite velocity", false);
+    if (*h->h_err & BAD_X) return refuse("non-finite position", false);
+    if (*h->h_err & BAD_Q) return refuse("q above Z", (fields & MD_FIELD_X) != 0);
+    if (*h->h_err & BAD_H) return refuse("h must be 0 or 1", (fields & (MD_FIELD_X | MD_FIELD_Q)) != 0);
     if (rep_fields) {
         RepState* rs = h->h_rs;
         for (int r = 0; r < R; ++r) {
             if (fields & MD_FIELD_PLASMA) {
-                if (!in->n_e || !in->e_gas_mev) return fail(h, MD_ERR_INVALID_ARG, "plasma buffers missing");
-                if (in->n_e[r] < 0 || in->e_gas_mev[r] < 0) return fail(h, MD_ERR_INVALID_ARG, "negative plasma counter");
                 rs[r].n_e = in->n_e[r];
                 rs[r].e_gas = in->e_gas_mev[r];
             }
@@ -1609,7 +1626,6 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
         CU(cudaMemcpyAsync(h->P.rs, rs, R * sizeof(RepState), cudaMemcpyHostToDevice, s));
     }
     if (fields & MD_FIELD_STEP) {
-        if (in->step < 0 || in->step > h->cfg.max_steps) return fail(h, MD_ERR_INVALID_ARG, "step out of range");
         h->host_step = in->step;
         CU(cudaMemcpyAsync(h->P.step, &h->host_step, sizeof(long long), cudaMemcpyHostToDevice, s));
     }
@@ -1618,14 +1634,13 @@ static md_status md_set_state_body(md_handle* h, const md_state* in, unsigned fi
     h->poisoned = false;
     bool from_ref = false;
     if (fields & MD_FIELD_XLIST) {
-        if (!in->x_list) return fail(h, MD_ERR_INVALID_ARG, "x_list buffer missing");
         if (h->P.xr) {   // buffered list: rebuild it where the checkpointed run built it
             double* const dst[3] = {h->P.xr, h->P.yr, h->P.zr};
             CU(cudaMemcpyAsync(h->d_scratch, in->x_list, nv, cudaMemcpyHostToDevice, s));
             launch_store_vectors(h->d_scratch, N, dst, h->d_bad, BAD_XLIST, s);
             CU(cudaMemcpyAsync(h->h_err, h->d_bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
             CU(cudaStreamSynchronize(s));
-            if (*h->h_err & BAD_XLIST) return fail(h, MD_ERR_INVALID_ARG, "non-finite list position");
+            if (*h->h_err & BAD_XLIST) return refuse("non-finite list position", true);
             from_ref = true;
         }
     }

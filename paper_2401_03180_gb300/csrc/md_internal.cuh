@@ -341,8 +341,9 @@ void launch_energy(const Params& p, int n_parts, const int4* part, const int* pa
 void launch_philox(unsigned long long seed, const uint32_t* ctr, long long n, uint32_t* out,
                    cudaStream_t s);
 void launch_force_out(const Params& p, double* d_f_out, cudaStream_t s);
-// state exchange: check (bit != 0) and split an [n][3] array, join one, check and store bytes
-void launch_store_vectors(const double* a, int n, double* const dst[3], unsigned* bad, unsigned bit, cudaStream_t s);
+// state exchange: check (bit != 0) and split an [n][3] array (clearing *flag if it is stored), join one, check and store bytes
+void launch_store_vectors(const double* a, int n, double* const dst[3], unsigned* bad, unsigned bit, cudaStream_t s,
+                          int* flag = nullptr);
 void launch_join_vectors(const double* const src[3], int n, double* a, cudaStream_t s);
 void launch_store_bytes(const uint8_t* a, int n, uint8_t* dst, const uint8_t* species, const int* zs, unsigned* bad, unsigned bit,
                         cudaStream_t s);
