@@ -48,7 +48,7 @@ struct Prec<false> {
     using T = float;
     using T4 = float4;         // global packed position + charge
     using S4 = float4;         // shared-memory copy
-    using C2 = float2;         // -6 c6, -ln2 c12
+    using C2 = float2;         // 6 c6, 6 c12
     static __device__ __forceinline__ T4 pos(const Params& p, int slot) { return p.xq[slot]; }
     // single MUFU operations (arguments are far from the denormal range)
     static __device__ __forceinline__ T rsq(T x)
@@ -1006,7 +1006,7 @@ __device__ __forceinline__ void pair2(const PairCtx& c, const float4& xi, const 
         if constexpr (HYB) {
             // each ion's phi - phi(r_cut) from its own form, the constants staged with the
             // atoms (read from the replica's table per pair in range, in a branch each,
-            // they took the pass for 30,000 atoms from 283 to 641 us)
+            // they took md_get_energies of 30,000 atoms 641 us; 269 this way)
             const float2 q2 = make_float2(zq.z, zq.w), er = __fmul2_rn(e, rinv);
             const float2 ii = __ffma2_rn(make_float2(xi.w, xi.w), rinv,
                                          __ffma2_rn(make_float2(-c.hf * c.c2, -c.hf * c.c2), r2, make_float2(iCe.x, iCe.x)));
@@ -1081,11 +1081,6 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
 
     const int tx = lane & 7, ty = lane >> 3;
     const int lj_addr = (int)__cvta_generic_to_shared(smem);
-    // after the j-force reduction lane (tx, ty) holds component tx & 3 (3: none)
-    // of j-atom 2 ty (tx < 4) or 2 ty + 1 (tx >= 4)
-    const int comp = tx & 3;
-    const bool up = tx >= 4;
-    long long* const jdst = (comp == 0 ? p.fx : (comp == 1 ? p.fy : p.fz)) + 2 * ty + (up ? 1 : 0);
     // In the step of a Verlet-buffered build the positions are the build's:
     // i-clusters with no pair within r_cut + skin are dropped from an entry's
     // mask for the list's lifetime (they cannot come within r_cut before the
@@ -1328,8 +1323,9 @@ __global__ void __maxnreg__(REGS) k_pair(Params p)
 // Per group of kGroup64 entries the lanes first test their pairs in FP32 with a
 // margin that covers the rounding of the coordinates, each keeping its pairs in
 // range as bits, and then evaluate those in FP64, every lane its own next one:
-// idle lanes only where a lane has fewer pairs than the fullest one (about 67 %
-// of the issued evaluations lie within r_cut, 38 % when all lanes followed the
+// idle lanes only where a lane has fewer pairs than the fullest one (71 % of
+// the issued evaluations lie within r_cut, counted in a water box and a methane
+// cluster; 38 % when all lanes followed the
 // entries' masks together).  The pairs left out only ever added exact zeros and
 // the others keep their order, so the sums are the same bit for bit.
 // Per launch, 30,000-atom water box: 2,730 -> 1,600 us; 8 warps per SM and 4 in
@@ -1930,7 +1926,8 @@ static size_t pair_smem(int n_ts, int warps)
 // Registers of the mixed-precision force kernel: 96 (20 warps per SM) where
 // chunks are plenty; 128 (16 warps, no recomputation) for the hybrid and the
 // energy instances, which spill otherwise, and for systems with too few chunks
-// to fill more warps: per launch 1,500 atoms 18.4 (96) and 15.6 us (128; 10.5 since), 8,005
+// to fill more warps (atoms stand for chunks, which are counted on the device after
+// the instance has been captured): per launch 1,500 atoms 18.4 (96) and 15.6 us (128; 10.5 since), 8,005
 // atoms in unbuffered lists 25.9 and 23.9, 30,000 atoms 64.6 and 65.0.
 constexpr int kFewChunksAtoms = 16384;
 template <bool FP64, bool ENERGY, bool HYB, bool FEW, bool LIGHT>

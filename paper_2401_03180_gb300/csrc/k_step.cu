@@ -1085,7 +1085,10 @@ __global__ void k_force_out(Params p, double* out)
 // State exchange: the caller's arrays of structures (x y z per atom) are copied
 // as they are and split or joined here, next to their check.  Bound by memory;
 // doing the same on the host cost 25 ms to restore and 13 ms to read a state of
-// 2 M atoms (copies 0.6 and 0.9 ms), these take 0.03 ms per field.
+// 2 M atoms, these take 0.03 ms per field.  The copies take 0.25 ms a field from and
+// into host memory that is pinned or already mapped; a read into arrays fresh from the
+// allocator adds the host's page faults, 3.9 ms for positions and velocities (0.57 ->
+// 4.45 ms).
 // A check that fails sets its bit in *bad; the kernels that would write the
 // state afterwards then do nothing.
 // ---------------------------------------------------------------------------
