@@ -441,7 +441,10 @@ md_status md_get_state(md_handle* h, md_state* out, unsigned fields);
  * Checkpoint/resume with md_get_state(MD_FIELD_ALL) continues bit for bit
  * (the paper has no checkpoint; the state is the one Sec. II.A-II.B evolve).
  * Errors: INVALID_ARG (a null buffer for a requested field, charges above Z,
- * non-finite values), BAD_STATE, OOM, CUDA. */
+ * non-finite values), BAD_STATE, OOM, CUDA.  What is found missing or out of range
+ * on the host refuses the call before anything is stored; a field whose values are
+ * refused is not stored, nor are the ones after it (in the order v, x, q, h, plasma,
+ * step, x_list), and the run can go on from the ones before it. */
 md_status md_set_state(md_handle* h, const md_state* in, unsigned fields);
 
 /* Kinetic and cutoff-shifted potential energy per replica ([n_replicas]
